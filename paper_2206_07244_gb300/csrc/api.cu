@@ -700,7 +700,7 @@ int read_counters(spgemm_handle *h) {
 // rows to temporary memory, n_nz to C.rpt); rows past the symbolic hash bins
 // and mispredicted rows go to the exact bitmap kernels. Ends like the plain
 // symbolic phase: C.rpt holds every row's n_nz and the total is known.
-int symbolic_learned(spgemm_handle *h, const Operands &op, int64_t mrows, int64_t *crpt,
+int symbolic_learned(spgemm_handle *h, const Operands &op, int64_t mrows, int64_t annz, int64_t *crpt,
                      int64_t *nnz_out) {
     const int64_t mw = op.mw;
     int rc = ensure_lscratch(h, mw);
@@ -715,7 +715,7 @@ int symbolic_learned(spgemm_handle *h, const Operands &op, int64_t mrows, int64_
     unsigned *fmx = reinterpret_cast<unsigned *>(L.fws + sizeof(long long) * (size_t)mw);
     unsigned *fmn = fmx + mw;
     time_begin(h, kSlotFeatures, s);
-    CK(launch_features(op, mrows, fnp, fmx, fmn, L.X, h->sm_count * 8, s));
+    CK(launch_features(op, annz, mrows, fnp, fmx, fmn, L.X, h->sm_count * 8, s));
     time_end(h, kSlotFeatures, s);
     time_begin(h, kSlotMlp, s);
     CK(launch_mlp_forward(h->theta, L.X, mw, nullptr, L.pred, h->margin, cap + 1, s));
@@ -1089,7 +1089,7 @@ int spgemm_symbolic(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_i
     // column windows (built here, used by both phases; the symbolic kernel
     // checks on the device that B is sorted)
     if (h->split_on || h->mode == SPGEMM_MODE_LEARNED) {
-        if (note(launch_sorted_check(op, B->rows, B->nnz, d_counters(h, 1), h->sm_count * 4, h->stream)) !=
+        if (note(launch_setup(op, 0, nullptr, B->rows, B->nnz, d_counters(h, 1), h->sm_count * 8, h->stream)) !=
             cudaSuccess)
             return fail(SPGEMM_ERR_CUDA);
         if (h->split_on && (rc = build_bindex(h, op, B))) return fail(rc);
@@ -1098,7 +1098,7 @@ int spgemm_symbolic(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_i
         // the one-phase kernels multiply during this call: they read values
         if ((A->nnz > 0 && !A->val) || (B->nnz > 0 && !B->val)) return fail(SPGEMM_ERR_INVALID);
         int64_t nnz = 0;
-        if ((rc = symbolic_learned(h, op, A->rows, crpt, &nnz))) {
+        if ((rc = symbolic_learned(h, op, A->rows, A->nnz, crpt, &nnz))) {
             dev_free(h, h->tcol);
             dev_free(h, h->tval);
             h->tcol = nullptr;
@@ -1117,18 +1117,15 @@ int spgemm_symbolic(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_i
         *nnzC = nnz;
         return SPGEMM_OK;
     }
-    // rows of B must be sorted for the windowed pass 2 of the numeric bitmap kernel
-    // step 1: n_prod per row into C.rpt
+    // step 1: n_prod per row into C.rpt; in the same launch B's column order
+    // (unless checked above): the windowed kernels need sorted rows, the
+    // warp-row numeric hash kernels skip value atomics when columns are distinct
     time_begin(h, kSlotNprod, h->stream);
-    if (note(launch_nprod(op, crpt, h->sm_count * 8, h->stream)) != cudaSuccess) return fail(SPGEMM_ERR_CUDA);
+    if (note(launch_setup(op, A->nnz, crpt, B->rows, B->nnz, h->split_on ? nullptr : d_counters(h, 1),
+                          h->sm_count * 8, h->stream)) != cudaSuccess)
+        return fail(SPGEMM_ERR_CUDA);
     time_end(h, kSlotNprod, h->stream);
     h->rplan = run_plan(h->cfg, h->smem_dyn_max, B->cols);
-    // B's column order: the windowed kernels need sorted rows, the warp-row
-    // numeric hash kernels skip value atomics when columns are distinct
-    if (!h->split_on &&
-        note(launch_sorted_check(op, B->rows, B->nnz, d_counters(h, 1), h->sm_count * 4, h->stream)) !=
-            cudaSuccess)
-        return fail(SPGEMM_ERR_CUDA);
     // step 2: symbolic binning by n_prod
     Ranges rs{};
     rs.nb = h->cfg.sym_nbins;
@@ -1511,7 +1508,7 @@ static int multiply_host(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_
         const Operands op = make_operands(&dA, &dB, 0, M);
         std::vector<int64_t> np((size_t)M);
         if (cudaMemsetAsync(d_np, 0, sizeof(int64_t) * (size_t)M, h->stream) != cudaSuccess ||
-            note(launch_nprod(op, d_np, h->sm_count * 8, h->stream)) != cudaSuccess ||
+            note(launch_setup(op, A->nnz, d_np, 0, 0, nullptr, h->sm_count * 8, h->stream)) != cudaSuccess ||
             cudaMemcpyAsync(np.data(), d_np, sizeof(int64_t) * (size_t)M, cudaMemcpyDeviceToHost,
                             h->stream) != cudaSuccess ||
             cudaStreamSynchronize(h->stream) != cudaSuccess) {
@@ -1964,7 +1961,7 @@ int spgemm_batch_create(spgemm_batch **out, spgemm_handle *h, int n, const spgem
             op.brpt = d_rp; op.b64 = 1;
         }
         CK(cudaMemsetAsync(d_b, 0, sizeof(int64_t) * (size_t)(M + 1), h->stream));
-        CK(launch_nprod(op, d_b, h->sm_count * 4, h->stream));
+        CK(launch_setup(op, A[i].nnz, d_b, 0, 0, nullptr, h->sm_count * 8, h->stream));
         bound[i].resize((size_t)M);
         if (M > 0)
             CK(cudaMemcpyAsync(bound[i].data(), d_b, sizeof(int64_t) * (size_t)M, cudaMemcpyDeviceToHost,

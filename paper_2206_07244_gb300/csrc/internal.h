@@ -122,17 +122,23 @@ struct KernelDesc {
 };
 
 // --- setup.cu ----------------------------------------------------------------
-cudaError_t launch_nprod(const Operands &op, int64_t *nprod, int grid, cudaStream_t s);
+// n_prod of every row of the window, added into nprod (zeroed by the caller;
+// nullptr: not wanted), and B's column order: bit 0 of cnt->flags set when
+// some row of B has a column smaller than the one before it, bit 1 when a
+// row repeats a column (cnt nullptr: not wanted). annz: A's entries (sizes
+// the grid); grid: blocks of each part, at most.
+cudaError_t launch_setup(const Operands &op, int64_t annz, int64_t *nprod, int64_t brows, int64_t bnnz,
+                         Counters *cnt, int grid, cudaStream_t s);
+// n_prod, and the longest and shortest referenced B row, of every row of the
+// window (0, 0 and UINT_MAX before).
+cudaError_t launch_feature_scan(const Operands &op, int64_t annz, int64_t *nprod, unsigned *maxlen, unsigned *minlen,
+                                int grid, cudaStream_t s);
 cudaError_t launch_bin_pass1(const int64_t *sizes, int64_t n, const Ranges &rg,
                              const Operands &op, Counters *cnt, long long *tile_sums,
                              cudaStream_t s);
 cudaError_t launch_bin_pass2(const int64_t *sizes, int64_t n, const Ranges &rg,
                              const long long *offsets, Counters *cnt, int32_t *bins,
                              cudaStream_t s);
-// Sets bit 0 of cnt->flags when some row of B has a column smaller than the
-// one before it.
-cudaError_t launch_sorted_check(const Operands &op, int64_t brows, int64_t bnnz, Counters *cnt,
-                                int grid, cudaStream_t s);
 // In-place exclusive scan of crpt[0..n) using per-tile sums from pass 1;
 // writes crpt[n] = total. tile_sums needs room for ntiles + 1 entries.
 cudaError_t launch_scan(int64_t *crpt, int64_t n, long long *tile_sums, cudaStream_t s);
@@ -279,7 +285,7 @@ cudaError_t launch_batch(int variant, int grid, const BatchProb *probs, const Ba
 
 // --- learned.cu ----------------------------------------------------------------
 int mlp_param_count();
-cudaError_t launch_features(const Operands &op, int64_t mrows, long long *nprod, unsigned *maxlen,
+cudaError_t launch_features(const Operands &op, int64_t annz, int64_t mrows, long long *nprod, unsigned *maxlen,
                             unsigned *minlen, float *X, int grid, cudaStream_t s);
 cudaError_t launch_mlp_forward(const float *theta, const float *X, int64_t n, float *y,
                                long long *sizes, float margin, long long cap, cudaStream_t s);

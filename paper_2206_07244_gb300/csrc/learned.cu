@@ -19,72 +19,10 @@
 namespace ops {
 
 // ---------------------------------------------------------------------------
-// Features (one flat pass over A's non-zeros, like nprod_kernel): per row
+// Features (one flat pass over A's non-zeros, launch_feature_scan): per row
 // n_prod, max and min referenced B-row length; then per row the six
 // features: log1p(nnz A_i), log1p(n_prod), log1p(max), log1p(mean),
 // log1p(min), log((i + 1) / M); empty A rows have max = mean = min = 0.
-constexpr int kFeatBlock = 256;
-constexpr int kFeatItems = 8;
-
-__global__ void __launch_bounds__(kFeatBlock)
-feature_scan_kernel(Operands op, long long *nprod, unsigned *maxlen, unsigned *minlen) {
-    constexpr int kTile = kFeatBlock * kFeatItems;
-    __shared__ TileRpt<kTile> tr;
-    const int64_t lo = op.row0, hi = op.row0 + op.mw;
-    const int64_t pb = ld_rpt(op.arpt, op.a64, lo);
-    const int64_t pe = ld_rpt(op.arpt, op.a64, hi);
-    for (int64_t base = pb + static_cast<int64_t>(blockIdx.x) * kTile; base < pe;
-         base += static_cast<int64_t>(gridDim.x) * kTile) {
-        stage_tile_rpt<kTile>(op, lo, hi, base, base + kTile < pe ? base + kTile : pe, &tr);
-        const int64_t p0 = base + static_cast<int64_t>(threadIdx.x) * kFeatItems;
-        if (p0 >= pe) continue;
-        const int n = tr.n;
-        int ti = 0;
-        int64_t row, next;
-        if (n > 0) {
-            ti = tile_row(tr.r, 0, n, p0);
-            row = tr.rlo + ti;
-            next = tr.r[ti + 1];
-        } else {
-            row = upper_bound_rpt(op.arpt, op.a64, lo, hi, p0);
-            next = ld_rpt(op.arpt, op.a64, row + 1);
-        }
-        long long acc = 0;
-        unsigned mx = 0, mn = UINT_MAX;
-        auto flush = [&]() {
-            const int64_t r = row - lo;
-            if (acc) atomicAdd(reinterpret_cast<unsigned long long *>(nprod + r),
-                               static_cast<unsigned long long>(acc));
-            atomicMax(maxlen + r, mx);
-            atomicMin(minlen + r, mn);
-        };
-        for (int j = 0; j < kFeatItems; ++j) {
-            const int64_t p = p0 + j;
-            if (p >= pe) break;
-            if (p >= next) {
-                flush();
-                acc = 0;
-                mx = 0;
-                mn = UINT_MAX;
-                if (n > 0) {
-                    ti = tile_row(tr.r, ti + 1, n, p);
-                    row = tr.rlo + ti;
-                    next = tr.r[ti + 1];
-                } else {
-                    row = upper_bound_rpt(op.arpt, op.a64, row + 1, hi, p);
-                    next = ld_rpt(op.arpt, op.a64, row + 1);
-                }
-            }
-            const int k = __ldg(op.acol + p);
-            const long long len = ld_rpt(op.brpt, op.b64, k + 1) - ld_rpt(op.brpt, op.b64, k);
-            acc += len;
-            mx = max(mx, static_cast<unsigned>(len));
-            mn = min(mn, static_cast<unsigned>(len));
-        }
-        flush();
-    }
-}
-
 __global__ void feature_finish_kernel(Operands op, int64_t mrows, const long long *nprod,
                                       const unsigned *maxlen, const unsigned *minlen, float *X) {
     const int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -105,15 +43,14 @@ __global__ void feature_finish_kernel(Operands op, int64_t mrows, const long lon
     x[5] = logf(static_cast<float>(static_cast<double>(i + 1) / static_cast<double>(mrows)));
 }
 
-cudaError_t launch_features(const Operands &op, int64_t mrows, long long *nprod, unsigned *maxlen,
+cudaError_t launch_features(const Operands &op, int64_t annz, int64_t mrows, long long *nprod, unsigned *maxlen,
                             unsigned *minlen, float *X, int grid, cudaStream_t s) {
     if (op.mw <= 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(nprod, 0, sizeof(long long) * (size_t)op.mw, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(maxlen, 0, sizeof(unsigned) * (size_t)op.mw, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(minlen, 0xff, sizeof(unsigned) * (size_t)op.mw, s);
     if (e != cudaSuccess) return e;
-    feature_scan_kernel<<<grid, kFeatBlock, 0, s>>>(op, nprod, maxlen, minlen);
-    e = cudaGetLastError();
+    e = launch_feature_scan(op, annz, reinterpret_cast<int64_t *>(nprod), maxlen, minlen, grid, s);
     if (e != cudaSuccess) return e;
     const int64_t g2 = (op.mw + 255) / 256;
     feature_finish_kernel<<<static_cast<unsigned>(g2), 256, 0, s>>>(op, mrows, nprod, maxlen, minlen, X);
@@ -403,7 +340,7 @@ int spgemm_features(const spgemm_csr_in *A, const spgemm_csr_in *B, int64_t row_
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return launch_features(op, A->rows, np, mx, mn, X, sms * 8, static_cast<cudaStream_t>(stream)) ==
+    return launch_features(op, A->nnz, A->rows, np, mx, mn, X, sms * 8, static_cast<cudaStream_t>(stream)) ==
                    cudaSuccess
                ? SPGEMM_OK
                : SPGEMM_ERR_CUDA;

@@ -102,7 +102,7 @@ extern "C" int spgemm_rowptr_noalloc(const spgemm_csr_in *A, const spgemm_csr_in
         return SPGEMM_ERR_CUDA;
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (launch_nprod(op, crpt, sms * 8, s) != cudaSuccess) return SPGEMM_ERR_CUDA;
+    if (launch_setup(op, A->nnz, crpt, 0, 0, nullptr, sms * 8, s) != cudaSuccess) return SPGEMM_ERR_CUDA;
     // default symbolic bins: every hash table at least 1.2x its bin's
     // largest n_prod, the bitmap kernel for the rest
     Ranges rs{};
