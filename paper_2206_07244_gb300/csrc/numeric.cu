@@ -133,9 +133,9 @@ __device__ __forceinline__ void warp_bitonic(unsigned (&x)[NR]) {
 }
 
 // One warp: sort the n condensed entries (tk[e], tv[e]), e < n <= NR * 32,
-// by column and store the first m to ocol/oval. Keys are (column << 8 | e):
-// columns below 2^24, n <= 256.
-template <int NR>
+// by column and store the first m to ocol/oval. Keys are (column << BITS | e):
+// columns below 2^(32 - BITS), n <= 2^BITS.
+template <int NR, int BITS>
 __device__ __forceinline__ void warp_sort_store(const int *tk, const double *tv, int n, int64_t m,
                                                 int32_t *ocol, double *oval, bool store) {
     const int lane = threadIdx.x & 31;
@@ -143,7 +143,7 @@ __device__ __forceinline__ void warp_sort_store(const int *tk, const double *tv,
 #pragma unroll
     for (int q = 0; q < NR; ++q) {
         const int e = q * 32 + lane;
-        x[q] = e < n ? (static_cast<unsigned>(tk[e]) << 8) | static_cast<unsigned>(e) : 0xffffffffu;
+        x[q] = e < n ? (static_cast<unsigned>(tk[e]) << BITS) | static_cast<unsigned>(e) : 0xffffffffu;
     }
     warp_bitonic<NR>(x);
     if (!store) return;
@@ -151,8 +151,8 @@ __device__ __forceinline__ void warp_sort_store(const int *tk, const double *tv,
     for (int q = 0; q < NR; ++q) {
         const int e = q * 32 + lane;
         if (e < m) {
-            ocol[e] = static_cast<int32_t>(x[q] >> 8);
-            oval[e] = tv[x[q] & 255u];
+            ocol[e] = static_cast<int32_t>(x[q] >> BITS);
+            oval[e] = tv[x[q] & ((1u << BITS) - 1u)];
         }
     }
 }
@@ -164,7 +164,8 @@ __device__ __forceinline__ void warp_sort_store(const int *tk, const double *tv,
 // registers: warp-per-row kernels that sort in registers 1280 threads (48
 // registers; 27-point stencil 128^3: 10.64 -> 9.72 ms against 1536 threads),
 // block-per-row kernels 1536 (40 registers; block-diagonal n = 2^20:
-// 12.43 -> 10.44 ms against 2048).
+// 12.43 -> 10.44 ms against 2048). The warp-per-row forms of the 512- and
+// 1024-slot tables get the threads that their shared memory allows.
 // ONE_PHASE (learned sizing): the row's size is not known; the table was
 // chosen from a prediction. A probe that finds no free slot, or more keys
 // than the table can sort in place, marks the row as mispredicted: it is
@@ -172,7 +173,7 @@ __device__ __forceinline__ void warp_sort_store(const int *tk, const double *tv,
 // size goes to C.rpt and its sorted entries to its temporary slot.
 template <int TPR, int BLOCK, int T, bool ONE_PHASE = false, bool MULTI = false>
 __global__ void __launch_bounds__(BLOCK, (T * 12 * (BLOCK / TPR) > 110 * 1024) ? 1
-                                         : ((TPR == 32 && T <= 256) ? 1280 : (TPR > 32 ? 1536 : 2048)) / BLOCK)
+                                         : (TPR == 32 ? (T <= 256 ? 1280 : T <= 512 ? 896 : 576) : (TPR > 32 ? 1536 : 2048)) / BLOCK)
 num_hash_kernel(Operands op, BinWork w) {
     constexpr int RPB = BLOCK / TPR;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -291,8 +292,9 @@ num_hash_kernel(Operands op, BinWork w) {
             P = 1;
         }
     }
-    if constexpr (TPR == 32 && T <= 256) {
-        if (op.ncols <= (int64_t{1} << 24)) {   // uniform
+    if constexpr (TPR == 32 && T <= 1024) {
+        constexpr int kBits = T <= 256 ? 8 : 9;
+        if (op.ncols <= (int64_t{1} << (32 - kBits)) && n <= (1 << kBits)) {   // uniform over the warp
             // one warp per row: sort (column << 8 | slot) in registers, then
             // store columns and the values of their slots in order
             const int64_t m = n < n_expect ? n : n_expect;
@@ -306,10 +308,11 @@ num_hash_kernel(Operands op, BinWork w) {
                 if (valid && !in_bounds && lg == 0) set_error(w.err, DERR_BOUNDS);
             }
             const bool store = valid && in_bounds;
-            if (n <= 32) warp_sort_store<1>(tk, tv, n, m, ocol, oval, store);
-            else if (n <= 64) warp_sort_store<2>(tk, tv, n, m, ocol, oval, store);
-            else if (n <= 128 || T <= 128) warp_sort_store<(T < 128 ? T / 32 : 4)>(tk, tv, n, m, ocol, oval, store);
-            else warp_sort_store<T / 32>(tk, tv, n, m, ocol, oval, store);
+            if (n <= 32) warp_sort_store<1, kBits>(tk, tv, n, m, ocol, oval, store);
+            else if (n <= 64) warp_sort_store<2, kBits>(tk, tv, n, m, ocol, oval, store);
+            else if (n <= 128) warp_sort_store<4, kBits>(tk, tv, n, m, ocol, oval, store);
+            else if (n <= 256) warp_sort_store<8, kBits>(tk, tv, n, m, ocol, oval, store);
+            else if constexpr (kBits > 8) warp_sort_store<16, kBits>(tk, tv, n, m, ocol, oval, store);
             return;   // uniform over the warp; no block barrier follows
         }
     }
@@ -823,6 +826,27 @@ static NumFn g_num_onephase[] = {NUM_TABLE(NUM_ONEPHASE_ENTRY)};
 // the plain kernels with the read-then-swap probe (BinWork::multi)
 #define NUM_MULTI_ENTRY(TPR, BLOCK, T) &num_hash_kernel<TPR, BLOCK, T, false, true>,
 static NumFn g_num_multi[] = {NUM_TABLE(NUM_MULTI_ENTRY)};
+// The 512- and 1024-slot kernels with a warp per row instead of 64 and 128
+// threads: no block barriers in the walk, the condense and the sort, values
+// without atomics where B's rows are distinct and long, and rows of up to 512
+// entries sorted in registers, which needs the column and the slot in one 32-bit
+// key, so B has at most 2^23 columns. Bound by the chain of table probes.
+// (Rows of about 190 entries of unstructured factors, 25,069 rows: 401 ->
+// 132 us; about 290 entries, 7,482 rows: 239 -> 94 us; block-diagonal n = 2^20
+// with 437 entries a row: 11.9 -> 9.5 ms.) Wider B takes the block kernels,
+// which sort by a span bitmap or in shared memory, 64 and 128 threads wide;
+// so does the read-then-swap probe.
+constexpr int64_t kWarpRowCols = int64_t{1} << 23;
+#define NUM_WARP(BLOCK, T)                                                                          \
+    {BLOCK, (sizeof(int) + sizeof(double)) * (BLOCK / 32 * (size_t)T + kStage * (size_t)BLOCK),      \
+     &num_hash_kernel<32, BLOCK, T>, &num_hash_kernel<32, BLOCK, T, true>}
+static const struct {
+    int block;
+    size_t smem;
+    NumFn fn, onephase;
+} g_num_warp[] = {NUM_WARP(128, 512), NUM_WARP(64, 1024)};
+constexpr int kNumWarpFirst = 3;   // kernels 3 and 4 of the table
+
 static constexpr int kNumHash = sizeof(g_num) / sizeof(g_num[0]);
 static KernelDesc g_num_bitmap{1024, 1024, 0, LLONG_MAX, 1, 0};
 
@@ -863,6 +887,13 @@ cudaError_t num_prepare(int smem_optin) {
                                  static_cast<int>(g_num[i].d.smem));
         if (e != cudaSuccess) return e;
     }
+    for (const auto &v : g_num_warp)
+        for (const NumFn fn : {v.fn, v.onephase}) {
+            const cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(fn),
+                                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       static_cast<int>(v.smem));
+            if (e != cudaSuccess) return e;
+        }
     g_num_bitmap.table = static_cast<long long>((smem_optin - sizeof(WalkScratch)) / 12) * 64;
     for (const auto &v : g_num_bm) {
         cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(v.fn),
@@ -894,9 +925,22 @@ static int pick_bitmap_variant(size_t smem_total, int iters) {
     return 0;
 }
 
+// The warp-per-row form of kernel `id` for these operands, -1: none.
+static int warp_row_form(int id, const Operands &op, const BinWork &w) {
+    const int k = id - kNumWarpFirst;
+    return k >= 0 && k < static_cast<int>(sizeof(g_num_warp) / sizeof(g_num_warp[0])) && op.ncols <= kWarpRowCols &&
+                   !w.multi ? k : -1;
+}
+
 cudaError_t launch_num_onephase(int id, const Operands &op, const BinWork &w, cudaStream_t s) {
     if (w.cnt <= 0) return cudaSuccess;
     if (id < 0 || id >= kNumHash) return cudaErrorInvalidValue;
+    if (const int k = warp_row_form(id, op, w); k >= 0) {
+        const auto &v = g_num_warp[k];
+        const int64_t rpb = v.block / 32;
+        v.onephase<<<static_cast<unsigned>((w.cnt + rpb - 1) / rpb), v.block, v.smem, s>>>(op, w);
+        return cudaGetLastError();
+    }
     const KernelDesc &d = g_num[id].d;
     const int rpb = d.block / d.tpr;
     const int64_t grid = (w.cnt + rpb - 1) / rpb;
@@ -954,7 +998,11 @@ cudaError_t launch_copy_rows(const BinWork &w, cudaStream_t s) {
 cudaError_t launch_num(int id, const Operands &op, const BinWork &w, size_t smem_bitmap,
                        cudaStream_t s) {
     if (w.cnt <= 0) return cudaSuccess;
-    if (id < kNumHash) {
+    if (const int k = warp_row_form(id, op, w); k >= 0) {
+        const auto &v = g_num_warp[k];
+        const int64_t rpb = v.block / 32;
+        v.fn<<<static_cast<unsigned>((w.cnt + rpb - 1) / rpb), v.block, v.smem, s>>>(op, w);
+    } else if (id < kNumHash) {
         const KernelDesc &d = g_num[id].d;
         const int rpb = d.block / d.tpr;
         const int64_t grid = (w.cnt + rpb - 1) / rpb;
