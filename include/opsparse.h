@@ -274,8 +274,9 @@ int spgemm_window_stats(const spgemm_handle *h, int64_t *out, int n);
  * the symbolic bins, 16-31 the numeric bins, 32 n_prod, 33/34 symbolic
  * binning passes 1/2, 35/36 numeric binning passes 1/2, 37 the scan; in
  * learned mode also 38 the row features, 39 the MLP forward with the sizes
- * and binning by prediction, 40 the copy of one-phase rows into C (41
- * slots). reset != 0 clears the totals. */
+ * and binning by prediction, 40 the copy of one-phase rows into C; 41 the
+ * row patterns of A and B, 42 the numeric kernels of the rows that repeat
+ * the pattern of the row before (43 slots). reset != 0 clears the totals. */
 int spgemm_set_timing(spgemm_handle *h, int enable);
 int spgemm_kernel_times(spgemm_handle *h, double *ms, int64_t *launches, int n,
                         int reset);

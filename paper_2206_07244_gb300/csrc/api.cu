@@ -49,7 +49,9 @@ enum Slot {
     kSlotFeatures = 38,   // learned mode: row features
     kSlotMlp = 39,        // learned mode: MLP forward, sizes, binning by prediction
     kSlotCopy = 40,       // learned mode: one-phase rows copied into C
-    kSlots = 41,
+    kSlotPatterns = 41,   // row patterns of A and B, repeating rows of C
+    kSlotRepeat = 42,     // numeric kernels of the repeating rows
+    kSlots = 43,
 };
 
 }  // namespace
@@ -105,8 +107,9 @@ struct spgemm_handle {
                                   // adapted from call to call (load feedback)
     unsigned char *lscratch = nullptr;
     size_t lscratch_bytes = 0;
-    int32_t *tcol = nullptr;      // temporary one-phase rows of the current call
-    double *tval = nullptr;
+    int32_t *tcol = nullptr;      // temporary one-phase rows of the current call (kept for the next
+    double *tval = nullptr;       // one up to kTempKeep entries)
+    long long tcap_have = 0;
     long long lsize[kMaxBins] = {}, loff[kMaxBins] = {}, ltbase[kMaxBins] = {}, ltcap[kMaxBins] = {};
     long long ltotal = 0;
     bool lid = false;
@@ -114,6 +117,13 @@ struct spgemm_handle {
     int64_t lstats[6 + kMaxBins] = {};  // one-phase rows, mispredicted rows, exact rows, temp
                                         // entries, rows > 3/4 full, rows that fit the next
                                         // smaller table, factor exponents used per class
+    // repeating rows of C (repeat.cu)
+    uint8_t *rcode = nullptr;     // pattern codes of B's rows, then of A's window rows (B's own when A is B)
+    size_t rcode_bytes = 0;
+    RepWord *rwords = nullptr;    // the last symbolic call's words, one per 32 window rows, and as many unfinished ones
+    size_t rwords_bytes = 0;
+    bool rep_num = false;         // the numeric phase leaves them out of its bins
+    long long rep_cnt[kRepClasses] = {};   // rows per class
     // column-window numeric path for the last numeric bin (window.cu)
     WinPlan wplan;                // plan of the last symbolic call
     bool wp_on = false;           // the symbolic call prepared cell counts and a window count
@@ -239,23 +249,21 @@ long long *d_tiles(spgemm_handle *h) {
                                          align256(sizeof(int32_t) * (size_t)std::max<int64_t>(h->mw, 1)));
 }
 
-// Learned-sizing scratch per window row: features (6 floats), prediction,
-// binning size, exact-path list, and the feature kernel's n_prod/max/min.
+// Learned-sizing scratch per window row: prediction, binning size, exact-path
+// list, class, and the scan's longest and shortest referenced B row.
 struct LScratch {
-    float *X;
     long long *pred;
     int64_t *lsizes;
     int32_t *xlist;
     uint8_t *cls;         // class of each row (bin of its prediction)
     unsigned long long *fb;   // load feedback counters (kFbCounters)
-    unsigned char *fws;   // n_prod (8 B) + max (4 B) + min (4 B) per row
+    unsigned char *fws;   // longest and shortest referenced B row (4 B each) per row
 };
 
 LScratch lscratch_layout(spgemm_handle *h, int64_t mw) {
     const size_t m = (size_t)std::max<int64_t>(mw, 1);
     unsigned char *p = h->lscratch;
     LScratch L;
-    L.X = reinterpret_cast<float *>(p);                 p += align256(sizeof(float) * 6 * m);
     L.pred = reinterpret_cast<long long *>(p);          p += align256(sizeof(long long) * m);
     L.lsizes = reinterpret_cast<int64_t *>(p);          p += align256(sizeof(int64_t) * m);
     L.xlist = reinterpret_cast<int32_t *>(p);           p += align256(sizeof(int32_t) * m);
@@ -267,8 +275,8 @@ LScratch lscratch_layout(spgemm_handle *h, int64_t mw) {
 
 int ensure_lscratch(spgemm_handle *h, int64_t mw) {
     const size_t m = (size_t)std::max<int64_t>(mw, 1);
-    const size_t need = align256(24 * m) + 2 * align256(8 * m) + align256(4 * m) + align256(m) +
-                        align256(sizeof(unsigned long long) * kFbCounters) + align256(16 * m) + 256;
+    const size_t need = 2 * align256(8 * m) + align256(4 * m) + align256(m) +
+                        align256(sizeof(unsigned long long) * kFbCounters) + align256(8 * m) + 256;
     if (h->lscratch && h->lscratch_bytes >= need) return SPGEMM_OK;
     if (h->lscratch) {
         if (cudaStreamSynchronize(h->stream) != cudaSuccess) return SPGEMM_ERR_CUDA;
@@ -277,6 +285,18 @@ int ensure_lscratch(spgemm_handle *h, int64_t mw) {
     h->lscratch = static_cast<unsigned char *>(dev_alloc(h, need));
     h->lscratch_bytes = h->lscratch ? need : 0;
     return h->lscratch ? SPGEMM_OK : SPGEMM_ERR_OOM;
+}
+
+// The one-phase rows' temporary memory is allocated while the GPU waits, so up
+// to 2^25 entries (400 MB) stay with the handle from call to call.
+constexpr long long kTempKeep = 1ll << 25;
+
+void release_temp(spgemm_handle *h) {
+    dev_free(h, h->tcol);
+    dev_free(h, h->tval);
+    h->tcol = nullptr;
+    h->tval = nullptr;
+    h->tcap_have = 0;
 }
 
 unsigned long long *d_xcount(spgemm_handle *h) {
@@ -667,16 +687,69 @@ int run_bins(spgemm_handle *h, int phase, const Operands &op, const long long *s
 
 // Bin sizes -> (offsets, identity?) : identity when one bin holds every row
 // (the generalisation of Algorithm 3: no scatter pass, rows in index order).
-bool plan_bins(const Counters &c, int nb, long long *size, long long *offset) {
+// own_only: the bins hold only the rows that do not repeat a row before.
+bool plan_bins(const Counters &c, int nb, long long *size, long long *offset, bool own_only = false) {
     long long acc = 0;
     int nonempty = 0;
+    bool all = true;
     for (int j = 0; j < nb; ++j) {
-        size[j] = static_cast<long long>(c.bin_cnt[j]);
+        size[j] = static_cast<long long>(own_only ? c.bin_own[j] : c.bin_cnt[j]);
+        all &= !own_only || c.bin_own[j] == c.bin_cnt[j];
         offset[j] = acc;
         acc += size[j];
         nonempty += size[j] > 0;
     }
-    return nonempty <= 1;
+    return all && nonempty <= 1;
+}
+
+// Compares the rows of A and B with the row before them when the product is
+// large enough for repeating rows to pay (kRepMinRows and following; *on).
+// A goes first: without an eighth of its rows repeating (*gate) B is not
+// looked at. The column-window form (bitmap_path 2) plans its windows from
+// the sizes of all rows before they are filled in, and the read-then-swap
+// probe is there to be measured: both multiply every row on its own.
+int scan_patterns(spgemm_handle *h, const Operands &op, const spgemm_csr_in *A, const spgemm_csr_in *B,
+                  const uint8_t **acode, RepGate *gate, bool *on) {
+    const int64_t mw = op.mw;
+    *on = false;
+    if (mw < kRepMinRows || h->wp_on || h->cfg.hash_access) return SPGEMM_OK;   // A and B have rows, then
+    const double per_row = static_cast<double>(A->nnz) / static_cast<double>(A->rows) *
+                           (static_cast<double>(B->nnz) / static_cast<double>(std::max<int64_t>(B->rows, 1)));
+    if (per_row < kRepMinProducts || (mw < kRepManyRows && per_row * static_cast<double>(mw) < kRepManyProducts))
+        return SPGEMM_OK;
+    const bool same = A->rpt == B->rpt && A->rpt_is_i64 == B->rpt_is_i64 && A->col == B->col && A->rows == B->rows;
+    int rc = ensure_buf(h, &h->rcode, &h->rcode_bytes, (size_t)B->rows + (same ? 0 : (size_t)mw));
+    if (rc || (rc = ensure_buf(h, &h->rwords, &h->rwords_bytes, 2 * sizeof(RepWord) * (size_t)((mw + 31) / 32)))) return rc;
+    uint8_t *code = same ? h->rcode + op.row0 : h->rcode + B->rows;
+    unsigned long long *found = &d_counters(h, 0)->rep_found;
+    gate->found = found;
+    gate->least = static_cast<unsigned long long>(std::max<int64_t>(1, (same ? B->rows : mw) / 8));
+    if (!same)
+        CK(launch_row_patterns(op.arpt, op.a64, op.acol, op.row0, mw, A->nnz, code, found, RepGate(), h->stream));
+    CK(launch_row_patterns(op.brpt, op.b64, op.bcol, 0, B->rows, B->nnz, h->rcode, same ? found : nullptr,
+                           same ? RepGate() : *gate, h->stream));
+    *acode = code;
+    *on = true;
+    return SPGEMM_OK;
+}
+
+// Numeric kernels of the repeating rows, after the bins' kernels.
+int run_repeats(spgemm_handle *h, const Operands &op, const int64_t *crpt, int32_t *ccol, double *cval) {
+    // a class of few rows goes with the next larger one: its own launch would
+    // look at every run again (27-point stencil 101^3: 102 us for the rows
+    // along the edges of the box)
+    int present = 0;
+    long long more = 0;
+    for (int c = kRepClasses - 1; c >= 0; --c) {
+        if (h->rep_cnt[c] > 0 && 8 * h->rep_cnt[c] >= more) present |= 1 << c;
+        more += h->rep_cnt[c];
+    }
+    time_begin(h, kSlotRepeat, h->stream);
+    for (int c = 0; c < kRepClasses; ++c)
+        if ((present >> c) & 1)
+            CK(launch_repeat_numeric(c, present, op, h->rwords, crpt, ccol, cval, d_err(h), h->stream));
+    time_end(h, kSlotRepeat, h->stream);
+    return SPGEMM_OK;
 }
 
 int read_counters(spgemm_handle *h) {
@@ -700,9 +773,9 @@ int read_counters(spgemm_handle *h) {
 // rows to temporary memory, n_nz to C.rpt); rows past the symbolic hash bins
 // and mispredicted rows go to the exact bitmap kernels. Ends like the plain
 // symbolic phase: C.rpt holds every row's n_nz and the total is known.
-int symbolic_learned(spgemm_handle *h, const Operands &op, int64_t mrows, int64_t annz, int64_t *crpt,
-                     int64_t *nnz_out) {
-    const int64_t mw = op.mw;
+int symbolic_learned(spgemm_handle *h, const Operands &op, const spgemm_csr_in *A, const spgemm_csr_in *B,
+                     int64_t *crpt, int64_t *nnz_out) {
+    const int64_t mw = op.mw, mrows = A->rows, annz = A->nnz;
     int rc = ensure_lscratch(h, mw);
     if (rc) return rc;
     const LScratch L = lscratch_layout(h, mw);
@@ -710,35 +783,99 @@ int symbolic_learned(spgemm_handle *h, const Operands &op, int64_t mrows, int64_
     const int nb = h->cfg.num_nbins;
     const int last = nb - 1;   // the numeric bitmap bin: exact path
     const int64_t cap = nb >= 2 ? h->cfg.num_range[nb - 2] : 0;
-    // the features kernel also leaves n_prod of every row in C.rpt (step 1)
-    long long *fnp = reinterpret_cast<long long *>(crpt);
-    unsigned *fmx = reinterpret_cast<unsigned *>(L.fws + sizeof(long long) * (size_t)mw);
-    unsigned *fmn = fmx + mw;
-    time_begin(h, kSlotFeatures, s);
-    CK(launch_features(op, annz, mrows, fnp, fmx, fmn, L.X, h->sm_count * 8, s));
-    time_end(h, kSlotFeatures, s);
-    time_begin(h, kSlotMlp, s);
-    CK(launch_mlp_forward(h->theta, L.X, mw, nullptr, L.pred, h->margin, cap + 1, s));
     const int64_t exact_above = h->cfg.sym_nbins >= 2 ? h->cfg.sym_range[h->cfg.sym_nbins - 2] : -1;
     SizeFactors sf{};
     sf.nb = nb;
-    for (int j = 0; j < nb; ++j) {
-        sf.lim[j] = h->cfg.num_range[j];
-        sf.k[j] = h->lfk[j];
-    }
-    CK(cudaMemsetAsync(L.fb, 0, sizeof(unsigned long long) * kFbCounters, s));
-    CK(launch_learned_sizes(crpt, L.pred, mw, exact_above, LLONG_MAX / 4, L.lsizes, sf, L.cls, L.fb, s));
     Ranges rn{};
     rn.nb = nb;
-    for (int j = 0; j < nb; ++j) rn.r[j] = h->cfg.num_range[j];
-    CK(launch_bin_pass1(L.lsizes, mw, rn, op, d_counters(h, 0), nullptr, s));
-    time_end(h, kSlotMlp, s);
-    if ((rc = read_counters(h))) return rc;
-    // B's column order (checked before this call): distinct columns let the
-    // warp-row one-phase kernels update values without atomics
-    h->b_distinct = (h->h_cnt[1].flags & 3ull) == 0;
-    h->lid = plan_bins(h->h_cnt[0], nb, h->lsize, h->loff);
-    if (!h->lid) CK(launch_bin_pass2(L.lsizes, mw, rn, h->loff, d_counters(h, 0), d_bins(h), s));
+    for (int j = 0; j < nb; ++j) {
+        sf.lim[j] = rn.r[j] = h->cfg.num_range[j];
+        sf.k[j] = h->lfk[j];
+    }
+    unsigned *fmx = reinterpret_cast<unsigned *>(L.fws);
+    unsigned *fmn = fmx + mw;
+    // Repeating rows (repeat.cu) need no prediction. They have at most
+    // kRepMaxNnz products here (their size is not known before the bins are
+    // made, and all of them are added by the rank maps), and rows of B with
+    // distinct columns; where B turns out to have others, the bins are made
+    // again without repeating rows.
+    RepArgs rep;
+    RepGate gate;
+    const uint8_t *acode = nullptr;
+    bool repeats = false;
+    // B's column order is checked on a side stream, next to the pattern
+    // scans: nothing before the counters are read needs it (27-point stencil
+    // 128^3: 0.1 ms on its own). The handle's stream waits for it on every
+    // way out.
+    struct Aside {
+        cudaStream_t s = nullptr;
+        cudaEvent_t done = nullptr;
+        cudaError_t join() {
+            cudaEvent_t e = done;
+            done = nullptr;
+            return e ? cudaStreamWaitEvent(s, e, 0) : cudaSuccess;
+        }
+        ~Aside() { join(); }
+    } order;
+    cudaStream_t os = h->serial ? s : h->side[1];
+    if (!h->serial) {
+        CK(cudaEventRecord(h->ev_fork, s));
+        CK(cudaStreamWaitEvent(os, h->ev_fork, 0));
+    }
+    CK(launch_setup(op, 0, nullptr, B->rows, B->nnz, d_counters(h, 1), h->sm_count * 8, os));
+    if (!h->serial) {
+        CK(cudaEventRecord(h->ev_side[1], os));
+        order.s = s;
+        order.done = h->ev_side[1];
+    }
+    time_begin(h, kSlotPatterns, s);
+    if ((rc = scan_patterns(h, op, A, B, &acode, &gate, &repeats))) return rc;
+    RepWord *found_words = repeats ? h->rwords + (mw + 31) / 32 : nullptr;
+    if (repeats) {
+        CK(launch_repeats(op, annz, acode, h->rcode, found_words, gate, s));
+        time_end(h, kSlotPatterns, s);
+    }
+    for (bool again = false;; again = true) {
+        if (again) {
+            CK(cudaMemsetAsync(d_counters(h, 0), 0, sizeof(Counters), s));
+            CK(cudaMemsetAsync(crpt, 0, sizeof(int64_t) * (size_t)mw, s));
+        }
+        // n_prod of every row goes to C.rpt (step 1): from the plain scan when
+        // most rows repeat, from the features' scan otherwise
+        time_begin(h, kSlotFeatures, s);
+        CK(cudaMemsetAsync(fmx, 0, sizeof(unsigned) * (size_t)mw, s));
+        CK(cudaMemsetAsync(fmn, 0xff, sizeof(unsigned) * (size_t)mw, s));
+        if (repeats)
+            CK(launch_setup(op, annz, crpt, 0, 0, nullptr, h->sm_count * 8, s, found_words, gate, true));
+        CK(launch_feature_scan(op, annz, crpt, fmx, fmn, h->sm_count * 8, s, repeats ? gate : RepGate()));
+        if (repeats) {
+            CK(launch_repeats_finish(mw, crpt, kRepMaxNnz, found_words, h->rwords, s));
+            rep.words = h->rwords;
+            rep.max_nnz = LLONG_MAX;
+        }
+        time_end(h, kSlotFeatures, s);
+        time_begin(h, kSlotMlp, s);
+        CK(cudaMemsetAsync(L.fb, 0, sizeof(unsigned long long) * kFbCounters, s));
+        if (repeats) {
+            CK(launch_predict_few(op, mrows, h->theta, crpt, fmx, fmn, rep.words, gate, exact_above, LLONG_MAX / 4,
+                                  L.pred, L.lsizes, sf, L.cls, L.fb, h->margin, cap + 1, s));
+        } else {
+            CK(launch_predict(op, mrows, h->theta, crpt, fmx, fmn, L.pred, h->margin, cap + 1, s));
+            CK(launch_learned_sizes(crpt, L.pred, mw, exact_above, LLONG_MAX / 4, L.lsizes, sf, L.cls, L.fb, s));
+        }
+        CK(launch_bin_pass1(L.lsizes, mw, rn, op, d_counters(h, 0), nullptr, s, rep));
+        time_end(h, kSlotMlp, s);
+        CK(order.join());
+        if ((rc = read_counters(h))) return rc;
+        // distinct columns let the warp-row one-phase kernels update values without atomics
+        h->b_distinct = (h->h_cnt[1].flags & 3ull) == 0;
+        if (!repeats || h->b_distinct) break;
+        repeats = false;
+        found_words = nullptr;
+        rep = RepArgs{};
+    }
+    h->lid = plan_bins(h->h_cnt[0], nb, h->lsize, h->loff, repeats);
+    if (!h->lid) CK(launch_bin_pass2(L.lsizes, mw, rn, h->loff, d_counters(h, 0), d_bins(h), s, rep));
     // the exact list starts with the rows of the bitmap bin
     const long long cnt_last = h->lsize[last];
     if (cnt_last > 0) {
@@ -757,13 +894,13 @@ int symbolic_learned(spgemm_handle *h, const Operands &op, int64_t mrows, int64_
         h->ltbase[j] = total_t;
         total_t += h->lsize[j] * h->ltcap[j];
     }
-    h->tcol = nullptr;
-    h->tval = nullptr;
     h->ltotal = total_t;
-    if (total_t > 0) {
+    if (total_t > h->tcap_have) {
+        release_temp(h);
         h->tcol = static_cast<int32_t *>(dev_alloc(h, sizeof(int32_t) * (size_t)total_t));
         h->tval = static_cast<double *>(dev_alloc(h, sizeof(double) * (size_t)total_t));
         if (!h->tcol || !h->tval) return SPGEMM_ERR_OOM;
+        h->tcap_have = total_t;
     }
     // one-phase kernels, largest rows first on the side streams
     CK(cudaEventRecord(h->ev_fork, s));
@@ -798,12 +935,28 @@ int symbolic_learned(spgemm_handle *h, const Operands &op, int64_t mrows, int64_
         CK(cudaEventRecord(h->ev_side[i], h->side[i]));
         CK(cudaStreamWaitEvent(s, h->ev_side[i], 0));
     }
-    CK(cudaMemcpyAsync(h_x, d_xcount(h), sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
-    h->xcount = static_cast<int64_t>(*h_x);
-    if (h->xcount > mw) return SPGEMM_ERR_INTERNAL;
+    unsigned long long *h_fb = reinterpret_cast<unsigned long long *>(
+        reinterpret_cast<unsigned char *>(h->h_cnt) + 2 * sizeof(Counters) + 64);
+    // total n_nz and the scan's tile sums; the load feedback and the length
+    // of the exact list come back with them
+    auto count_rows = [&]() -> int {
+        Ranges all{};
+        all.nb = 1;
+        all.r[0] = -1;
+        if (repeats) {
+            rep.fill = crpt;
+            rep.max_nnz = kRepMaxNnz;
+        }
+        time_begin(h, kSlotNumPass1, s);
+        CK(launch_bin_pass1(crpt, mw, all, op, d_counters(h, 1), d_tiles(h), s, rep));
+        time_end(h, kSlotNumPass1, s);
+        CK(cudaMemcpyAsync(h_fb, L.fb, sizeof(unsigned long long) * kFbCounters, cudaMemcpyDeviceToHost, s));
+        CK(cudaMemcpyAsync(h_x, d_xcount(h), sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+        return read_counters(h);
+    };
     // exact symbolic for the bitmap-bin rows and the mispredicted rows
-    if (h->xcount > 0) {
+    auto exact_rows = [&]() -> int {
+        if (h->split_on && (rc = build_bindex(h, op, B))) return rc;
         BinWork w{};
         w.bins = L.xlist; w.off = 0; w.cnt = h->xcount;
         w.crpt = crpt;
@@ -824,22 +977,40 @@ int symbolic_learned(spgemm_handle *h, const Operands &op, int64_t mrows, int64_
         time_begin(h, kSlotSymBin + 15, s);
         CK(launch_sym(sym_kernel_count() - 1, op, w, static_cast<size_t>(std::max<int64_t>(words, 1)) * 4, s));
         time_end(h, kSlotSymBin + 15, s);
+        return SPGEMM_OK;
+    };
+    // Without rows of the bitmap bin the exact list is expected to stay
+    // empty, and the rows are counted before its length is known; a
+    // misprediction then costs a second count. (The sizes that the count
+    // fills in for repeating rows of a mispredicted row are its n_prod, which
+    // they held before.)
+    if (cnt_last == 0) {
+        if ((rc = count_rows())) return rc;
+        h->xcount = static_cast<int64_t>(*h_x);
+    } else {
+        CK(cudaMemcpyAsync(h_x, d_xcount(h), sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        h->xcount = static_cast<int64_t>(*h_x);
     }
-    // total n_nz and the scan's tile sums
-    Ranges all{};
-    all.nb = 1;
-    all.r[0] = -1;
-    time_begin(h, kSlotNumPass1, s);
-    CK(launch_bin_pass1(crpt, mw, all, op, d_counters(h, 1), d_tiles(h), s));
-    time_end(h, kSlotNumPass1, s);
-    unsigned long long *h_fb = reinterpret_cast<unsigned long long *>(
-        reinterpret_cast<unsigned char *>(h->h_cnt) + 2 * sizeof(Counters) + 64);
-    CK(cudaMemcpyAsync(h_fb, L.fb, sizeof(unsigned long long) * kFbCounters, cudaMemcpyDeviceToHost, s));
-    if ((rc = read_counters(h))) return rc;
+    if (h->xcount > mw) return SPGEMM_ERR_INTERNAL;
+    if (h->xcount > 0 && (rc = exact_rows())) return rc;
+    if (cnt_last > 0 || h->xcount > 0) {
+        const unsigned long long flags = h->h_cnt[1].flags;   // B's order
+        CK(cudaMemsetAsync(d_counters(h, 1), 0, sizeof(Counters), s));
+        if ((rc = count_rows())) return rc;
+        h->h_cnt[1].flags = flags;
+    }
     h->b_unsorted = (h->h_cnt[1].flags & 1ull) != 0;
     *nnz_out = static_cast<int64_t>(h->h_cnt[1].total);
     h->lstats[0] = 0;
     for (int j = 0; j < last; ++j) h->lstats[0] += h->lsize[j];
+    // a repeating row is multiplied once, too
+    h->rep_num = false;
+    for (int c = 0; c < kRepClasses; ++c) {
+        h->rep_cnt[c] = repeats ? static_cast<long long>(h->h_cnt[1].rep_cnt[c]) : 0;
+        h->lstats[0] += h->rep_cnt[c];
+        h->rep_num |= h->rep_cnt[c] > 0;
+    }
     h->lstats[1] = h->xcount - cnt_last;
     h->lstats[0] -= h->lstats[1];
     h->lstats[2] = cnt_last;
@@ -885,22 +1056,39 @@ int numeric_learned(spgemm_handle *h, const Operands &op, int64_t *crpt, int32_t
         if (!*pcol || !*pval) return SPGEMM_ERR_OOM;
     }
     const int last = h->cfg.num_nbins - 1;
+    // Repeating rows read only the columns of the rows copied here: those
+    // rows' values are then copied next to the repeating rows' kernels, on a
+    // side stream that the handle's stream waits for before it goes on.
+    const bool aside = h->rep_num && !h->serial;
+    auto copy_bins = [&](bool cols, bool vals, cudaStream_t cs) -> cudaError_t {
+        for (int j = 0; j < last; ++j) {
+            if (h->lsize[j] <= 0) continue;
+            BinWork w{};
+            w.bins = h->lid ? nullptr : d_bins(h);
+            w.off = h->lid ? 0 : h->loff[j];
+            w.cnt = h->lsize[j];
+            w.crpt = crpt; w.ccol = *pcol; w.cval = *pval;
+            w.tcol = h->tcol; w.tval = h->tval;
+            w.tbase = h->ltbase[j]; w.tcap = h->ltcap[j];
+            w.tlimit = h->ltotal;
+            w.pred = L.pred;
+            w.err = d_err(h);
+            const cudaError_t e = launch_copy_rows(w, cols, vals, cs);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    };
     time_begin(h, kSlotCopy, s);
-    for (int j = 0; j < last; ++j) {
-        if (h->lsize[j] <= 0) continue;
-        BinWork w{};
-        w.bins = h->lid ? nullptr : d_bins(h);
-        w.off = h->lid ? 0 : h->loff[j];
-        w.cnt = h->lsize[j];
-        w.crpt = crpt; w.ccol = *pcol; w.cval = *pval;
-        w.tcol = h->tcol; w.tval = h->tval;
-        w.tbase = h->ltbase[j]; w.tcap = h->ltcap[j];
-        w.tlimit = h->ltotal;
-        w.pred = L.pred;
-        w.err = d_err(h);
-        CK(launch_copy_rows(w, s));
-    }
+    CK(copy_bins(true, !aside, s));
     time_end(h, kSlotCopy, s);
+    cudaError_t copied = cudaSuccess;
+    if (aside) {
+        CK(cudaEventRecord(h->ev_fork, s));
+        CK(cudaStreamWaitEvent(h->side[0], h->ev_fork, 0));
+        copied = copy_bins(false, true, h->side[0]);
+        const cudaError_t e = cudaEventRecord(h->ev_side[0], h->side[0]);
+        if (copied == cudaSuccess) copied = e;
+    }
     if (h->xcount > 0) {
         BinWork w{};
         w.bins = L.xlist; w.off = 0; w.cnt = h->xcount;
@@ -922,10 +1110,14 @@ int numeric_learned(spgemm_handle *h, const Operands &op, int64_t *crpt, int32_t
         CK(launch_num(num_kernel_count() - 1, op, w, static_cast<size_t>(std::max<int64_t>(words, 1)) * 12, s));
         time_end(h, kSlotNumBin + 15, s);
     }
-    dev_free(h, h->tcol);
-    dev_free(h, h->tval);
-    h->tcol = nullptr;
-    h->tval = nullptr;
+    const int rc = h->rep_num ? run_repeats(h, op, crpt, *pcol, *pval) : SPGEMM_OK;
+    if (aside) {
+        const cudaError_t e = cudaStreamWaitEvent(s, h->ev_side[0], 0);
+        if (copied == cudaSuccess) copied = e;
+        CK(copied);
+    }
+    if (rc) return rc;
+    if (h->tcap_have > kTempKeep) release_temp(h);
     return SPGEMM_OK;
 }
 
@@ -1055,11 +1247,8 @@ int spgemm_symbolic(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_i
     h->reuse = false;   // the binning below overwrites the kept rows
     if (h->state == 1) {  // an earlier symbolic result was never consumed
         dev_free(h, h->crpt);
-        dev_free(h, h->tcol);
-        dev_free(h, h->tval);
+        release_temp(h);
         h->crpt = nullptr;
-        h->tcol = nullptr;
-        h->tval = nullptr;
         h->state = 0;
     }
     const int64_t mw = row_end - row_begin;
@@ -1088,21 +1277,19 @@ int spgemm_symbolic(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_i
     // cell index of B's long rows for kernels that cover rows in several
     // column windows (built here, used by both phases; the symbolic kernel
     // checks on the device that B is sorted)
-    if (h->split_on || h->mode == SPGEMM_MODE_LEARNED) {
+    // (learned sizing has use for it only when the exact list is not empty)
+    if (h->split_on && h->mode == SPGEMM_MODE_PLAIN) {
         if (note(launch_setup(op, 0, nullptr, B->rows, B->nnz, d_counters(h, 1), h->sm_count * 8, h->stream)) !=
             cudaSuccess)
             return fail(SPGEMM_ERR_CUDA);
-        if (h->split_on && (rc = build_bindex(h, op, B))) return fail(rc);
+        if ((rc = build_bindex(h, op, B))) return fail(rc);
     }
     if (h->mode == SPGEMM_MODE_LEARNED) {
         // the one-phase kernels multiply during this call: they read values
         if ((A->nnz > 0 && !A->val) || (B->nnz > 0 && !B->val)) return fail(SPGEMM_ERR_INVALID);
         int64_t nnz = 0;
-        if ((rc = symbolic_learned(h, op, A->rows, A->nnz, crpt, &nnz))) {
-            dev_free(h, h->tcol);
-            dev_free(h, h->tval);
-            h->tcol = nullptr;
-            h->tval = nullptr;
+        if ((rc = symbolic_learned(h, op, A, B, crpt, &nnz))) {
+            release_temp(h);
             return fail(rc);
         }
         h->stats[0] = 0;
@@ -1117,13 +1304,34 @@ int spgemm_symbolic(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_i
         *nnzC = nnz;
         return SPGEMM_OK;
     }
+    // rows of C that repeat the row before: their products and sizes are those
+    // of the row they go back to
+    RepArgs rep;
+    RepGate gate;
+    const uint8_t *acode = nullptr;
+    bool repeats = false;
+    RepWord *found_words = nullptr;
+    time_begin(h, kSlotPatterns, h->stream);
+    if ((rc = scan_patterns(h, op, A, B, &acode, &gate, &repeats))) return fail(rc);
+    if (repeats) {
+        found_words = h->rwords + (mw + 31) / 32;
+        if (note(launch_repeats(op, A->nnz, acode, h->rcode, found_words, gate, h->stream)) != cudaSuccess)
+            return fail(SPGEMM_ERR_CUDA);
+        time_end(h, kSlotPatterns, h->stream);
+    }
     // step 1: n_prod per row into C.rpt; in the same launch B's column order
     // (unless checked above): the windowed kernels need sorted rows, the
     // warp-row numeric hash kernels skip value atomics when columns are distinct
     time_begin(h, kSlotNprod, h->stream);
     if (note(launch_setup(op, A->nnz, crpt, B->rows, B->nnz, h->split_on ? nullptr : d_counters(h, 1),
-                          h->sm_count * 8, h->stream)) != cudaSuccess)
+                          h->sm_count * 8, h->stream, found_words, gate)) != cudaSuccess)
         return fail(SPGEMM_ERR_CUDA);
+    if (repeats) {
+        if (note(launch_repeats_finish(mw, crpt, kRepMaxProd, found_words, h->rwords, h->stream)) != cudaSuccess)
+            return fail(SPGEMM_ERR_CUDA);
+        rep.words = h->rwords;
+        rep.max_nnz = LLONG_MAX;   // every repeating row takes the size of the row it goes back to
+    }
     time_end(h, kSlotNprod, h->stream);
     h->rplan = run_plan(h->cfg, h->smem_dyn_max, B->cols);
     // step 2: symbolic binning by n_prod
@@ -1131,18 +1339,22 @@ int spgemm_symbolic(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_i
     rs.nb = h->cfg.sym_nbins;
     for (int j = 0; j < rs.nb; ++j) rs.r[j] = h->cfg.sym_range[j];
     time_begin(h, kSlotSymPass1, h->stream);
-    if (note(launch_bin_pass1(crpt, mw, rs, op, d_counters(h, 0), nullptr, h->stream)) != cudaSuccess)
+    if (note(launch_bin_pass1(crpt, mw, rs, op, d_counters(h, 0), nullptr, h->stream, rep)) != cudaSuccess)
         return fail(SPGEMM_ERR_CUDA);
     time_end(h, kSlotSymPass1, h->stream);
     if ((rc = read_counters(h))) return fail(rc);
     long long ssize[kMaxBins] = {}, soff[kMaxBins] = {};
-    const bool sid = plan_bins(h->h_cnt[0], rs.nb, ssize, soff);
+    const bool sid = plan_bins(h->h_cnt[0], rs.nb, ssize, soff, rep.words != nullptr);
+    // no repeating rows: the numeric phase need not look for them
+    repeats = false;
+    for (int j = 0; j < rs.nb; ++j) repeats |= h->h_cnt[0].bin_cnt[j] != h->h_cnt[0].bin_own[j];
+    if (!repeats) rep = RepArgs{};
     h->stats[0] = static_cast<int64_t>(h->h_cnt[0].total);
     h->stats[1] = static_cast<int64_t>(h->h_cnt[0].max_size);
-    for (int j = 0; j < SPGEMM_MAX_BINS; ++j) h->stats[4 + j] = j < rs.nb ? ssize[j] : 0;
+    for (int j = 0; j < SPGEMM_MAX_BINS; ++j) h->stats[4 + j] = j < rs.nb ? static_cast<int64_t>(h->h_cnt[0].bin_cnt[j]) : 0;
     if (!sid) {
         time_begin(h, kSlotSymPass2, h->stream);
-        if (note(launch_bin_pass2(crpt, mw, rs, soff, d_counters(h, 0), d_bins(h), h->stream)) != cudaSuccess)
+        if (note(launch_bin_pass2(crpt, mw, rs, soff, d_counters(h, 0), d_bins(h), h->stream, rep)) != cudaSuccess)
             return fail(SPGEMM_ERR_CUDA);
         time_end(h, kSlotSymPass2, h->stream);
     }
@@ -1172,7 +1384,9 @@ int spgemm_symbolic(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_i
     rn.nb = h->cfg.num_nbins;
     for (int j = 0; j < rn.nb; ++j) rn.r[j] = h->cfg.num_range[j];
     time_begin(h, kSlotNumPass1, h->stream);
-    if (note(launch_bin_pass1(crpt, mw, rn, op, d_counters(h, 1), d_tiles(h), h->stream)) != cudaSuccess)
+    rep.fill = crpt;
+    rep.max_nnz = kRepMaxNnz;
+    if (note(launch_bin_pass1(crpt, mw, rn, op, d_counters(h, 1), d_tiles(h), h->stream, rep)) != cudaSuccess)
         return fail(SPGEMM_ERR_CUDA);
     time_end(h, kSlotNumPass1, h->stream);
     if ((rc = read_counters(h))) return fail(rc);
@@ -1184,7 +1398,14 @@ int spgemm_symbolic(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_i
     h->stats[3] = static_cast<int64_t>(h->h_cnt[1].max_size);
     for (int j = 0; j < SPGEMM_MAX_BINS; ++j)
         h->stats[4 + SPGEMM_MAX_BINS + j] = j < rn.nb ? static_cast<int64_t>(h->h_cnt[1].bin_cnt[j]) : 0;
-    for (int j = 0; j < kMaxBins; ++j) h->num_size[j] = j < rn.nb ? h->h_cnt[1].bin_cnt[j] : 0;
+    // repeating rows are added without atomics: distinct columns in B's rows
+    h->rep_num = false;
+    for (int c = 0; c < kRepClasses; ++c) {
+        h->rep_cnt[c] = h->b_distinct ? static_cast<long long>(h->h_cnt[1].rep_cnt[c]) : 0;
+        h->rep_num |= h->rep_cnt[c] > 0;
+    }
+    for (int j = 0; j < kMaxBins; ++j)
+        h->num_size[j] = j < rn.nb ? (h->rep_num ? h->h_cnt[1].bin_own[j] : h->h_cnt[1].bin_cnt[j]) : 0;
     h->crpt = crpt;
     h->row0 = row_begin;
     h->ncols = B->cols;
@@ -1221,10 +1442,7 @@ int spgemm_numeric(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_in
                 dev_free(h, ccol);
                 dev_free(h, cval);
             }
-            dev_free(h, h->tcol);
-            dev_free(h, h->tval);
-            h->tcol = nullptr;
-            h->tval = nullptr;
+            release_temp(h);
             return rc;
         }
         C->rows = h->mw; C->cols = h->ncols; C->nnz = h->nnz;
@@ -1244,7 +1462,12 @@ int spgemm_numeric(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_in
     RunPlan rp = h->rplan;
     if (h->b_unsorted || !num_kernel(h->cfg.num_kernel[nb - 1]).bitmap || h->num_size[nb - 1] <= 0)
         rp = RunPlan{};
-    const bool nid = nonempty <= 1;
+    const bool nid = nonempty <= 1 && !h->rep_num;
+    RepArgs rep;
+    if (h->rep_num) {
+        rep.words = h->rwords;
+        rep.max_nnz = kRepMaxNnz;
+    }
     Ranges rn{};
     rn.nb = nb;
     for (int j = 0; j < nb; ++j) rn.r[j] = h->cfg.num_range[j];
@@ -1260,7 +1483,7 @@ int spgemm_numeric(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_in
     };
     if (!nid) {
         time_begin(h, kSlotNumPass2, h->stream);
-        if (note(launch_bin_pass2(crpt, h->mw, rn, off, d_counters(h, 1), d_bins(h), h->stream)) != cudaSuccess)
+        if (note(launch_bin_pass2(crpt, h->mw, rn, off, d_counters(h, 1), d_bins(h), h->stream, rep)) != cudaSuccess)
             return fail(SPGEMM_ERR_CUDA);
         time_end(h, kSlotNumPass2, h->stream);
     }
@@ -1341,6 +1564,7 @@ int spgemm_numeric(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_in
         rp.bs = bs;
     }
     rc = run_bins(h, 1, op, h->num_size, off, nid, crpt, ccol, cval, &rp, &wc);
+    if (!rc && h->rep_num) rc = run_repeats(h, op, crpt, ccol, cval);
     dev_free(h, bs);
     if (rc) {
         win_release(h);
@@ -1414,8 +1638,10 @@ int spgemm_numeric_values(spgemm_handle *h, const spgemm_csr_in *A, const spgemm
         wc.bslot = h->wbslot;
         wc.bidx = h->wbidx;
     }
-    return run_bins(h, 1, op, h->num_size, off, nonempty <= 1, static_cast<int64_t *>(C->rpt), C->col,
-                    C->val, nullptr, &wc);
+    int64_t *crpt = static_cast<int64_t *>(C->rpt);
+    rc = run_bins(h, 1, op, h->num_size, off, nonempty <= 1 && !h->rep_num, crpt, C->col, C->val, nullptr, &wc);
+    if (!rc && h->rep_num) rc = run_repeats(h, op, crpt, C->col, C->val);
+    return rc;
 }
 
 int spgemm_multiply(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_in *B,
@@ -1816,6 +2042,8 @@ int spgemm_destroy(spgemm_handle *h) {
     dev_free(h, h->lscratch);
     dev_free(h, h->arena);
     win_release(h);
+    dev_free(h, h->rcode);
+    dev_free(h, h->rwords);
     dev_free(h, h->wcells);
     dev_free(h, h->wcslot);
     dev_free(h, h->wspill);
@@ -2134,6 +2362,7 @@ cudaError_t prepare_device(int dev, int smem_dyn_max) {
     cudaError_t e = sym_prepare(smem_dyn_max);
     if (e == cudaSuccess) e = num_prepare(smem_dyn_max);
     if (e == cudaSuccess) e = win_prepare(smem_dyn_max);
+    if (e == cudaSuccess) e = rep_prepare();
     if (e == cudaSuccess) done[dev] = true;
     return e;
 }

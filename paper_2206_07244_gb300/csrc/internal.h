@@ -92,12 +92,93 @@ struct Ranges {
     int nb;
 };
 
+// --- repeated rows (repeat.cu) ------------------------------------------------
+// 32 consecutive window rows: bit b of `fol` set when row b's columns in C are
+// those of the row before, all moved by one when bit b of `one` is set too.
+// A run of repeating rows goes back to the last row before it whose bit is
+// clear: a row of the same word or, when the run begins at bit 0, the row
+// `back` rows before the word, with `moved` moves by one after that row and
+// before the word. A run ends at the next multiple of kRepSpan rows.
+struct __align__(16) RepWord {
+    uint32_t fol, one;
+    int32_t back, moved;
+};
+constexpr int kRepSpan = 256;
+
+#ifdef __CUDACC__
+// The row that repeating row i goes back to.
+__device__ __forceinline__ int64_t rep_own(const RepWord &w, int64_t i) {
+    const unsigned below = ~w.fol & ((1u << (i & 31)) - 1u);
+    return below ? (i & ~int64_t{31}) + 31 - __clz(below) : (i & ~int64_t{31}) - w.back;
+}
+#endif
+
+// Repeating rows by products and entries of C per row: one launch per class
+// (threads per block, products in the rank map, accumulator entries).
+struct RepClass {
+    int threads;
+    int max_prod, max_nnz;
+    int accs;   // accumulators of max_nnz entries that the shared memory holds
+};
+constexpr int kRepClasses = 4;
+constexpr RepClass kRepClass[kRepClasses] = {
+    {128, 256, 64, 16}, {128, 1024, 256, 8}, {256, 4608, 512, 8}, {256, 18432, 1024, 7}};
+constexpr int kRepMaxLen = 256;                                  // A entries of a repeating row
+constexpr int kRepMaxProd = kRepClass[kRepClasses - 1].max_prod;
+constexpr int kRepMaxNnz = kRepClass[kRepClasses - 1].max_nnz;   // larger rows are multiplied on their own
+constexpr int kRepMinRun = 4;                                    // repeating rows in a row, at least
+// When the symbolic phase looks for repeating rows (rows of the window, and
+// products per row estimated from the mean lengths of A's and B's rows): the
+// scans and extra launches cost 30 us to 40 us on products of that size, and
+// a run's map about 10 us before its rows start. 27-point stencil, whole
+// product without and with: 26^3 (11M products) 319 and 336 us, 32^3 (24M)
+// 378 and 359, 48^3 1118 and 632; tridiagonal, 2^19 rows of 9 products, 428
+// and 232 us. Rows of fewer products cost the hash kernels no more than the
+// map (7-point times piecewise-constant prolongation, 7 products).
+constexpr int64_t kRepMinRows = 4096;
+constexpr int64_t kRepManyRows = 32768;
+constexpr double kRepManyProducts = 16e6;
+constexpr double kRepMinProducts = 8.0;
+
+// First class that takes rows of `prod` products and `nnz` entries, -1: none.
+template <int C = 0>
+__host__ __device__ __forceinline__ int rep_class(long long prod, long long nnz) {
+    if constexpr (C < kRepClasses) {
+        constexpr RepClass k = kRepClass[C];
+        return prod <= k.max_prod && nnz <= k.max_nnz ? C : rep_class<C + 1>(prod, nnz);
+    } else {
+        return -1;
+    }
+}
+
+// The work that follows a pattern scan is skipped when the scan found fewer
+// than `least` rows (found nullptr: never skipped).
+struct RepGate {
+    const unsigned long long *found = nullptr;
+    unsigned long long least = 0;
+#ifdef __CUDACC__
+    __device__ __forceinline__ bool shut() const { return found && __ldcg(found) < least; }
+#endif
+};
+
+// What a binning pass does with repeating rows: it leaves them out of the
+// bins when their size is at most max_nnz, and with `fill` writes the size of
+// the row they repeat over their own first (words nullptr: no such rows).
+struct RepArgs {
+    const RepWord *words = nullptr;
+    int64_t *fill = nullptr;
+    long long max_nnz = 0;
+};
+
 // Counters written by the binning passes (device memory, zeroed per call).
 struct Counters {
     unsigned long long bin_cnt[kMaxBins];   // pass 1: rows per bin
     unsigned long long cursor[kMaxBins];    // pass 2: fill cursor per bin
     unsigned long long bin_sum[kMaxBins];   // pass 1: sum of the sizes per bin
     unsigned long long bin_nnza[kMaxBins];  // pass 1: A entries of the bin's rows
+    unsigned long long bin_own[kMaxBins];   // pass 1: the bin's rows that do not repeat a row before
+    unsigned long long rep_cnt[kRepClasses];   // numeric pass 1: repeating rows per class
+    unsigned long long rep_found;           // rows of A that look like the row before
     unsigned long long max_size;
     unsigned long long total;
     unsigned long long flags;         // bit 0: some row of B has decreasing columns; bit 1: repeated ones
@@ -126,19 +207,23 @@ struct KernelDesc {
 // nullptr: not wanted), and B's column order: bit 0 of cnt->flags set when
 // some row of B has a column smaller than the one before it, bit 1 when a
 // row repeats a column (cnt nullptr: not wanted). annz: A's entries (sizes
-// the grid); grid: blocks of each part, at most.
+// the grid); grid: blocks of each part, at most. words: rows with their bit
+// of fol set are left out (nullptr, or gate shut: none). only_open: no n_prod
+// when the gate is shut.
 cudaError_t launch_setup(const Operands &op, int64_t annz, int64_t *nprod, int64_t brows, int64_t bnnz,
-                         Counters *cnt, int grid, cudaStream_t s);
+                         Counters *cnt, int grid, cudaStream_t s, const RepWord *words = nullptr,
+                         const RepGate &gate = RepGate(), bool only_open = false);
 // n_prod, and the longest and shortest referenced B row, of every row of the
-// window (0, 0 and UINT_MAX before).
+// window (0, 0 and UINT_MAX before); with a gate only when it is shut (n_prod
+// may be there already).
 cudaError_t launch_feature_scan(const Operands &op, int64_t annz, int64_t *nprod, unsigned *maxlen, unsigned *minlen,
-                                int grid, cudaStream_t s);
+                                int grid, cudaStream_t s, const RepGate &gate = RepGate());
 cudaError_t launch_bin_pass1(const int64_t *sizes, int64_t n, const Ranges &rg,
                              const Operands &op, Counters *cnt, long long *tile_sums,
-                             cudaStream_t s);
+                             cudaStream_t s, const RepArgs &rep = RepArgs());
 cudaError_t launch_bin_pass2(const int64_t *sizes, int64_t n, const Ranges &rg,
                              const long long *offsets, Counters *cnt, int32_t *bins,
-                             cudaStream_t s);
+                             cudaStream_t s, const RepArgs &rep = RepArgs());
 // In-place exclusive scan of crpt[0..n) using per-tile sums from pass 1;
 // writes crpt[n] = total. tile_sums needs room for ntiles + 1 entries.
 cudaError_t launch_scan(int64_t *crpt, int64_t n, long long *tile_sums, cudaStream_t s);
@@ -165,6 +250,30 @@ cudaError_t launch_num(int id, const Operands &op, const BinWork &w, size_t smem
                        cudaStream_t s);
 // one-phase numeric kernel `id` (a hash kernel of the numeric table)
 cudaError_t launch_num_onephase(int id, const Operands &op, const BinWork &w, cudaStream_t s);
+
+// --- repeat.cu -----------------------------------------------------------------
+cudaError_t rep_prepare();
+// code[i] of rows first + i, i < n: bit 0 when the row's columns are those
+// of the row before moved by one, bit 1 when they are the same (row `first`,
+// empty rows and rows of more than kRepMaxNnz entries: 0); their number is
+// added to *found (nullptr: not wanted).
+cudaError_t launch_row_patterns(const void *rpt, int is64, const int32_t *col, int64_t first, int64_t n,
+                                int64_t entries, uint8_t *code, unsigned long long *found, const RepGate &gate,
+                                cudaStream_t s);
+// fol and one of the window's rows from the codes of A's rows (window rows)
+// and of B's rows.
+cudaError_t launch_repeats(const Operands &op, int64_t annz, const uint8_t *acode, const uint8_t *bcode,
+                           RepWord *words, const RepGate &gate, cudaStream_t s);
+// The words complete (words -> out), without the runs of more than max_prod
+// products a row; nprod, known for the other rows, filled in for the
+// repeating ones.
+cudaError_t launch_repeats_finish(int64_t mw, int64_t *nprod, long long max_prod, const RepWord *words, RepWord *out,
+                                  cudaStream_t s);
+// The repeating rows of class `cls` and of the smaller classes that are not
+// launched (C.rpt holds offsets, the rows that they repeat are complete).
+// present: bit c set when class c is launched.
+cudaError_t launch_repeat_numeric(int cls, int present, const Operands &op, const RepWord *words, const int64_t *crpt,
+                                  int32_t *ccol, double *cval, int *err, cudaStream_t s);
 
 // --- runs.cu -------------------------------------------------------------------
 // Run boundaries of B rows at column sub-ranges of 2^gshift columns
@@ -287,8 +396,7 @@ cudaError_t launch_batch(int variant, int grid, const BatchProb *probs, const Ba
 int mlp_param_count();
 cudaError_t launch_features(const Operands &op, int64_t annz, int64_t mrows, long long *nprod, unsigned *maxlen,
                             unsigned *minlen, float *X, int grid, cudaStream_t s);
-cudaError_t launch_mlp_forward(const float *theta, const float *X, int64_t n, float *y,
-                               long long *sizes, float margin, long long cap, cudaStream_t s);
+cudaError_t launch_mlp_forward(const float *theta, const float *X, int64_t n, float *y, cudaStream_t s);
 cudaError_t launch_mlp_train(const float *theta, const float *X, const float *t, int64_t n,
                              int64_t n_total, float *grad, float *loss, cudaStream_t s);
 cudaError_t launch_adam(float *theta, const float *grad, float *m, float *v, int n, int step,
@@ -298,7 +406,21 @@ cudaError_t launch_learned_sizes(const int64_t *nprod, const long long *pred, in
                                  long long exact_above, long long huge, int64_t *sizes,
                                  const SizeFactors &sf, uint8_t *cls, unsigned long long *fb,
                                  cudaStream_t s);
-// copy one-phase rows from temporary memory into C (rows whose pred is -1 skipped)
-cudaError_t launch_copy_rows(const BinWork &w, cudaStream_t s);
+// Predicted sizes max(1, ceil(expm1(y) * (1 + margin))), at most cap, of all
+// rows, after launch_feature_scan.
+cudaError_t launch_predict(const Operands &op, int64_t mrows, const float *theta, const int64_t *nprod,
+                           const unsigned *maxlen, const unsigned *minlen, long long *pred, float margin,
+                           long long cap, cudaStream_t s);
+// The same for the rows that do not repeat a row before (gate as in
+// launch_feature_scan), and launch_learned_sizes of all rows (repeating rows
+// take n_prod) in one launch.
+cudaError_t launch_predict_few(const Operands &op, int64_t mrows, const float *theta, const int64_t *nprod,
+                               const unsigned *maxlen, const unsigned *minlen, const RepWord *words,
+                               const RepGate &gate, long long exact_above, long long huge, long long *pred,
+                               int64_t *sizes, const SizeFactors &sf, uint8_t *cls, unsigned long long *fb,
+                               float margin, long long cap, cudaStream_t s);
+// copy one-phase rows from temporary memory into C (rows whose pred is -1
+// skipped): their columns, their values or both
+cudaError_t launch_copy_rows(const BinWork &w, bool cols, bool vals, cudaStream_t s);
 
 }  // namespace ops

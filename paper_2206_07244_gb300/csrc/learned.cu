@@ -23,24 +23,27 @@ namespace ops {
 // n_prod, max and min referenced B-row length; then per row the six
 // features: log1p(nnz A_i), log1p(n_prod), log1p(max), log1p(mean),
 // log1p(min), log((i + 1) / M); empty A rows have max = mean = min = 0.
-__global__ void feature_finish_kernel(Operands op, int64_t mrows, const long long *nprod,
-                                      const unsigned *maxlen, const unsigned *minlen, float *X) {
-    const int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (r >= op.mw) return;
+__device__ __forceinline__ void row_features(const Operands &op, int64_t r, int64_t mrows, long long np,
+                                             unsigned maxlen, unsigned minlen, float *x) {
     const int64_t i = op.row0 + r;
     const long long na = ld_rpt(op.arpt, op.a64, i + 1) - ld_rpt(op.arpt, op.a64, i);
-    const long long np = nprod[r];
-    float *x = X + 6 * r;
     x[0] = log1pf(static_cast<float>(na));
     x[1] = log1pf(static_cast<float>(np));
     if (na > 0) {
-        x[2] = log1pf(static_cast<float>(maxlen[r]));
+        x[2] = log1pf(static_cast<float>(maxlen));
         x[3] = log1pf(static_cast<float>(static_cast<double>(np) / static_cast<double>(na)));
-        x[4] = log1pf(static_cast<float>(minlen[r]));
+        x[4] = log1pf(static_cast<float>(minlen));
     } else {
         x[2] = x[3] = x[4] = 0.f;
     }
     x[5] = logf(static_cast<float>(static_cast<double>(i + 1) / static_cast<double>(mrows)));
+}
+
+__global__ void feature_finish_kernel(Operands op, int64_t mrows, const long long *nprod,
+                                      const unsigned *maxlen, const unsigned *minlen, float *X) {
+    const int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (r >= op.mw) return;
+    row_features(op, r, mrows, nprod[r], maxlen[r], minlen[r], X + 6 * r);
 }
 
 cudaError_t launch_features(const Operands &op, int64_t annz, int64_t mrows, long long *nprod, unsigned *maxlen,
@@ -67,76 +70,271 @@ static_assert(kParams == 4673, "parameter count");
 
 int mlp_param_count() { return kParams; }
 
-// One row through the network. Weights are read from shared memory four at
+// R rows through the network. Weights are read from shared memory four at
 // a time (16-byte broadcast loads: every thread of a warp reads the same
-// address); each hidden unit sums its inputs in ascending order.
-__device__ __forceinline__ float mlp_row(const float *w, const float *x) {
-    float h1[kH];
+// address) and serve all R rows; each hidden unit sums its inputs in
+// ascending order.
+template <int R>
+__device__ __forceinline__ void mlp_rows(const float *w, const float (&x)[R][kIn], float (&y)[R]) {
+    float h1[R][kH];
 #pragma unroll
     for (int a = 0; a < kH; a += 4) {
-        float4 z = *reinterpret_cast<const float4 *>(w + kOffB1 + a);
+        const float4 b = *reinterpret_cast<const float4 *>(w + kOffB1 + a);
+        float4 z[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) z[r] = b;
 #pragma unroll
         for (int f = 0; f < kIn; ++f) {
             const float4 wv = *reinterpret_cast<const float4 *>(w + kOffW1 + f * kH + a);
-            z.x = fmaf(x[f], wv.x, z.x);
-            z.y = fmaf(x[f], wv.y, z.y);
-            z.z = fmaf(x[f], wv.z, z.z);
-            z.w = fmaf(x[f], wv.w, z.w);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                z[r].x = fmaf(x[r][f], wv.x, z[r].x);
+                z[r].y = fmaf(x[r][f], wv.y, z[r].y);
+                z[r].z = fmaf(x[r][f], wv.z, z[r].z);
+                z[r].w = fmaf(x[r][f], wv.w, z[r].w);
+            }
         }
-        h1[a] = fmaxf(z.x, 0.f);
-        h1[a + 1] = fmaxf(z.y, 0.f);
-        h1[a + 2] = fmaxf(z.z, 0.f);
-        h1[a + 3] = fmaxf(z.w, 0.f);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            h1[r][a] = fmaxf(z[r].x, 0.f);
+            h1[r][a + 1] = fmaxf(z[r].y, 0.f);
+            h1[r][a + 2] = fmaxf(z[r].z, 0.f);
+            h1[r][a + 3] = fmaxf(z[r].w, 0.f);
+        }
     }
-    float y = w[kOffB3];
+#pragma unroll
+    for (int r = 0; r < R; ++r) y[r] = w[kOffB3];
     for (int j = 0; j < kH; j += 4) {
-        float4 z = *reinterpret_cast<const float4 *>(w + kOffB2 + j);
+        const float4 b = *reinterpret_cast<const float4 *>(w + kOffB2 + j);
+        float4 z[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) z[r] = b;
 #pragma unroll
         for (int a = 0; a < kH; ++a) {
             const float4 wv = *reinterpret_cast<const float4 *>(w + kOffW2 + a * kH + j);
-            z.x = fmaf(h1[a], wv.x, z.x);
-            z.y = fmaf(h1[a], wv.y, z.y);
-            z.z = fmaf(h1[a], wv.z, z.z);
-            z.w = fmaf(h1[a], wv.w, z.w);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                z[r].x = fmaf(h1[r][a], wv.x, z[r].x);
+                z[r].y = fmaf(h1[r][a], wv.y, z[r].y);
+                z[r].z = fmaf(h1[r][a], wv.z, z[r].z);
+                z[r].w = fmaf(h1[r][a], wv.w, z[r].w);
+            }
         }
         const float4 w3 = *reinterpret_cast<const float4 *>(w + kOffW3 + j);
-        y = fmaf(fmaxf(z.x, 0.f), w3.x, y);
-        y = fmaf(fmaxf(z.y, 0.f), w3.y, y);
-        y = fmaf(fmaxf(z.z, 0.f), w3.z, y);
-        y = fmaf(fmaxf(z.w, 0.f), w3.w, y);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            y[r] = fmaf(fmaxf(z[r].x, 0.f), w3.x, y[r]);
+            y[r] = fmaf(fmaxf(z[r].y, 0.f), w3.y, y[r]);
+            y[r] = fmaf(fmaxf(z[r].z, 0.f), w3.z, y[r]);
+            y[r] = fmaf(fmaxf(z[r].w, 0.f), w3.w, y[r]);
+        }
     }
-    return y;
 }
 
-// Inference: y[i] = MLP(X[i]); if sizes != nullptr also the predicted row
-// size max(1, ceil(expm1(y) * (1 + margin))), capped at cap.
+__device__ __forceinline__ long long predicted_size(float y, float margin, long long cap) {
+    const float e = expm1f(fminf(y, 40.f)) * (1.f + margin);
+    const long long s = static_cast<long long>(ceilf(e));
+    return s < 1 ? 1 : (s > cap ? cap : s);
+}
+
+// Inference: y[i] = MLP(X[i]).
 __global__ void __launch_bounds__(256)
-mlp_forward_kernel(const float *theta, const float *X, int64_t n, float *y, long long *sizes,
-                   float margin, long long cap) {
+mlp_forward_kernel(const float *theta, const float *X, int64_t n, float *y) {
     __shared__ __align__(16) float w[kParams + 3];
     for (int i = threadIdx.x; i < kParams; i += blockDim.x) w[i] = theta[i];
     __syncthreads();
     const int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (r >= n) return;
-    float x[kIn];
+    float x[1][kIn], o[1];
 #pragma unroll
-    for (int f = 0; f < kIn; ++f) x[f] = X[kIn * r + f];
-    const float out = mlp_row(w, x);
-    if (y) y[r] = out;
-    if (sizes) {
-        const float e = expm1f(fminf(out, 40.f)) * (1.f + margin);
-        long long s = static_cast<long long>(ceilf(e));
-        if (s < 1) s = 1;
-        if (s > cap) s = cap;
-        sizes[r] = s;
+    for (int f = 0; f < kIn; ++f) x[0][f] = X[kIn * r + f];
+    mlp_rows<1>(w, x, o);
+    y[r] = o[0];
+}
+
+// Predicted sizes of 1024 window rows, two rows per thread at a time: the
+// weights' shared-memory loads bound one row per thread.
+constexpr int kPredictBlock = 128;
+constexpr int kPredictRows = 1024;
+
+__global__ void __launch_bounds__(kPredictBlock)
+predict_kernel(Operands op, int64_t mrows, const float *theta, const int64_t *nprod, const unsigned *maxlen,
+               const unsigned *minlen, long long *sizes, float margin, long long cap) {
+    __shared__ __align__(16) float w[kParams + 3];
+    for (int i = threadIdx.x; i < kParams; i += kPredictBlock) w[i] = theta[i];
+    __syncthreads();
+    const int64_t r0 = static_cast<int64_t>(blockIdx.x) * kPredictRows;
+    const int64_t r1 = r0 + kPredictRows < op.mw ? r0 + kPredictRows : op.mw;
+    for (int64_t ra = r0 + threadIdx.x; ra < r1; ra += 2 * kPredictBlock) {
+        const int64_t rb = ra + kPredictBlock < r1 ? ra + kPredictBlock : ra;   // the second row, or the first again
+        float x[2][kIn], y[2];
+        row_features(op, ra, mrows, nprod[ra], maxlen[ra], minlen[ra], x[0]);
+        row_features(op, rb, mrows, nprod[rb], maxlen[rb], minlen[rb], x[1]);
+        mlp_rows<2>(w, x, y);
+        sizes[ra] = predicted_size(y[0], margin, cap);
+        if (rb != ra) sizes[rb] = predicted_size(y[1], margin, cap);
     }
 }
 
-cudaError_t launch_mlp_forward(const float *theta, const float *X, int64_t n, float *y,
-                               long long *sizes, float margin, long long cap, cudaStream_t s) {
+// Size of a row for the binning by prediction: rows whose n_prod passes
+// exact_above go to the exact path (huge); the others take their class's
+// factor on the predicted size (class = bin of the prediction), at least 1 and
+// at most n_prod (an upper bound of n_nz). hist counts, per class, the rows
+// that land in a hash bin.
+__device__ __forceinline__ long long binned_size(long long np, long long p, long long exact_above, long long huge,
+                                                 const SizeFactors &sf, uint8_t *cls, unsigned *hist) {
+    int b = 0;
+    while (b < sf.nb - 1 && p > sf.lim[b]) ++b;
+    *cls = static_cast<uint8_t>(b);
+    if (np > exact_above) return huge;
+    const int k = sf.k[b];
+    long long q = k >= 0 ? (p << k) : ((p + (1ll << -k) - 1) >> -k);
+    if (q < 1) q = 1;
+    const long long sz = q < np ? q : np;
+    if (b < sf.nb - 1 && sz <= sf.lim[sf.nb - 2]) atomicAdd(&hist[b], 1u);
+    return sz;
+}
+
+__device__ __forceinline__ void add_feedback(const unsigned *hist, unsigned long long *fb) {
+    if (fb && threadIdx.x < kMaxBins && hist[threadIdx.x] > 0u)
+        atomicAdd(fb + threadIdx.x * kLoadSlots + blockIdx.x % kLoadSlots,
+                  static_cast<unsigned long long>(hist[threadIdx.x]));
+}
+
+// The same for the rows that do not repeat a row before, where most rows
+// repeat (of a 27-point stencil 128^3 one in 25 does not): a block finds too few for a row per thread (a thread's 4,673 multiply-adds would be the
+// block's time), so a warp takes a row, two hidden units per lane.
+__global__ void __launch_bounds__(256)
+predict_few_kernel(Operands op, int64_t mrows, const float *theta, const int64_t *nprod, const unsigned *maxlen,
+                   const unsigned *minlen, const RepWord *words, RepGate gate, long long exact_above, long long huge,
+                   long long *pred, int64_t *sizes, SizeFactors sf, uint8_t *cls, unsigned long long *fb, float margin,
+                   long long cap) {
+    __shared__ unsigned hist[kMaxBins];
+    if (threadIdx.x < kMaxBins) hist[threadIdx.x] = 0u;
+    const bool scanned = gate.shut();   // the setup scan went over every row: maxlen and minlen are there
+    __shared__ float w[kParams];
+    __shared__ int s_row[kPredictRows], s_n;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    const int64_t r0 = static_cast<int64_t>(blockIdx.x) * kPredictRows;
+    for (int k = threadIdx.x; k < kPredictRows; k += 256) {
+        const int64_t r = r0 + k;
+        if (r >= op.mw) continue;
+        if ((words[r >> 5].fol >> (r & 31)) & 1u) sizes[r] = nprod[r];   // in no bin
+        else s_row[atomicAdd(&s_n, 1)] = k;
+    }
+    for (int i = threadIdx.x; i < kParams; i += 256) w[i] = theta[i];
+    __syncthreads();
+    const int n = s_n, lane = threadIdx.x & 31;
+    constexpr int kBatch = 4;   // rows a warp takes at a time (8 lanes each): they share the loads of the weights
+    __shared__ __align__(16) float s_h[8][kBatch][kH];
+    float(*h)[kH] = s_h[threadIdx.x >> 5];
+    for (int j0 = (threadIdx.x >> 5) * kBatch; j0 < n; j0 += 8 * kBatch) {   // uniform over the warp
+        // features of one row per lane (lane l: row l % kBatch)
+        const int at = j0 + lane % kBatch;
+        const int64_t mine = r0 + s_row[at < n ? at : j0];
+        unsigned mx = 0, mn = UINT_MAX;
+        if (scanned) {
+            mx = maxlen[mine];
+            mn = minlen[mine];
+        } else {
+            // the longest and shortest B row, 8 lanes per row; rows past
+            // exact_above products take the exact path anyway
+            const int64_t r = __shfl_sync(0xffffffffu, mine, lane >> 3);
+            if (nprod[r] <= exact_above) {
+                const int64_t e = ld_rpt(op.arpt, op.a64, op.row0 + r + 1);
+                for (int64_t p = ld_rpt(op.arpt, op.a64, op.row0 + r) + (lane & 7); p < e; p += 8) {
+                    const int k = __ldg(op.acol + p);
+                    const unsigned len =
+                        static_cast<unsigned>(ld_rpt(op.brpt, op.b64, k + 1) - ld_rpt(op.brpt, op.b64, k));
+                    mx = max(mx, len);
+                    mn = min(mn, len);
+                }
+            }
+            for (int o = 4; o > 0; o >>= 1) {
+                mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+                mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+            }
+            mx = __shfl_sync(0xffffffffu, mx, (lane % kBatch) * 8);
+            mn = __shfl_sync(0xffffffffu, mn, (lane % kBatch) * 8);
+        }
+        float x[kIn];
+        row_features(op, mine, mrows, nprod[mine], mx, mn, x);
+        __syncwarp();   // readers of the batch before are done
+#pragma unroll
+        for (int q = 0; q < kBatch; ++q) {
+            float a = w[kOffB1 + lane], b = w[kOffB1 + 32 + lane];
+#pragma unroll
+            for (int f = 0; f < kIn; ++f) {
+                const float xf = __shfl_sync(0xffffffffu, x[f], q);
+                a = fmaf(xf, w[kOffW1 + f * kH + lane], a);
+                b = fmaf(xf, w[kOffW1 + f * kH + 32 + lane], b);
+            }
+            h[q][lane] = fmaxf(a, 0.f);
+            h[q][32 + lane] = fmaxf(b, 0.f);
+        }
+        __syncwarp();
+        float z[kBatch][2];
+#pragma unroll
+        for (int q = 0; q < kBatch; ++q) {
+            z[q][0] = w[kOffB2 + lane];
+            z[q][1] = w[kOffB2 + 32 + lane];
+        }
+        for (int a = 0; a < kH; a += 4) {   // inputs in ascending order
+            float wa[4], wb[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                wa[k] = w[kOffW2 + (a + k) * kH + lane];
+                wb[k] = w[kOffW2 + (a + k) * kH + 32 + lane];
+            }
+#pragma unroll
+            for (int q = 0; q < kBatch; ++q) {
+                const float4 v = *reinterpret_cast<const float4 *>(&h[q][a]);
+                z[q][0] = fmaf(v.w, wa[3], fmaf(v.z, wa[2], fmaf(v.y, wa[1], fmaf(v.x, wa[0], z[q][0]))));
+                z[q][1] = fmaf(v.w, wb[3], fmaf(v.z, wb[2], fmaf(v.y, wb[1], fmaf(v.x, wb[0], z[q][1]))));
+            }
+        }
+        float out = 0.f;
+#pragma unroll
+        for (int q = 0; q < kBatch; ++q) {
+            float y = fmaf(fmaxf(z[q][0], 0.f), w[kOffW3 + lane], fmaxf(z[q][1], 0.f) * w[kOffW3 + 32 + lane]);
+            for (int o = 16; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+            if (lane == q) out = y + w[kOffB3];
+        }
+        if (lane < kBatch && at < n) {
+            const long long p = predicted_size(out, margin, cap);
+            pred[mine] = p;
+            sizes[mine] = binned_size(nprod[mine], p, exact_above, huge, sf, cls + mine, hist);
+        }
+    }
+    __syncthreads();
+    add_feedback(hist, fb);
+}
+
+cudaError_t launch_predict(const Operands &op, int64_t mrows, const float *theta, const int64_t *nprod,
+                           const unsigned *maxlen, const unsigned *minlen, long long *pred, float margin,
+                           long long cap, cudaStream_t s) {
+    if (op.mw <= 0) return cudaSuccess;
+    predict_kernel<<<static_cast<unsigned>((op.mw + kPredictRows - 1) / kPredictRows), kPredictBlock, 0, s>>>(
+        op, mrows, theta, nprod, maxlen, minlen, pred, margin, cap);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_predict_few(const Operands &op, int64_t mrows, const float *theta, const int64_t *nprod,
+                               const unsigned *maxlen, const unsigned *minlen, const RepWord *words,
+                               const RepGate &gate, long long exact_above, long long huge, long long *pred,
+                               int64_t *sizes, const SizeFactors &sf, uint8_t *cls, unsigned long long *fb,
+                               float margin, long long cap, cudaStream_t s) {
+    if (op.mw <= 0) return cudaSuccess;
+    if (sf.nb < 1 || sf.nb > kMaxBins) return cudaErrorInvalidValue;
+    predict_few_kernel<<<static_cast<unsigned>((op.mw + kPredictRows - 1) / kPredictRows), 256, 0, s>>>(
+        op, mrows, theta, nprod, maxlen, minlen, words, gate, exact_above, huge, pred, sizes, sf, cls, fb, margin, cap);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mlp_forward(const float *theta, const float *X, int64_t n, float *y, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    mlp_forward_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, s>>>(theta, X, n, y, sizes,
-                                                                              margin, cap);
+    mlp_forward_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, s>>>(theta, X, n, y);
     return cudaGetLastError();
 }
 
@@ -266,11 +464,8 @@ cudaError_t launch_adam(float *theta, const float *grad, float *m, float *v, int
 // Sizes for the learned binning: rows past the symbolic hash bins go to
 // the exact path (a huge size); others get min(prediction, n_prod), since a
 // row never has more distinct keys than products.
-// Sizes for the binning by prediction: rows whose n_prod passes exact_above
-// go to the exact path (huge); the others take their class's factor on the
-// predicted size (class = bin of the prediction), at least 1 and at most
-// n_prod (an upper bound of n_nz). Each block counts its rows per class that
-// land in a hash bin (tried in one phase) into the feedback counters.
+// Each block of these kernels counts its rows per class that land in a hash
+// bin (tried in one phase) into the feedback counters.
 __global__ void __launch_bounds__(256)
 learned_sizes_kernel(const int64_t *nprod, const long long *pred, int64_t n, long long exact_above,
                      long long huge, int64_t *sizes, SizeFactors sf, uint8_t *cls,
@@ -280,25 +475,10 @@ learned_sizes_kernel(const int64_t *nprod, const long long *pred, int64_t n, lon
     __syncthreads();
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i < n) {
-        const long long np = nprod[i];
-        const long long p = pred[i];
-        int b = 0;
-        while (b < sf.nb - 1 && p > sf.lim[b]) ++b;
-        long long sz = huge;
-        if (np <= exact_above) {
-            const int k = sf.k[b];
-            long long q = k >= 0 ? (p << k) : ((p + (1ll << -k) - 1) >> -k);
-            if (q < 1) q = 1;
-            sz = q < np ? q : np;
-            if (b < sf.nb - 1 && sz <= sf.lim[sf.nb - 2]) atomicAdd(&hist[b], 1u);
-        }
-        sizes[i] = sz;
-        cls[i] = static_cast<uint8_t>(b);
+        sizes[i] = binned_size(nprod[i], pred[i], exact_above, huge, sf, cls + i, hist);
     }
     __syncthreads();
-    if (fb && threadIdx.x < kMaxBins && hist[threadIdx.x] > 0u)
-        atomicAdd(fb + threadIdx.x * kLoadSlots + blockIdx.x % kLoadSlots,
-                  static_cast<unsigned long long>(hist[threadIdx.x]));
+    add_feedback(hist, fb);
 }
 
 cudaError_t launch_learned_sizes(const int64_t *nprod, const long long *pred, int64_t n,
@@ -348,7 +528,7 @@ int spgemm_features(const spgemm_csr_in *A, const spgemm_csr_in *B, int64_t row_
 
 int spgemm_mlp_forward(const float *theta, const float *X, int64_t n, float *y, void *stream) {
     if (!theta || (n > 0 && (!X || !y)) || n < 0) return SPGEMM_ERR_INVALID;
-    return launch_mlp_forward(theta, X, n, y, nullptr, 0.f, 0, static_cast<cudaStream_t>(stream)) ==
+    return launch_mlp_forward(theta, X, n, y, static_cast<cudaStream_t>(stream)) ==
                    cudaSuccess
                ? SPGEMM_OK
                : SPGEMM_ERR_CUDA;

@@ -950,6 +950,7 @@ cudaError_t launch_num_onephase(int id, const Operands &op, const BinWork &w, cu
 
 // Copies the one-phase rows of a bin from their temporary slots into C: one
 // warp per row, rows marked -1 in pred (mispredicted) are skipped.
+template <bool COLS, bool VALS>
 __global__ void copy_rows_kernel(BinWork w) {
     const int64_t r = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
@@ -972,26 +973,24 @@ __global__ void copy_rows_kernel(BinWork w) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int64_t t = t0 + u * 32 + lane;
-            if (t < n) {
-                c[u] = __ldg(scol + t);
-                v[u] = __ldg(sval + t);
-            }
+            if (COLS && t < n) c[u] = __ldg(scol + t);
+            if (VALS && t < n) v[u] = __ldg(sval + t);
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int64_t t = t0 + u * 32 + lane;
-            if (t < n) {
-                w.ccol[base + t] = c[u];
-                w.cval[base + t] = v[u];
-            }
+            if (COLS && t < n) w.ccol[base + t] = c[u];
+            if (VALS && t < n) w.cval[base + t] = v[u];
         }
     }
 }
 
-cudaError_t launch_copy_rows(const BinWork &w, cudaStream_t s) {
+cudaError_t launch_copy_rows(const BinWork &w, bool cols, bool vals, cudaStream_t s) {
     if (w.cnt <= 0) return cudaSuccess;
     const int64_t threads = w.cnt * 32;
-    copy_rows_kernel<<<static_cast<unsigned>((threads + 255) / 256), 256, 0, s>>>(w);
+    const auto kernel = !vals ? &copy_rows_kernel<true, false>
+                              : !cols ? &copy_rows_kernel<false, true> : &copy_rows_kernel<true, true>;
+    kernel<<<static_cast<unsigned>((threads + 255) / 256), 256, 0, s>>>(w);
     return cudaGetLastError();
 }
 

@@ -57,11 +57,12 @@ __device__ __forceinline__ int lanes_per_row(int64_t entries, int64_t rows) {
 // Block `blk` of `nblk`: lengths of the B rows that A's entries in the
 // window reference, reduced per row: the sum into nprod and, with FEAT, the
 // largest and smallest into maxlen / minlen (all set to their neutral value
-// before). A row inside one tile is stored by one thread, a row cut by a
+// before). With `words` the repeating rows are left out, and the entries of
+// the others are not staged (most of the tile is not read). A row inside one tile is stored by one thread, a row cut by a
 // tile's edge is combined with atomics.
 template <bool FEAT>
 __device__ __forceinline__ void row_lengths(const Operands &op, int64_t *nprod, unsigned *maxlen, unsigned *minlen,
-                                            int blk, int nblk, int *s_len) {
+                                            const RepWord *words, int blk, int nblk, int *s_len) {
     const int64_t lo = op.row0, hi = op.row0 + op.mw;
     const int64_t pb = ld_rpt(op.arpt, op.a64, lo), pe = ld_rpt(op.arpt, op.a64, hi);
     const int64_t tiles = (pe - pb + kTileEntries - 1) / kTileEntries;
@@ -78,7 +79,7 @@ __device__ __forceinline__ void row_lengths(const Operands &op, int64_t *nprod, 
 #pragma unroll
         for (int j = 0; j < kTileItems; ++j) {
             const int64_t p = t0 + j * kTileBlock + threadIdx.x;
-            k[j] = p < t1 ? __ldg(op.acol + p) : -1;
+            k[j] = !words && p < t1 ? __ldg(op.acol + p) : -1;
         }
 #pragma unroll
         for (int j = 0; j < kTileItems; ++j)
@@ -96,23 +97,30 @@ __device__ __forceinline__ void row_lengths(const Operands &op, int64_t *nprod, 
                 e = ld_rpt(op.arpt, op.a64, i + 1);
             }
             const int a = static_cast<int>((s > t0 ? s : t0) - t0), b = static_cast<int>((e < t1 ? e : t1) - t0);
-            if (s < t1)
+            const bool own = s < t1 && !(words && ((words[(i - lo) >> 5].fol >> ((i - lo) & 31)) & 1u));
+            if (own)
                 for (int q = a + l; q < b; q += L) {
-                    const int len = s_len[q];
+                    int len;
+                    if (words) {
+                        const int c = __ldg(op.acol + t0 + q);
+                        len = static_cast<int>(ld_rpt(op.brpt, op.b64, c + 1) - ld_rpt(op.brpt, op.b64, c));
+                    } else {
+                        len = s_len[q];
+                    }
                     sum += len;
                     if (FEAT) {
                         mx = max(mx, static_cast<unsigned>(len));
                         mn = min(mn, static_cast<unsigned>(len));
                     }
                 }
-            for (int o = L >> 1; o > 0; o >>= 1) {
+            for (int o = __any_sync(0xffffffffu, own) ? L >> 1 : 0; o > 0; o >>= 1) {
                 sum += __shfl_xor_sync(0xffffffffu, sum, o);
                 if (FEAT) {
                     mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
                     mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
                 }
             }
-            if (l == 0 && s < t1 && a < b) {
+            if (l == 0 && own && a < b) {
                 const int64_t r = i - lo;
                 if (s >= t0 && e <= t1) {
                     nprod[r] = sum;
@@ -192,19 +200,23 @@ __device__ __forceinline__ void order_check(const Operands &op, int64_t brows, i
 // Both scans in one launch: the first `nprod_blocks` blocks count products,
 // the others check B's order (either part may have no blocks).
 __global__ void __launch_bounds__(kTileBlock)
-setup_kernel(Operands op, int64_t *nprod, int nprod_blocks, int64_t brows, int64_t bnnz, Counters *cnt) {
+setup_kernel(Operands op, int64_t *nprod, const RepWord *words, RepGate gate, bool only_open, int nprod_blocks,
+             int64_t brows, int64_t bnnz, Counters *cnt) {
     __shared__ int s_len[kTileEntries + 4];
-    if (static_cast<int>(blockIdx.x) < nprod_blocks)
-        row_lengths<false>(op, nprod, nullptr, nullptr, blockIdx.x, nprod_blocks, s_len);
-    else
+    if (static_cast<int>(blockIdx.x) < nprod_blocks) {
+        const bool shut = gate.shut();
+        if (shut && only_open) return;   // uniform over the block
+        row_lengths<false>(op, nprod, nullptr, nullptr, shut ? nullptr : words, blockIdx.x, nprod_blocks, s_len);
+    } else
         order_check(op, brows, bnnz, cnt, blockIdx.x - nprod_blocks, gridDim.x - nprod_blocks,
                     reinterpret_cast<unsigned char *>(s_len));
 }
 
 __global__ void __launch_bounds__(kTileBlock)
-feature_scan_kernel(Operands op, int64_t *nprod, unsigned *maxlen, unsigned *minlen) {
+feature_scan_kernel(Operands op, int64_t *nprod, unsigned *maxlen, unsigned *minlen, RepGate gate) {
     __shared__ int s_len[kTileEntries];
-    row_lengths<true>(op, nprod, maxlen, minlen, blockIdx.x, gridDim.x, s_len);
+    if (gate.found && !gate.shut()) return;   // uniform over the grid
+    row_lengths<true>(op, nprod, maxlen, minlen, nullptr, blockIdx.x, gridDim.x, s_len);
 }
 
 // Blocks for `entries` entries: at most `grid`, no more than there are tiles.
@@ -214,18 +226,19 @@ static int tile_grid(int64_t entries, int grid) {
 }
 
 cudaError_t launch_setup(const Operands &op, int64_t annz, int64_t *nprod, int64_t brows, int64_t bnnz,
-                         Counters *cnt, int grid, cudaStream_t s) {
+                         Counters *cnt, int grid, cudaStream_t s, const RepWord *words, const RepGate &gate,
+                         bool only_open) {
     const int na = nprod && op.mw > 0 ? tile_grid(annz, grid) : 0;
     const int nb = cnt && bnnz > 1 && brows > 0 ? tile_grid(bnnz, grid) : 0;
     if (na + nb == 0) return cudaSuccess;
-    setup_kernel<<<na + nb, kTileBlock, 0, s>>>(op, nprod, na, brows, bnnz, cnt);
+    setup_kernel<<<na + nb, kTileBlock, 0, s>>>(op, nprod, words, gate, only_open, na, brows, bnnz, cnt);
     return cudaGetLastError();
 }
 
 cudaError_t launch_feature_scan(const Operands &op, int64_t annz, int64_t *nprod, unsigned *maxlen, unsigned *minlen,
-                                int grid, cudaStream_t s) {
+                                int grid, cudaStream_t s, const RepGate &gate) {
     if (op.mw <= 0) return cudaSuccess;
-    feature_scan_kernel<<<tile_grid(annz, grid), kTileBlock, 0, s>>>(op, nprod, maxlen, minlen);
+    feature_scan_kernel<<<tile_grid(annz, grid), kTileBlock, 0, s>>>(op, nprod, maxlen, minlen, gate);
     return cudaGetLastError();
 }
 
@@ -264,8 +277,10 @@ __device__ __forceinline__ unsigned long long group_total(unsigned same, unsigne
 // for: 57 us for 4,096 rows, 0.265 ms for 2.1M rows in one bin.)
 __global__ void __launch_bounds__(kBinBlock)
 bin_pass1_kernel(const int64_t *sizes, int64_t n, Ranges rg, Operands op, Counters *cnt,
-                 long long *tile_sums) {
+                 long long *tile_sums, RepArgs rep) {
     constexpr int kWarps = kBinBlock / 32;
+    __shared__ unsigned s_own[kWarps][kMaxBins];
+    __shared__ unsigned s_rep[kRepClasses];
     __shared__ unsigned s_cnt[kWarps][kMaxBins];
     __shared__ unsigned long long s_bsum[kWarps][kMaxBins];
     __shared__ unsigned long long s_bnza[kWarps][kMaxBins];
@@ -273,8 +288,13 @@ bin_pass1_kernel(const int64_t *sizes, int64_t n, Ranges rg, Operands op, Counte
     const unsigned lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
     if (lane < kMaxBins) {
         s_cnt[w][lane] = 0;
+        s_own[w][lane] = 0;
         s_bsum[w][lane] = 0;
         s_bnza[w][lane] = 0;
+    }
+    if (rep.words) {   // uniform
+        if (threadIdx.x < kRepClasses) s_rep[threadIdx.x] = 0;
+        __syncthreads();
     }
     __syncwarp();
     const int64_t tile0 = static_cast<int64_t>(blockIdx.x) * kBinTile;
@@ -289,10 +309,31 @@ bin_pass1_kernel(const int64_t *sizes, int64_t n, Ranges rg, Operands op, Counte
             na[it] = static_cast<unsigned long long>(ld_rpt(op.arpt, op.a64, ar + 1) - ld_rpt(op.arpt, op.a64, ar));
         }
     }
+    unsigned out = 0;   // bit it: the row is left out of the bins
+    if (rep.words) {
+#pragma unroll
+        for (int it = 0; it < kBinItems; ++it) {
+            const int64_t i = tile0 + it * kBinBlock + threadIdx.x;
+            const RepWord rw = i < n ? rep.words[i >> 5] : RepWord{};
+            int c = -1;
+            if ((rw.fol >> (i & 31)) & 1u) {
+                if (rep.fill) {
+                    const long long np = static_cast<long long>(v[it]);
+                    v[it] = static_cast<unsigned long long>(sizes[rep_own(rw, i)]);
+                    rep.fill[i] = static_cast<int64_t>(v[it]);
+                    if (static_cast<long long>(v[it]) <= rep.max_nnz) c = rep_class(np, static_cast<long long>(v[it]));
+                }
+                if (static_cast<long long>(v[it]) <= rep.max_nnz) out |= 1u << it;
+            }
+            const unsigned same = __match_any_sync(0xffffffffu, c);
+            if (c >= 0 && lane == static_cast<unsigned>(__ffs(same) - 1)) atomicAdd(&s_rep[c], __popc(same));
+        }
+    }
     unsigned long long my_max = 0;
 #pragma unroll
     for (int it = 0; it < kBinItems; ++it) {
         const bool valid = tile0 + it * kBinBlock + threadIdx.x < n;
+        const unsigned left = __ballot_sync(0xffffffffu, (out >> it) & 1u);
         my_max = my_max > v[it] ? my_max : v[it];
         const int j = valid ? bin_of(static_cast<long long>(v[it]), rg) : -1;
         const unsigned same = __match_any_sync(0xffffffffu, j);
@@ -300,6 +341,7 @@ bin_pass1_kernel(const int64_t *sizes, int64_t n, Ranges rg, Operands op, Counte
         const unsigned long long sv = group_total(same, v[it], small), sn = group_total(same, na[it], small);
         if (valid && lane == static_cast<unsigned>(__ffs(same) - 1)) {
             s_cnt[w][j] += static_cast<unsigned>(__popc(same));
+            s_own[w][j] += static_cast<unsigned>(__popc(same & ~left));
             s_bsum[w][j] += sv;
             s_bnza[w][j] += sn;
         }
@@ -312,11 +354,12 @@ bin_pass1_kernel(const int64_t *sizes, int64_t n, Ranges rg, Operands op, Counte
     if (lane == 0) s_max[w] = my_max;
     __syncthreads();
     if (w == 0) {
-        unsigned c = 0;
+        unsigned c = 0, own = 0;
         unsigned long long bs = 0, bn = 0, mx = 0;
         for (int q = 0; q < kWarps; ++q) {
             if (lane < kMaxBins) {
                 c += s_cnt[q][lane];
+                own += s_own[q][lane];
                 bs += s_bsum[q][lane];
                 bn += s_bnza[q][lane];
             }
@@ -328,7 +371,10 @@ bin_pass1_kernel(const int64_t *sizes, int64_t n, Ranges rg, Operands op, Counte
             atomicAdd(&cnt->bin_cnt[lane], static_cast<unsigned long long>(c));
             atomicAdd(&cnt->bin_sum[lane], bs);
             atomicAdd(&cnt->bin_nnza[lane], bn);
+            if (own) atomicAdd(&cnt->bin_own[lane], static_cast<unsigned long long>(own));
         }
+        if (rep.words && lane < kRepClasses && s_rep[lane])
+            atomicAdd(&cnt->rep_cnt[lane], static_cast<unsigned long long>(s_rep[lane]));
         if (lane == 0) {
             atomicMax(&cnt->max_size, mx);
             atomicAdd(&cnt->total, sum);
@@ -339,7 +385,7 @@ bin_pass1_kernel(const int64_t *sizes, int64_t n, Ranges rg, Operands op, Counte
 
 __global__ void __launch_bounds__(kBinBlock)
 bin_pass2_kernel(const int64_t *sizes, int64_t n, Ranges rg, Counters *cnt, int32_t *bins,
-                 Ranges off) {
+                 Ranges off, RepArgs rep) {
     __shared__ unsigned s_cnt[kMaxBins];
     __shared__ long long s_base[kMaxBins];
     if (threadIdx.x < kMaxBins) s_cnt[threadIdx.x] = 0;
@@ -351,8 +397,10 @@ bin_pass2_kernel(const int64_t *sizes, int64_t n, Ranges rg, Counters *cnt, int3
 #pragma unroll
     for (int it = 0; it < kBinItems; ++it) {
         const int64_t i = tile0 + it * kBinBlock + threadIdx.x;
-        const bool valid = i < n;
-        const int j = valid ? bin_of(sizes[i], rg) : -1;
+        bool valid = i < n;
+        const long long v = valid ? sizes[i] : 0;
+        if (rep.words && valid) valid = !((rep.words[i >> 5].fol >> (i & 31)) & 1u) || v > rep.max_nnz;
+        const int j = valid ? bin_of(v, rg) : -1;
         const unsigned same = __match_any_sync(0xffffffffu, j);
         const int leader = __ffs(same) - 1;
         unsigned wbase = 0;
@@ -374,30 +422,30 @@ bin_pass2_kernel(const int64_t *sizes, int64_t n, Ranges rg, Counters *cnt, int3
 #pragma unroll
     for (int it = 0; it < kBinItems; ++it) {
         const int64_t i = tile0 + it * kBinBlock + threadIdx.x;
-        if (i < n) bins[s_base[jv[it]] + pos[it]] = static_cast<int32_t>(i);
+        if (jv[it] >= 0) bins[s_base[jv[it]] + pos[it]] = static_cast<int32_t>(i);
     }
 }
 
 cudaError_t launch_bin_pass1(const int64_t *sizes, int64_t n, const Ranges &rg,
                              const Operands &op, Counters *cnt, long long *tile_sums,
-                             cudaStream_t s) {
+                             cudaStream_t s, const RepArgs &rep) {
     if (n <= 0) return cudaSuccess;
     const int64_t grid = (n + kBinTile - 1) / kBinTile;
     bin_pass1_kernel<<<static_cast<unsigned>(grid), kBinBlock, 0, s>>>(sizes, n, rg, op, cnt,
-                                                                       tile_sums);
+                                                                       tile_sums, rep);
     return cudaGetLastError();
 }
 
 cudaError_t launch_bin_pass2(const int64_t *sizes, int64_t n, const Ranges &rg,
                              const long long *offsets, Counters *cnt, int32_t *bins,
-                             cudaStream_t s) {
+                             cudaStream_t s, const RepArgs &rep) {
     if (n <= 0) return cudaSuccess;
     Ranges off{};
     off.nb = rg.nb;
     for (int j = 0; j < rg.nb; ++j) off.r[j] = offsets[j];
     const int64_t grid = (n + kBinTile - 1) / kBinTile;
     bin_pass2_kernel<<<static_cast<unsigned>(grid), kBinBlock, 0, s>>>(sizes, n, rg, cnt, bins,
-                                                                       off);
+                                                                       off, rep);
     return cudaGetLastError();
 }
 
