@@ -619,4 +619,68 @@ __device__ __forceinline__ void group_row_walk(const Operands &op, int64_t p0, i
     }
 }
 
+// --- rows of at most 8 products -----------------------------------------------
+// A row group of 8 lanes holds such a row in registers, one product per lane
+// in the order of A's entries, when the row has at most 8 A entries. Equal
+// columns are found by comparing with the other 7 lanes, so the row needs no
+// table, no probes and no sort, and repeated or unsorted columns are handled
+// like any other. Bound by the chain of loads to B (7-point operator 128^3
+// times a piecewise-constant prolongation, 2.1M rows of 7 products).
+struct TinyRow {
+    int total;         // products (the row is only usable when tiny_load returned true)
+    int col;           // the lane's column, -1 past the products
+    double a, b;       // its values (NEED_VAL)
+    unsigned lt, eq;   // products of the row with a smaller / the same column
+    bool first;        // the first product of its column
+    unsigned heads;    // first products of the row
+};
+
+// Loads the row [p0, p1) of A (p0 == p1: none). True on every lane of the
+// warp, and r set, when all four rows of the warp fit.
+template <bool NEED_VAL>
+__device__ __forceinline__ bool tiny_load(const Operands &op, int64_t p0, int64_t p1, TinyRow &r) {
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31, lg = lane & 7;
+    const int64_t na = p1 - p0;
+    if (!__all_sync(kAll, na <= 8)) return false;
+    long long q0 = 0, len64 = 0;
+    double a = 0.0;
+    if (lg < na) {
+        const int k = __ldg(op.acol + p0 + lg);
+        q0 = ld_rpt(op.brpt, op.b64, k);
+        len64 = ld_rpt(op.brpt, op.b64, k + 1) - q0;
+        if (NEED_VAL) a = __ldg(op.aval + p0 + lg);
+    }
+    const int len = static_cast<int>(len64 < 9 ? len64 : 9);   // 9: too many, and no overflow in the sums
+    int inc = len;
+    for (int o = 1; o < 8; o <<= 1) {
+        const int y = __shfl_up_sync(kAll, inc, o, 8);
+        if (lg >= o) inc += y;
+    }
+    r.total = __shfl_sync(kAll, inc, 7, 8);
+    if (!__all_sync(kAll, r.total <= 8)) return false;
+    // product lg belongs to the entry e with inc[e - 1] <= lg < inc[e]
+    int e = 0;
+#pragma unroll
+    for (int step = 4; step > 0; step >>= 1)
+        if (__shfl_sync(kAll, inc, e + step - 1, 8) <= lg) e += step;
+    const bool valid = lg < r.total;
+    const long long q = __shfl_sync(kAll, q0, e, 8) + lg - __shfl_sync(kAll, inc - len, e, 8);
+    r.col = valid ? __ldg(op.bcol + q) : -1;
+    if (NEED_VAL) {
+        r.a = __shfl_sync(kAll, a, e, 8);
+        r.b = valid ? __ldg(op.bval + q) : 0.0;
+    }
+    r.lt = r.eq = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const int c = __shfl_sync(kAll, r.col, j, 8);
+        r.lt |= (c >= 0 && c < r.col ? 1u : 0u) << j;
+        r.eq |= (c == r.col ? 1u : 0u) << j;
+    }
+    r.first = valid && (r.eq & ((1u << lg) - 1u)) == 0;
+    r.heads = (__ballot_sync(kAll, r.first) >> (lane - lg)) & 0xffu;
+    return true;
+}
+
 }  // namespace ops

@@ -190,10 +190,6 @@ num_hash_kernel(Operands op, BinWork w) {
     const int64_t r = static_cast<int64_t>(blockIdx.x) * RPB + g;
     const bool valid = r < w.cnt;
     const int64_t row = valid ? (w.bins ? static_cast<int64_t>(w.bins[w.off + r]) : w.off + r) : 0;
-    for (int s = lg; s < T; s += TPR) {
-        tk[s] = -1;
-        tv[s] = 0.0;
-    }
     int64_t cbase = 0, n_expect = 0, p0 = 0, p1 = 0;
     if (valid) {
         if (!ONE_PHASE) {
@@ -203,6 +199,32 @@ num_hash_kernel(Operands op, BinWork w) {
         const int64_t ar = op.row0 + row;
         p0 = ld_rpt(op.arpt, op.a64, ar);
         p1 = ld_rpt(op.arpt, op.a64, ar + 1);
+    }
+    if constexpr (TPR == 8 && !ONE_PHASE && !MULTI) {
+        // all four rows of the warp have at most 8 products (2.1M rows of 7:
+        // 862 -> 277 us)
+        TinyRow t;
+        if (tiny_load<true>(op, p0, p1, t)) {
+            double sum = 0.0;
+            unsigned m = t.first ? t.eq : 0u;
+            while (__any_sync(0xffffffffu, m)) {   // in the order of A's entries
+                const int j = m ? __ffs(m) - 1 : 0;
+                const double a = __shfl_sync(0xffffffffu, t.a, j, 8), b = __shfl_sync(0xffffffffu, t.b, j, 8);
+                if (m) sum = fma(a, b, sum);
+                m &= m - 1;
+            }
+            const int rank = __popc(t.lt & t.heads);
+            if (t.first && rank < n_expect) {
+                w.ccol[cbase + rank] = t.col;
+                w.cval[cbase + rank] = sum;
+            }
+            if (valid && lg == 0 && __popc(t.heads) != n_expect) set_error(w.err, DERR_COUNT_MISMATCH);
+            return;   // uniform over the warp; no block barrier follows
+        }
+    }
+    for (int s = lg; s < T; s += TPR) {
+        tk[s] = -1;
+        tv[s] = 0.0;
     }
     const int S = numeric_lanes<TPR>(op, w.lanes, p0, p1, lg, red64);
     group_sync<TPR>();
