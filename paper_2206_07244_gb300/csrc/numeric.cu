@@ -93,6 +93,34 @@ __device__ __forceinline__ int numeric_lanes(const Operands &op, int fixed, int6
     return pick_lanes_distinct(0, sum, p1 - p0, TPR);
 }
 
+// Accumulator of a column that no product has reached: a signalling NaN, which
+// no arithmetic result is.
+constexpr long long kNoEntry = 0x7ff0000000000001ll;
+
+// Products of the row [p0, p1) and, for rows of B in strictly ascending
+// order, its first column and the number of columns up to its last one (0
+// for no products, INT_MAX when it does not fit an int), by one warp.
+__device__ __forceinline__ void row_span(const Operands &op, int64_t p0, int64_t p1, long long &sum, int &col0,
+                                         int &span) {
+    int mn = INT_MAX, mx = -1;
+    sum = 0;
+    for (int64_t p = p0 + (threadIdx.x & 31); p < p1; p += 32) {
+        const int k = __ldg(op.acol + p);
+        const int64_t q0 = ld_rpt(op.brpt, op.b64, k), q1 = ld_rpt(op.brpt, op.b64, k + 1);
+        sum += q1 - q0;
+        if (q1 > q0) {
+            mn = min(mn, __ldg(op.bcol + q0));
+            mx = max(mx, __ldg(op.bcol + q1 - 1));
+        }
+    }
+    sum = warp_sum_xor(sum, 32);
+    mn = __reduce_min_sync(0xffffffffu, mn);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    col0 = mn;
+    const long long s = mx >= mn ? static_cast<long long>(mx) - mn + 1 : 0;
+    span = s > INT_MAX ? INT_MAX : static_cast<int>(s);
+}
+
 // Ascending bitonic sort of the NR * 32 values one warp holds in registers,
 // element e = r * 32 + lane in x[r] (striped, so the sorted result stores
 // coalesced). Every loop has a compile-time trip count and unrolls fully, so
@@ -177,14 +205,12 @@ __global__ void __launch_bounds__(BLOCK, (T * 12 * (BLOCK / TPR) > 110 * 1024) ?
 num_hash_kernel(Operands op, BinWork w) {
     constexpr int RPB = BLOCK / TPR;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double *vals_all = reinterpret_cast<double *>(smem_raw);
-    int *keys_all = reinterpret_cast<int *>(vals_all + RPB * T);
     __shared__ long long red64[32];
     __shared__ int red32[33];
     __shared__ int full[RPB];   // one-phase: a probe found no free slot in this row's table
     const int g = threadIdx.x / TPR, lg = threadIdx.x % TPR;
-    int *tk = keys_all + g * T;
-    double *tv = vals_all + g * T;
+    double *tv = reinterpret_cast<double *>(smem_raw + static_cast<size_t>(g) * (T * 12));   // the row's table
+    int *tk = reinterpret_cast<int *>(tv + T);
     bool failed = false;
     if (lg == 0) full[g] = 0;
     const int64_t r = static_cast<int64_t>(blockIdx.x) * RPB + g;
@@ -222,11 +248,30 @@ num_hash_kernel(Operands op, BinWork w) {
             return;   // uniform over the warp; no block barrier follows
         }
     }
-    for (int s = lg; s < T; s += TPR) {
-        tk[s] = -1;
-        tv[s] = 0.0;
+    // A warp's row whose columns span at most kSpan columns is accumulated by
+    // column in the table's memory (B's rows strictly ascending): no probes, no
+    // condense and no sort.
+    constexpr bool kMaySpan = TPR == 32 && !MULTI;
+    constexpr int kSpan = (T * 12 / 8) / 32 * 32;
+    int S = TPR, col0 = 0, span = 0;
+    if (kMaySpan && w.distinct && w.lanes == 0) {
+        long long sum;
+        row_span(op, p0, p1, sum, col0, span);
+        S = pick_lanes_distinct(0, sum, p1 - p0, TPR);
+        if (span > kSpan) span = 0;
+    } else {
+        S = numeric_lanes<TPR>(op, w.lanes, p0, p1, lg, red64);
     }
-    const int S = numeric_lanes<TPR>(op, w.lanes, p0, p1, lg, red64);
+    const bool dense = kMaySpan && span > 0;   // uniform over the warp, and over the row group
+    if (dense) {
+        long long *acc = reinterpret_cast<long long *>(tv);
+        for (int s = lg; s < span; s += TPR) acc[s] = kNoEntry;
+    } else {
+        for (int s = lg; s < T; s += TPR) {
+            tk[s] = -1;
+            tv[s] = 0.0;
+        }
+    }
     group_sync<TPR>();
     if constexpr (TPR > 32) {
         // one row per block: flattened walk over B-row pieces
@@ -235,7 +280,7 @@ num_hash_kernel(Operands op, BinWork w) {
         block_row_walk<BLOCK, true>(op, p0, p1, S, sc, [&](int key, double a, double b) {
             if (!num_insert<T, MULTI>(tk, tv, key, a, b)) failed = true;
         });
-    } else if (!MULTI && w.distinct && S == TPR) {
+    } else if (!MULTI && w.distinct && (S == TPR || dense)) {
         // one B row per step, its columns distinct: values without atomics,
         // B's entries staged in shared memory by cp.async (after the tables:
         // kStage * TPR values, then as many columns, per row group)
@@ -245,9 +290,21 @@ num_hash_kernel(Operands op, BinWork w) {
                                                                       (sizeof(int) + sizeof(double)) * (size_t)RPB * T) +
                                           static_cast<size_t>(RPB) * kStage * TPR) +
                   static_cast<size_t>(g) * kStage * TPR;
-        group_row_walk_staged<TPR>(op, p0, p1, sc, sv, [&](int key, double a, double b) {
-            if (!num_insert_owned<T>(tk, tv, key, a, b)) failed = true;
-        });
+        if (dense)
+            group_row_walk_staged<TPR>(op, p0, p1, sc, sv, [&](int key, double a, double b) {
+                // inside, unless B's rows changed since their order was checked
+                const unsigned at = static_cast<unsigned>(key) - static_cast<unsigned>(col0);
+                if (at < static_cast<unsigned>(span)) {
+                    const double v = tv[at];
+                    tv[at] = fma(a, b, __double_as_longlong(v) == kNoEntry ? 0.0 : v);
+                } else {
+                    failed = true;
+                }
+            });
+        else
+            group_row_walk_staged<TPR>(op, p0, p1, sc, sv, [&](int key, double a, double b) {
+                if (!num_insert_owned<T>(tk, tv, key, a, b)) failed = true;
+            });
     } else {
         group_row_walk<TPR, true>(op, p0, p1, S, [&](int key, double a, double b) {
             if (!num_insert<T, MULTI>(tk, tv, key, a, b)) failed = true;
@@ -262,7 +319,11 @@ num_hash_kernel(Operands op, BinWork w) {
     // never lands past the chunk that was just read.
     int n = 0;
     int kmin = INT_MAX, kmax = -1;   // this thread's smallest and largest key
-    for (int c = 0; c < T; c += TPR) {
+    if (dense) {
+        for (int s = lg; s < span; s += TPR) n += reinterpret_cast<const long long *>(tv)[s] != kNoEntry;
+        if constexpr (TPR <= 32) n = warp_sum_xor(n, TPR);
+    }
+    for (int c = 0; c < T && !dense; c += TPR) {
         const int s = c + lg;
         int k = -1;
         double v = 0.0;
@@ -312,6 +373,37 @@ num_hash_kernel(Operands op, BinWork w) {
         if (P > T) {  // cannot happen within the kernel's capacity; never index past the table
             set_error(w.err, DERR_TABLE_FULL);
             P = 1;
+        }
+    }
+    if constexpr (kMaySpan) {
+        if (dense) {
+            // entries in column order: the ones before in their 32 columns by
+            // ballot, the ones before those by a running count
+            const int64_t m = n < n_expect ? n : n_expect;
+            int32_t *ocol = w.ccol + cbase;
+            double *oval = w.cval + cbase;
+            bool store = valid;
+            if (ONE_PHASE) {
+                ocol = w.tcol + w.tbase + r * w.tcap;
+                oval = w.tval + w.tbase + r * w.tcap;
+                const bool in_bounds = m <= w.tcap && w.tbase + r * w.tcap + m <= w.tlimit;
+                if (valid && !in_bounds && lg == 0) set_error(w.err, DERR_BOUNDS);
+                store &= in_bounds;
+            }
+            int64_t at = 0;
+            for (int s0 = 0; s0 < span; s0 += 32) {
+                const int s = s0 + lg;
+                const double v = s < span ? tv[s] : __longlong_as_double(kNoEntry);
+                const bool here = __double_as_longlong(v) != kNoEntry;
+                const unsigned bal = __ballot_sync(0xffffffffu, here);
+                const int64_t o = at + __popc(bal & ((1u << lg) - 1u));
+                if (here && store && o < m) {
+                    ocol[o] = col0 + s;
+                    oval[o] = v;
+                }
+                at += __popc(bal);
+            }
+            return;   // uniform over the warp; no block barrier follows
         }
     }
     if constexpr (TPR == 32 && T <= 1024) {
