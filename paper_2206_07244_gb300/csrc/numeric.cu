@@ -94,8 +94,97 @@ __device__ __forceinline__ int numeric_lanes(const Operands &op, int fixed, int6
 }
 
 // Accumulator of a column that no product has reached: a signalling NaN, which
-// no arithmetic result is.
-constexpr long long kNoEntry = 0x7ff0000000000001ll;
+// no arithmetic result is; the upper half tells it from every other value that
+// an accumulator holds.
+constexpr long long kNoEntry = 0x7ff0000100000000ll;
+__device__ __forceinline__ bool no_entry(double v) { return __double2hiint(v) == static_cast<int>(kNoEntry >> 32); }
+
+// Adds the products of the row [p0, p1) of A to acc[column - col0], by one
+// warp. A's entries go through shared memory 32 at a time (ent: their values
+// and B rows, len: lengths), and a lane loads its product of kU B rows before
+// using any; one B row at a time is added (distinct columns: no atomics), in
+// the order of A's entries. False when a column lies outside [0, span): B
+// changed since its order was checked. Bound by instruction issue, about 20
+// per B row of at most 32 entries, and the float64 pipe (16 cycles).
+struct __align__(16) SpanEntry {
+    double a;
+    long long q;
+};
+__device__ __forceinline__ bool span_walk(const Operands &op, int64_t p0, int64_t p1, int col0, int span, double *acc,
+                                          SpanEntry *ent, int *len) {
+    constexpr int kU = 4;
+    const int lane = threadIdx.x & 31;
+    bool inside = true;
+    auto add = [&](int c, double a, double b) {
+        const unsigned at = static_cast<unsigned>(c) - static_cast<unsigned>(col0);
+        if (at < static_cast<unsigned>(span)) {
+            const double v = acc[at];
+            acc[at] = fma(a, b, no_entry(v) ? 0.0 : v);
+        } else {
+            inside = false;
+        }
+    };
+    for (int64_t p = p0; p < p1; p += 32) {
+        const int cnt = static_cast<int>(p1 - p < 32 ? p1 - p : 32);
+        __syncwarp();   // readers of the entries before are done
+        int mine = 0;
+        if (lane < cnt) {
+            const int k = __ldg(op.acol + p + lane);
+            const int64_t q = ld_rpt(op.brpt, op.b64, k);
+            mine = static_cast<int>(ld_rpt(op.brpt, op.b64, k + 1) - q);
+            ent[lane] = SpanEntry{__ldg(op.aval + p + lane), q};
+        }
+        len[lane] = mine;   // 0 past the entries
+        const bool one_piece = __all_sync(0xffffffffu, mine <= 32);
+        __syncwarp();
+        if (one_piece) {
+            for (int e = 0; e < cnt; e += kU) {   // uniform over the warp
+                int c[kU];
+                double a[kU], b[kU];
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    c[u] = -1;
+                    a[u] = b[u] = 0.0;
+                    if (lane < len[(e + u) & 31] && e + u < cnt) {
+                        const SpanEntry x = ent[e + u];
+                        a[u] = x.a;
+                        c[u] = __ldg(op.bcol + x.q + lane);
+                        b[u] = __ldg(op.bval + x.q + lane);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    if (c[u] >= 0) add(c[u], a[u], b[u]);
+                    __syncwarp();
+                }
+            }
+        } else {
+            for (int e = 0; e < cnt; ++e) {
+                const int n = len[e];
+                const SpanEntry x = ent[e];
+                for (int o = lane; o < n; o += 32 * kU) {
+                    int c[kU];
+                    double b[kU];
+#pragma unroll
+                    for (int u = 0; u < kU; ++u) {
+                        c[u] = -1;
+                        b[u] = 0.0;
+                        if (o + 32 * u < n) {
+                            c[u] = __ldg(op.bcol + x.q + o + 32 * u);
+                            b[u] = __ldg(op.bval + x.q + o + 32 * u);
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < kU; ++u)
+                        if (c[u] >= 0) add(c[u], x.a, b[u]);
+                }
+                __syncwarp();
+            }
+        }
+    }
+    __syncwarp();
+    return inside;
+}
 
 // Products of the row [p0, p1) and, for rows of B in strictly ascending
 // order, its first column and the number of columns up to its last one (0
@@ -265,6 +354,7 @@ num_hash_kernel(Operands op, BinWork w) {
     const bool dense = kMaySpan && span > 0;   // uniform over the warp, and over the row group
     if (dense) {
         long long *acc = reinterpret_cast<long long *>(tv);
+#pragma unroll 4
         for (int s = lg; s < span; s += TPR) acc[s] = kNoEntry;
     } else {
         for (int s = lg; s < T; s += TPR) {
@@ -291,16 +381,7 @@ num_hash_kernel(Operands op, BinWork w) {
                                           static_cast<size_t>(RPB) * kStage * TPR) +
                   static_cast<size_t>(g) * kStage * TPR;
         if (dense)
-            group_row_walk_staged<TPR>(op, p0, p1, sc, sv, [&](int key, double a, double b) {
-                // inside, unless B's rows changed since their order was checked
-                const unsigned at = static_cast<unsigned>(key) - static_cast<unsigned>(col0);
-                if (at < static_cast<unsigned>(span)) {
-                    const double v = tv[at];
-                    tv[at] = fma(a, b, __double_as_longlong(v) == kNoEntry ? 0.0 : v);
-                } else {
-                    failed = true;
-                }
-            });
+            failed = !span_walk(op, p0, p1, col0, span, tv, reinterpret_cast<SpanEntry *>(sv), sc);
         else
             group_row_walk_staged<TPR>(op, p0, p1, sc, sv, [&](int key, double a, double b) {
                 if (!num_insert_owned<T>(tk, tv, key, a, b)) failed = true;
@@ -320,8 +401,12 @@ num_hash_kernel(Operands op, BinWork w) {
     int n = 0;
     int kmin = INT_MAX, kmax = -1;   // this thread's smallest and largest key
     if (dense) {
-        for (int s = lg; s < span; s += TPR) n += reinterpret_cast<const long long *>(tv)[s] != kNoEntry;
-        if constexpr (TPR <= 32) n = warp_sum_xor(n, TPR);
+        if (ONE_PHASE) {
+            for (int s = lg; s < span; s += TPR) n += !no_entry(tv[s]);
+            if constexpr (TPR <= 32) n = warp_sum_xor(n, TPR);
+        } else {
+            n = static_cast<int>(n_expect < span ? n_expect : span);   // counted as it is stored
+        }
     }
     for (int c = 0; c < T && !dense; c += TPR) {
         const int s = c + lg;
@@ -379,30 +464,31 @@ num_hash_kernel(Operands op, BinWork w) {
         if (dense) {
             // entries in column order: the ones before in their 32 columns by
             // ballot, the ones before those by a running count
-            const int64_t m = n < n_expect ? n : n_expect;
             int32_t *ocol = w.ccol + cbase;
             double *oval = w.cval + cbase;
-            bool store = valid;
+            int m = valid ? n : 0;   // entries to store
             if (ONE_PHASE) {
                 ocol = w.tcol + w.tbase + r * w.tcap;
                 oval = w.tval + w.tbase + r * w.tcap;
-                const bool in_bounds = m <= w.tcap && w.tbase + r * w.tcap + m <= w.tlimit;
-                if (valid && !in_bounds && lg == 0) set_error(w.err, DERR_BOUNDS);
-                store &= in_bounds;
+                if (m > w.tcap || w.tbase + r * w.tcap + m > w.tlimit) {
+                    if (lg == 0) set_error(w.err, DERR_BOUNDS);
+                    m = 0;
+                }
             }
-            int64_t at = 0;
-            for (int s0 = 0; s0 < span; s0 += 32) {
-                const int s = s0 + lg;
+            int at = 0;
+#pragma unroll 4
+            for (int s = lg; s < span + lg; s += 32) {   // uniform over the warp
                 const double v = s < span ? tv[s] : __longlong_as_double(kNoEntry);
-                const bool here = __double_as_longlong(v) != kNoEntry;
+                const bool here = !no_entry(v);
                 const unsigned bal = __ballot_sync(0xffffffffu, here);
-                const int64_t o = at + __popc(bal & ((1u << lg) - 1u));
-                if (here && store && o < m) {
+                const int o = at + __popc(bal & ((1u << lg) - 1u));
+                if (here && o < m) {
                     ocol[o] = col0 + s;
                     oval[o] = v;
                 }
                 at += __popc(bal);
             }
+            if (!ONE_PHASE && valid && lg == 0 && at != n_expect) set_error(w.err, DERR_COUNT_MISMATCH);
             return;   // uniform over the warp; no block barrier follows
         }
     }
