@@ -596,7 +596,7 @@ int run_bins(spgemm_handle *h, int phase, const Operands &op, const long long *s
         w.lanes = phase ? h->cfg.num_lanes_per_brow : h->cfg.lanes_per_brow;
         w.unroll = h->cfg.bitmap_unroll;
         w.multi = h->cfg.hash_access;
-        w.distinct = phase == 1 && h->b_distinct;
+        w.distinct = h->b_distinct;
         w.clk = phase == 1 && h->phase_clk ? h->d_clk : nullptr;
         w.err = d_err(h);
         const KernelDesc &d = phase ? num_kernel(kid[j]) : sym_kernel(kid[j]);
@@ -1343,6 +1343,7 @@ int spgemm_symbolic(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_i
         return fail(SPGEMM_ERR_CUDA);
     time_end(h, kSlotSymPass1, h->stream);
     if ((rc = read_counters(h))) return fail(rc);
+    h->b_distinct = (h->h_cnt[1].flags & 3ull) == 0;   // B's order, from the setup scan
     long long ssize[kMaxBins] = {}, soff[kMaxBins] = {};
     const bool sid = plan_bins(h->h_cnt[0], rs.nb, ssize, soff, rep.words != nullptr);
     // no repeating rows: the numeric phase need not look for them

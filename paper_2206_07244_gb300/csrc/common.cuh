@@ -619,6 +619,36 @@ __device__ __forceinline__ void group_row_walk(const Operands &op, int64_t p0, i
     }
 }
 
+// Products of the row [p0, p1) and, for rows of B in ascending
+// order, its first column and the number of columns up to its last one (0
+// for no products, INT_MAX when it does not fit an int), by one warp; first /
+// len: the B row of the lane's first entry of A.
+__device__ __forceinline__ void row_span(const Operands &op, int64_t p0, int64_t p1, long long &sum, int &col0,
+                                         int &span, long long &first, int &len) {
+    int mn = INT_MAX, mx = -1;
+    sum = first = len = 0;
+    const int64_t mine = p0 + (threadIdx.x & 31);
+    for (int64_t p = mine; p < p1; p += 32) {
+        const int k = __ldg(op.acol + p);
+        const int64_t q0 = ld_rpt(op.brpt, op.b64, k), q1 = ld_rpt(op.brpt, op.b64, k + 1);
+        if (p == mine) {
+            first = q0;
+            len = static_cast<int>(q1 - q0);
+        }
+        sum += q1 - q0;
+        if (q1 > q0) {
+            mn = min(mn, __ldg(op.bcol + q0));
+            mx = max(mx, __ldg(op.bcol + q1 - 1));
+        }
+    }
+    sum = warp_sum_xor(sum, 32);
+    mn = __reduce_min_sync(0xffffffffu, mn);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    col0 = mn;
+    const long long s = mx >= mn ? static_cast<long long>(mx) - mn + 1 : 0;
+    span = s > INT_MAX ? INT_MAX : static_cast<int>(s);
+}
+
 // --- rows of at most 8 products -----------------------------------------------
 // A row group of 8 lanes holds such a row in registers, one product per lane
 // in the order of A's entries, when the row has at most 8 A entries. Equal

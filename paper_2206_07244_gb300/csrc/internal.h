@@ -46,8 +46,9 @@ struct BinWork {
     int lanes;            // threads per B row, 0 = per-row automatic
     int unroll;           // bitmap kernels: products in flight per lane (4 or 8; 0 = 4)
     int multi;            // plain hash kernels: read a slot before its compare-and-swap
-    int distinct;         // every row of B has distinct columns (checked): warp-row numeric
-                          // hash kernels may update values without atomics
+    int distinct;         // every row of B has strictly ascending columns (checked): warp-row
+                          // kernels may bound a row's columns by the ends of its B rows, and
+                          // update values without atomics
     int *err;             // device error word
     // numeric bitmap kernel, pass 2 by column windows (B rows sorted)
     const int32_t *bs;    // run boundaries of B rows at the sub-ranges (G + 1 per row), or nullptr

@@ -102,17 +102,21 @@ __device__ __forceinline__ bool no_entry(double v) { return __double2hiint(v) ==
 // Adds the products of the row [p0, p1) of A to acc[column - col0], by one
 // warp. A's entries go through shared memory 32 at a time (ent: their values
 // and B rows, len: lengths), and a lane loads its product of kU B rows before
-// using any; one B row at a time is added (distinct columns: no atomics), in
+// using any (8 where the tables leave the registers for it); one B row at a time is added (distinct columns: no atomics), in
 // the order of A's entries. False when a column lies outside [0, span): B
-// changed since its order was checked. Bound by instruction issue, about 20
-// per B row of at most 32 entries, and the float64 pipe (16 cycles).
+// changed since its order was checked. Bound by latency: the tables leave 16
+// to 40 warps on an SM, each waiting for its own loads and shared-memory
+// updates (49% of issue slots, 35% of the float64 pipe). Block-diagonal n =
+// 2^20, blocks of 1024 columns: numeric 9.49 ms by the table, 4.39 ms this way.
 struct __align__(16) SpanEntry {
     double a;
     long long q;
 };
-__device__ __forceinline__ bool span_walk(const Operands &op, int64_t p0, int64_t p1, int col0, int span, double *acc,
-                                          SpanEntry *ent, int *len) {
-    constexpr int kU = 4;
+// PRE: q0 / len0 hold the B row of A's entry p0 + lane (from row_span; the
+// 256-slot kernel has no registers for them).
+template <int kU, bool PRE>
+__device__ __forceinline__ bool span_walk(const Operands &op, int64_t p0, int64_t p1, long long q0, int len0, int col0,
+                                          int span, double *acc, SpanEntry *ent, int *len) {
     const int lane = threadIdx.x & 31;
     bool inside = true;
     auto add = [&](int c, double a, double b) {
@@ -129,9 +133,13 @@ __device__ __forceinline__ bool span_walk(const Operands &op, int64_t p0, int64_
         __syncwarp();   // readers of the entries before are done
         int mine = 0;
         if (lane < cnt) {
-            const int k = __ldg(op.acol + p + lane);
-            const int64_t q = ld_rpt(op.brpt, op.b64, k);
-            mine = static_cast<int>(ld_rpt(op.brpt, op.b64, k + 1) - q);
+            long long q = q0;
+            mine = len0;
+            if (!PRE || p > p0) {
+                const int k = __ldg(op.acol + p + lane);
+                q = ld_rpt(op.brpt, op.b64, k);
+                mine = static_cast<int>(ld_rpt(op.brpt, op.b64, k + 1) - q);
+            }
             ent[lane] = SpanEntry{__ldg(op.aval + p + lane), q};
         }
         len[lane] = mine;   // 0 past the entries
@@ -184,30 +192,6 @@ __device__ __forceinline__ bool span_walk(const Operands &op, int64_t p0, int64_
     }
     __syncwarp();
     return inside;
-}
-
-// Products of the row [p0, p1) and, for rows of B in strictly ascending
-// order, its first column and the number of columns up to its last one (0
-// for no products, INT_MAX when it does not fit an int), by one warp.
-__device__ __forceinline__ void row_span(const Operands &op, int64_t p0, int64_t p1, long long &sum, int &col0,
-                                         int &span) {
-    int mn = INT_MAX, mx = -1;
-    sum = 0;
-    for (int64_t p = p0 + (threadIdx.x & 31); p < p1; p += 32) {
-        const int k = __ldg(op.acol + p);
-        const int64_t q0 = ld_rpt(op.brpt, op.b64, k), q1 = ld_rpt(op.brpt, op.b64, k + 1);
-        sum += q1 - q0;
-        if (q1 > q0) {
-            mn = min(mn, __ldg(op.bcol + q0));
-            mx = max(mx, __ldg(op.bcol + q1 - 1));
-        }
-    }
-    sum = warp_sum_xor(sum, 32);
-    mn = __reduce_min_sync(0xffffffffu, mn);
-    mx = __reduce_max_sync(0xffffffffu, mx);
-    col0 = mn;
-    const long long s = mx >= mn ? static_cast<long long>(mx) - mn + 1 : 0;
-    span = s > INT_MAX ? INT_MAX : static_cast<int>(s);
 }
 
 // Ascending bitonic sort of the NR * 32 values one warp holds in registers,
@@ -342,10 +326,11 @@ num_hash_kernel(Operands op, BinWork w) {
     // condense and no sort.
     constexpr bool kMaySpan = TPR == 32 && !MULTI;
     constexpr int kSpan = (T * 12 / 8) / 32 * 32;
-    int S = TPR, col0 = 0, span = 0;
+    int S = TPR, col0 = 0, span = 0, len0 = 0;
+    long long q0 = 0;
     if (kMaySpan && w.distinct && w.lanes == 0) {
         long long sum;
-        row_span(op, p0, p1, sum, col0, span);
+        row_span(op, p0, p1, sum, col0, span, q0, len0);
         S = pick_lanes_distinct(0, sum, p1 - p0, TPR);
         if (span > kSpan) span = 0;
     } else {
@@ -381,7 +366,8 @@ num_hash_kernel(Operands op, BinWork w) {
                                           static_cast<size_t>(RPB) * kStage * TPR) +
                   static_cast<size_t>(g) * kStage * TPR;
         if (dense)
-            failed = !span_walk(op, p0, p1, col0, span, tv, reinterpret_cast<SpanEntry *>(sv), sc);
+            failed = !span_walk<(T >= 1024 ? 8 : 4), (T >= 512)>(op, p0, p1, q0, len0, col0, span, tv,
+                                                   reinterpret_cast<SpanEntry *>(sv), sc);
         else
             group_row_walk_staged<TPR>(op, p0, p1, sc, sv, [&](int key, double a, double b) {
                 if (!num_insert_owned<T>(tk, tv, key, a, b)) failed = true;

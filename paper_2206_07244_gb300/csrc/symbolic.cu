@@ -57,9 +57,10 @@ __device__ __forceinline__ int sym_insert(int *tab, int key, int *err) {
 
 // Minimum resident blocks: enough for 2048 threads per SM (<= 32 registers
 // per thread, Sec. 5.6) unless the table is so large that one block fills
-// the SM's shared memory anyway.
+// the SM's shared memory anyway; warp-per-row kernels 1536 (40 registers: the
+// column bitmap's walk spills at 32, block-diagonal n = 2^20 1.26 -> 1.16 ms).
 template <int TPR, int BLOCK, int T, bool MULTI = false>
-__global__ void __launch_bounds__(BLOCK, (T * 4 * (BLOCK / TPR) > 110 * 1024) ? 1 : 2048 / BLOCK)
+__global__ void __launch_bounds__(BLOCK, (T * 4 * (BLOCK / TPR) > 110 * 1024) ? 1 : (TPR == 32 && !MULTI ? 1536 : 2048) / BLOCK)
 sym_hash_kernel(Operands op, BinWork w) {
     constexpr int RPB = BLOCK / TPR;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -81,6 +82,42 @@ sym_hash_kernel(Operands op, BinWork w) {
                              valid ? ld_rpt(op.arpt, op.a64, ar + 1) : 0, t)) {
             if (valid && lg == 0) w.crpt[row] = __popc(t.heads);
             return;   // uniform over the warp; no block barrier follows
+        }
+    }
+    if constexpr (TPR == 32 && !MULTI) {
+        // A row whose columns span at most 32 T columns (B's rows ascending):
+        // a bit per column in the table's memory, set without a probe and
+        // counted at the end (block-diagonal n = 2^20, blocks of 1024 columns:
+        // 1.48 -> 1.16 ms).
+        if (w.distinct) {
+            int64_t p0 = 0, p1 = 0;
+            if (valid) {
+                p0 = ld_rpt(op.arpt, op.a64, op.row0 + row);
+                p1 = ld_rpt(op.arpt, op.a64, op.row0 + row + 1);
+            }
+            long long sum, first;
+            int col0, span, len;
+            row_span(op, p0, p1, sum, col0, span, first, len);
+            if (span <= 32 * T) {   // uniform over the warp
+                unsigned *bits = reinterpret_cast<unsigned *>(tab);
+                const int words = (span + 31) >> 5;
+                for (int i = lg; i < words; i += 32) bits[i] = 0u;
+                __syncwarp();
+                const int S = pick_lanes(w.lanes, sum, p1 - p0, TPR);
+                bool outside = false;
+                group_row_walk<TPR, false>(op, p0, p1, S, [&](int key, double, double) {
+                    const unsigned at = static_cast<unsigned>(key) - static_cast<unsigned>(col0);
+                    if (at < static_cast<unsigned>(span)) atomicOr(bits + (at >> 5), 1u << (at & 31));
+                    else outside = true;
+                });
+                if (outside) set_error(w.err, DERR_BOUNDS);
+                __syncwarp();
+                int n = 0;
+                for (int i = lg; i < words; i += 32) n += __popc(bits[i]);
+                n = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned>(n)));
+                if (valid && lg == 0) w.crpt[row] = n;
+                return;   // uniform over the warp; no block barrier follows
+            }
         }
     }
     for (int s = lg; s < T; s += TPR) tab[s] = -1;

@@ -1,5 +1,6 @@
 """Rows whose columns span few columns, which the warp-per-row numeric kernels
-accumulate by column: at the widest span of each table, one column past it,
+accumulate by column and the symbolic ones count by a bitmap: at the widest
+span of each table, one column past it,
 and with sums of zero, infinities and NaN (which stay entries of C), against
 the CPU oracle."""
 
@@ -51,6 +52,22 @@ def test_widest_span(slots, size, extra, first):
         C = h.multiply(dA, dB)
         h.status()
         assert sum(h.stats()["num_bins"]) == A.rows
+    for g, w in zip(C.numpy(), oracle.spgemm(A, B)[:3]):
+        assert np.array_equal(g, w)
+
+
+@pytest.mark.parametrize("extra", [0, 1])
+@pytest.mark.parametrize("slots, size", [(512, 150), (1024, 300)])   # about 2.5 size products a row
+def test_widest_span_of_the_symbolic_bitmap(slots, size, extra):
+    A, B = product(size, slots * 32 + extra, 11, 4)
+    table = ops.kernel_table(0)
+    kernel = next(k for k, t in enumerate(table) if t[0] == 32 and t[2] == slots)
+    cfg = ops.default_config()
+    cfg["sym_kernel"], cfg["sym_range"] = [kernel, len(table) - 1], [table[kernel][3], -1]
+    dA, dB = (ops.CSR.from_arrays(m.rows, m.cols, m.rpt, m.col, m.val) for m in (A, B))
+    with ops.Handle(cfg) as h:
+        C = h.multiply(dA, dB)
+        h.status()
     for g, w in zip(C.numpy(), oracle.spgemm(A, B)[:3]):
         assert np.array_equal(g, w)
 
