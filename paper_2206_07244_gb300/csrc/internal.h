@@ -343,7 +343,8 @@ cudaError_t win_prepare(int smem_optin);
 cudaError_t launch_win_count(const WinPlan &plan, const int64_t *crpt, int64_t mw, const uint16_t *cells,
                              const int32_t *cslot, unsigned long long *total, unsigned long long *total_col,
                              int *err, cudaStream_t s);
-// Cell index of the rows of B with at least `min_len` entries (slots up to cap).
+// Cell index of the rows of B with at least `min_len` entries (slots up to
+// cap). nslot: two counters, 0 before.
 cudaError_t launch_win_bindex(const Operands &op, int64_t brows, const WinPlan &plan, long long min_len,
                               int32_t *bslot, int32_t *bidx, long long cap, unsigned long long *nslot,
                               cudaStream_t s);

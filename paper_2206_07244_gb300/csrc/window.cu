@@ -256,7 +256,34 @@ cudaError_t launch_win_plan(const WinPlan &plan, const BinWork &w, const uint16_
 // first entry with column >= c * 2^cs (c = 0..ncells): entry e writes the
 // cells after the previous entry's cell up to its own; the last entry writes
 // the rest. Shorter rows (and rows past the cap) get slot -1 and are
-// searched.
+// searched. A thread loads four entries before using any. Rows of more than
+// kBindexLong entries are counted in nslot[1] and left to
+// win_bindex_long_kernel, a block per row: a power-law row of 10^5 entries on
+// one warp was the kernel's time (R-MAT n = 2^21, degree 32: 1.66 ms, now
+// 0.35 with both kernels).
+constexpr long long kBindexLong = 1024;
+
+__device__ __forceinline__ void fill_bindex(const Operands &op, int cs, int ncells, long long q0, long long len,
+                                            int32_t *x, int first, int step) {
+    constexpr int kU = 4;
+    for (long long e0 = first; e0 < len; e0 += static_cast<long long>(step) * kU) {
+        int cc[kU], pc[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const long long e = e0 + static_cast<long long>(u) * step;
+            cc[u] = e < len ? min(__ldg(op.bcol + q0 + e) >> cs, ncells) : -1;
+            pc[u] = e > 0 && e < len ? min(__ldg(op.bcol + q0 + e - 1) >> cs, ncells) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const long long e = e0 + static_cast<long long>(u) * step;
+            for (int c = pc[u] + 1; c <= cc[u]; ++c) x[c] = static_cast<int32_t>(e);
+            if (e + 1 == len)
+                for (int c = cc[u] + 1; c <= ncells; ++c) x[c] = static_cast<int32_t>(len);
+        }
+    }
+}
+
 __global__ void __launch_bounds__(256)
 win_bindex_kernel(Operands op, int64_t brows, int cs, int ncells, long long min_len, int32_t *bslot,
                   int32_t *bidx, long long cap, unsigned long long *nslot) {
@@ -269,17 +296,36 @@ win_bindex_kernel(Operands op, int64_t brows, int cs, int ncells, long long min_
     if (len >= min_len && lane == 0) {
         slot = static_cast<long long>(atomicAdd(nslot, 1ull));
         if (slot >= cap) slot = -1;
+        if (slot >= 0 && len > kBindexLong) atomicAdd(nslot + 1, 1ull);
     }
     slot = __shfl_sync(0xffffffffu, slot, 0);
     if (lane == 0) bslot[k] = static_cast<int32_t>(slot);
-    if (slot < 0) return;
-    int32_t *x = bidx + slot * (ncells + 1);
-    for (int64_t e = lane; e < len; e += 32) {
-        const int cc = min(__ldg(op.bcol + q0 + e) >> cs, ncells);
-        const int pc = e == 0 ? -1 : min(__ldg(op.bcol + q0 + e - 1) >> cs, ncells);
-        for (int c = pc + 1; c <= cc; ++c) x[c] = static_cast<int32_t>(e);
-        if (e + 1 == len)
-            for (int c = cc + 1; c <= ncells; ++c) x[c] = static_cast<int32_t>(len);
+    if (slot >= 0 && len <= kBindexLong) fill_bindex(op, cs, ncells, q0, len, bidx + slot * (ncells + 1), lane, 32);
+}
+
+// The long rows: block b looks at rows b, b + blocks, ... In power-law inputs
+// the longest rows are neighbours, and in R-MAT their ids differ by powers of
+// two as well, so a prime number of blocks spreads them (4,096 blocks: 1.71 ms
+// for the rows that block 0 got).
+__global__ void __launch_bounds__(256)
+win_bindex_long_kernel(Operands op, int64_t brows, int cs, int ncells, const int32_t *bslot, int32_t *bidx,
+                       const unsigned long long *nslot) {
+    if (__ldcg(nslot + 1) == 0) return;   // uniform over the grid
+    __shared__ long long s_row[256];
+    __shared__ int s_n;
+    for (int64_t base = blockIdx.x; base < brows; base += static_cast<int64_t>(gridDim.x) * 256) {
+        __syncthreads();   // readers of the list before are done
+        if (threadIdx.x == 0) s_n = 0;
+        __syncthreads();
+        const int64_t k = base + static_cast<int64_t>(threadIdx.x) * gridDim.x;
+        if (k < brows && bslot[k] >= 0 && ld_rpt(op.brpt, op.b64, k + 1) - ld_rpt(op.brpt, op.b64, k) > kBindexLong)
+            s_row[atomicAdd(&s_n, 1)] = k;
+        __syncthreads();
+        for (int j = 0; j < s_n; ++j) {
+            const int64_t r = s_row[j], q0 = ld_rpt(op.brpt, op.b64, r);
+            fill_bindex(op, cs, ncells, q0, ld_rpt(op.brpt, op.b64, r + 1) - q0,
+                        bidx + static_cast<long long>(bslot[r]) * (ncells + 1), threadIdx.x, 256);
+        }
     }
 }
 
@@ -290,6 +336,11 @@ cudaError_t launch_win_bindex(const Operands &op, int64_t brows, const WinPlan &
     const int64_t threads = brows * 32;
     win_bindex_kernel<<<static_cast<unsigned>((threads + 255) / 256), 256, 0, s>>>(
         op, brows, plan.cs, plan.ncells, min_len, bslot, bidx, cap, nslot);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const int64_t grid = (brows + 255) / 256 < 4093 ? (brows + 255) / 256 : 4093;   // a prime: see above
+    win_bindex_long_kernel<<<static_cast<unsigned>(grid), 256, 0, s>>>(op, brows, plan.cs, plan.ncells, bslot, bidx,
+                                                                      nslot);
     return cudaGetLastError();
 }
 
