@@ -945,6 +945,7 @@ int symbolic_learned(spgemm_handle *h, const Operands &op, const spgemm_csr_in *
         all.r[0] = -1;
         if (repeats) {
             rep.fill = crpt;
+            rep.nprod = L.lsizes;   // repeating rows: n_prod (binned by it, into no bin)
             rep.max_nnz = kRepMaxNnz;
         }
         time_begin(h, kSlotNumPass1, s);
@@ -981,9 +982,10 @@ int symbolic_learned(spgemm_handle *h, const Operands &op, const spgemm_csr_in *
     };
     // Without rows of the bitmap bin the exact list is expected to stay
     // empty, and the rows are counted before its length is known; a
-    // misprediction then costs a second count. (The sizes that the count
-    // fills in for repeating rows of a mispredicted row are its n_prod, which
-    // they held before.)
+    // misprediction then costs a second count. (The first count writes sizes
+    // over the repeating rows' n_prod in C.rpt, for rows of a mispredicted row
+    // its n_prod, the others' n_nz: the classes come from L.lsizes both times,
+    // and the second count writes every size again.)
     if (cnt_last == 0) {
         if ((rc = count_rows())) return rc;
         h->xcount = static_cast<int64_t>(*h_x);

@@ -165,9 +165,12 @@ struct RepGate {
 // What a binning pass does with repeating rows: it leaves them out of the
 // bins when their size is at most max_nnz, and with `fill` writes the size of
 // the row they repeat over their own first (words nullptr: no such rows).
+// nprod, read with `fill`: n_prod of the repeating rows, which their class
+// depends on; nullptr: the sizes hold it (no pass has filled them in yet).
 struct RepArgs {
     const RepWord *words = nullptr;
     int64_t *fill = nullptr;
+    const int64_t *nprod = nullptr;
     long long max_nnz = 0;
 };
 

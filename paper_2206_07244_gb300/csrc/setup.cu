@@ -318,7 +318,7 @@ bin_pass1_kernel(const int64_t *sizes, int64_t n, Ranges rg, Operands op, Counte
             int c = -1;
             if ((rw.fol >> (i & 31)) & 1u) {
                 if (rep.fill) {
-                    const long long np = static_cast<long long>(v[it]);
+                    const long long np = rep.nprod ? rep.nprod[i] : static_cast<long long>(v[it]);
                     v[it] = static_cast<unsigned long long>(sizes[rep_own(rw, i)]);
                     rep.fill[i] = static_cast<int64_t>(v[it]);
                     if (static_cast<long long>(v[it]) <= rep.max_nnz) c = rep_class(np, static_cast<long long>(v[it]));

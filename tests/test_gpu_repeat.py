@@ -189,3 +189,49 @@ def test_learned_sizing(name, trained):
             same(C, want)
         st = h.learned_stats()
         assert st["one_phase_rows"] + st["mispredicted_rows"] + st["exact_rows"] == A.rows
+
+
+def scatter(m, every, seed):
+    """Every `every`-th row references columns far apart, as many as before."""
+    rng = np.random.default_rng(seed)
+    lists = [m.col[m.rpt[i]:m.rpt[i + 1]] for i in range(m.rows)]
+    for i in range(every // 2, m.rows, every):
+        lists[i] = np.sort(rng.choice(m.cols, lists[i].size, replace=False))
+    return csr(m.rows, m.cols, lists, seed)
+
+
+# Rows of 257 to 1024 products and at most 64 entries, the second class by
+# their products and the first by their entries; a scattered row has as many
+# products as its neighbours and several times their entries.
+MIXED = {
+    "band 17": lambda: offsets(40000, range(-8, 9), 1),
+    "band 21": lambda: offsets(40000, range(-10, 11), 1),
+    "band 31": lambda: offsets(40000, range(-15, 16), 1),
+    "six unknowns a point": lambda: expand(offsets(40000 // 6, [-1, 0, 1], 1), 6, 2),
+    "ten unknowns a point": lambda: expand(offsets(4000, [-1, 0, 1], 1), 10, 2),
+    "blocks of 24": lambda: expand(offsets(40000 // 24, [0], 1), 24, 2),
+}
+
+
+@pytest.mark.parametrize("every", [10001, 39999])   # a handful of scattered rows, and one
+@pytest.mark.parametrize("name", MIXED)
+def test_learned_sizing_with_some_rows_mispredicted(name, every):
+    from paper_2206_07244_gb300 import learned
+    B = MIXED[name]()
+    A = scatter(B, every, 4)
+    dA, dB = dev(A), dev(B)
+    want = oracle.spgemm(A, B)[:3]
+    # predictions of the rows' own size, whatever the network says of them:
+    # the output bias alone, log1p of the entries of an unscattered row
+    theta = np.zeros_like(np.load(learned.WEIGHTS))
+    theta[-1] = np.log1p(np.median(np.diff(want[0])))
+    for weights in (np.load(learned.WEIGHTS), theta):
+        with ops.Handle() as h:
+            h.set_predictor(weights, 0.0)
+            h.set_mode("learned")
+            C = h.multiply(dA, dB)
+            st = h.learned_stats()
+            h.status()
+            same(C, want)
+            if weights is theta:
+                assert 0 < st["mispredicted_rows"] < A.rows // 2
