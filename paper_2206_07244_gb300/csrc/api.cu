@@ -574,6 +574,36 @@ Operands make_operands(const spgemm_csr_in *A, const spgemm_csr_in *B, int64_t r
     return op;
 }
 
+// Side streams with work of the current call. The handle's stream waits for
+// them on every way out, also when a launch in between fails: what they read
+// and write is freed, or handed back, on the handle's stream.
+struct SideWork {
+    spgemm_handle *h;
+    unsigned busy = 0;   // bit i: side stream i
+    explicit SideWork(spgemm_handle *handle) : h(handle) {}
+    SideWork(const SideWork &) = delete;
+    ~SideWork() { join(); }
+    // The stream that starts after ev_fork (recorded on the handle's stream).
+    cudaError_t fork(int i, cudaStream_t *s) {
+        *s = h->serial ? h->stream : h->side[i];
+        if (h->serial || ((busy >> i) & 1u)) return cudaSuccess;
+        const cudaError_t e = cudaStreamWaitEvent(*s, h->ev_fork, 0);
+        if (e == cudaSuccess) busy |= 1u << i;
+        return e;
+    }
+    cudaError_t join() {
+        cudaError_t first = cudaSuccess;
+        for (int i = 0; i < kSide; ++i) {
+            if (!((busy >> i) & 1u)) continue;
+            cudaError_t e = cudaEventRecord(h->ev_side[i], h->side[i]);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, h->ev_side[i], 0);
+            if (first == cudaSuccess) first = e;
+        }
+        busy = 0;
+        return first;
+    }
+};
+
 // Launch the kernels of one phase, one per non-empty bin, largest rows first,
 // spread over the side streams. runs: plan of a windowed pass 2 for the
 // numeric bitmap kernel (nullptr or runs->lists == 0: whole-row pass 2).
@@ -583,11 +613,12 @@ int run_bins(spgemm_handle *h, int phase, const Operands &op, const long long *s
     const int nb = phase ? h->cfg.num_nbins : h->cfg.sym_nbins;
     const int32_t *kid = phase ? h->cfg.num_kernel : h->cfg.sym_kernel;
     CK(cudaEventRecord(h->ev_fork, h->stream));
+    SideWork side(h);
     int used = 0;
     for (int j = nb - 1; j >= 0; --j) {
         if (size[j] <= 0) continue;
-        cudaStream_t s = h->serial ? h->stream : h->side[used % kSide];
-        if (!h->serial && used < kSide) CK(cudaStreamWaitEvent(s, h->ev_fork, 0));
+        cudaStream_t s;
+        CK(side.fork(used % kSide, &s));
         BinWork w{};
         w.bins = identity ? nullptr : d_bins(h);
         w.off = identity ? 0 : offset[j];
@@ -678,10 +709,7 @@ int run_bins(spgemm_handle *h, int phase, const Operands &op, const long long *s
         time_end(h, slot, s);
         ++used;
     }
-    for (int i = 0; !h->serial && i < std::min(used, kSide); ++i) {
-        CK(cudaEventRecord(h->ev_side[i], h->side[i]));
-        CK(cudaStreamWaitEvent(h->stream, h->ev_side[i], 0));
-    }
+    CK(side.join());
     return SPGEMM_OK;
 }
 
@@ -805,29 +833,12 @@ int symbolic_learned(spgemm_handle *h, const Operands &op, const spgemm_csr_in *
     bool repeats = false;
     // B's column order is checked on a side stream, next to the pattern
     // scans: nothing before the counters are read needs it (27-point stencil
-    // 128^3: 0.1 ms on its own). The handle's stream waits for it on every
-    // way out.
-    struct Aside {
-        cudaStream_t s = nullptr;
-        cudaEvent_t done = nullptr;
-        cudaError_t join() {
-            cudaEvent_t e = done;
-            done = nullptr;
-            return e ? cudaStreamWaitEvent(s, e, 0) : cudaSuccess;
-        }
-        ~Aside() { join(); }
-    } order;
-    cudaStream_t os = h->serial ? s : h->side[1];
-    if (!h->serial) {
-        CK(cudaEventRecord(h->ev_fork, s));
-        CK(cudaStreamWaitEvent(os, h->ev_fork, 0));
-    }
+    // 128^3: 0.1 ms on its own).
+    SideWork side(h);
+    cudaStream_t os;
+    CK(cudaEventRecord(h->ev_fork, s));
+    CK(side.fork(1, &os));
     CK(launch_setup(op, 0, nullptr, B->rows, B->nnz, d_counters(h, 1), h->sm_count * 8, os));
-    if (!h->serial) {
-        CK(cudaEventRecord(h->ev_side[1], os));
-        order.s = s;
-        order.done = h->ev_side[1];
-    }
     time_begin(h, kSlotPatterns, s);
     if ((rc = scan_patterns(h, op, A, B, &acode, &gate, &repeats))) return rc;
     RepWord *found_words = repeats ? h->rwords + (mw + 31) / 32 : nullptr;
@@ -865,7 +876,7 @@ int symbolic_learned(spgemm_handle *h, const Operands &op, const spgemm_csr_in *
         }
         CK(launch_bin_pass1(L.lsizes, mw, rn, op, d_counters(h, 0), nullptr, s, rep));
         time_end(h, kSlotMlp, s);
-        CK(order.join());
+        CK(side.join());
         if ((rc = read_counters(h))) return rc;
         // distinct columns let the warp-row one-phase kernels update values without atomics
         h->b_distinct = (h->h_cnt[1].flags & 3ull) == 0;
@@ -907,8 +918,8 @@ int symbolic_learned(spgemm_handle *h, const Operands &op, const spgemm_csr_in *
     int used = 0;
     for (int j = last - 1; j >= 0; --j) {
         if (h->lsize[j] <= 0) continue;
-        cudaStream_t ss = h->serial ? s : h->side[used % kSide];
-        if (!h->serial && used < kSide) CK(cudaStreamWaitEvent(ss, h->ev_fork, 0));
+        cudaStream_t ss;
+        CK(side.fork(used % kSide, &ss));
         BinWork w{};
         w.bins = h->lid ? nullptr : d_bins(h);
         w.off = h->lid ? 0 : h->loff[j];
@@ -931,10 +942,7 @@ int symbolic_learned(spgemm_handle *h, const Operands &op, const spgemm_csr_in *
         time_end(h, slot, ss);
         ++used;
     }
-    for (int i = 0; !h->serial && i < std::min(used, kSide); ++i) {
-        CK(cudaEventRecord(h->ev_side[i], h->side[i]));
-        CK(cudaStreamWaitEvent(s, h->ev_side[i], 0));
-    }
+    CK(side.join());
     unsigned long long *h_fb = reinterpret_cast<unsigned long long *>(
         reinterpret_cast<unsigned char *>(h->h_cnt) + 2 * sizeof(Counters) + 64);
     // total n_nz and the scan's tile sums; the load feedback and the length
@@ -1083,13 +1091,12 @@ int numeric_learned(spgemm_handle *h, const Operands &op, int64_t *crpt, int32_t
     time_begin(h, kSlotCopy, s);
     CK(copy_bins(true, !aside, s));
     time_end(h, kSlotCopy, s);
-    cudaError_t copied = cudaSuccess;
+    SideWork side(h);
     if (aside) {
+        cudaStream_t cs;
         CK(cudaEventRecord(h->ev_fork, s));
-        CK(cudaStreamWaitEvent(h->side[0], h->ev_fork, 0));
-        copied = copy_bins(false, true, h->side[0]);
-        const cudaError_t e = cudaEventRecord(h->ev_side[0], h->side[0]);
-        if (copied == cudaSuccess) copied = e;
+        CK(side.fork(0, &cs));
+        CK(copy_bins(false, true, cs));
     }
     if (h->xcount > 0) {
         BinWork w{};
@@ -1112,13 +1119,9 @@ int numeric_learned(spgemm_handle *h, const Operands &op, int64_t *crpt, int32_t
         CK(launch_num(num_kernel_count() - 1, op, w, static_cast<size_t>(std::max<int64_t>(words, 1)) * 12, s));
         time_end(h, kSlotNumBin + 15, s);
     }
-    const int rc = h->rep_num ? run_repeats(h, op, crpt, *pcol, *pval) : SPGEMM_OK;
-    if (aside) {
-        const cudaError_t e = cudaStreamWaitEvent(s, h->ev_side[0], 0);
-        if (copied == cudaSuccess) copied = e;
-        CK(copied);
-    }
-    if (rc) return rc;
+    if (h->rep_num)
+        if (const int rc = run_repeats(h, op, crpt, *pcol, *pval)) return rc;
+    CK(side.join());
     if (h->tcap_have > kTempKeep) release_temp(h);
     return SPGEMM_OK;
 }

@@ -1,0 +1,210 @@
+// A host stand-in for the CUDA runtime and the kernel launches, linked with
+// the object of api.cu: device memory is host memory, a launch only notes
+// that its stream has work, and launch number `k` fails. Drives one product
+// per k and reports memory that is freed, or a call that returns, while a
+// side stream has work that the handle's stream does not wait for.
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <map>
+
+#include "internal.h"
+#include "opsparse.h"
+
+using namespace ops;
+
+namespace {
+
+constexpr int64_t kRows = 40000;
+
+struct Event {
+    cudaStream_t s = nullptr;
+    long long at = 0;
+};
+std::map<cudaStream_t, long long> work, waited;   // last work of a stream; of it, what the main stream waits for
+std::map<cudaEvent_t, Event> events;
+long long now_ = 0, handles = 0;
+long long launches = 0, fail_at = 0;
+bool faults = false;
+const cudaStream_t kMain = reinterpret_cast<cudaStream_t>(uintptr_t{1});
+const char *where = "";
+
+void check(const char *what) {
+    for (const auto &[s, at] : work)
+        if (s != kMain && at > waited[s]) {
+            std::printf("%s, launch %lld failed: %s while a side stream has work\n", where, fail_at, what);
+            faults = true;
+            waited[s] = at;   // once
+        }
+}
+
+cudaError_t launch(cudaStream_t s) {
+    if (++launches == fail_at) return cudaErrorLaunchOutOfResources;
+    work[s] = ++now_;
+    return cudaSuccess;
+}
+
+void *take(size_t bytes, void *, void *) { return std::calloc(1, bytes); }
+void give(void *p, void *, void *) {
+    check("memory is freed");
+    std::free(p);
+}
+
+const KernelDesc kKernels[] = {{8, 256, 64, 32, 0, 0}, {32, 128, 256, 128, 0, 0}, {1024, 1024, 0, LLONG_MAX, 1, 0}};
+
+}  // namespace
+
+// --- the runtime ---------------------------------------------------------------
+extern "C" {
+cudaError_t cudaGetDevice(int *d) { *d = 0; return cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr a, int) {
+    *v = a == cudaDevAttrMultiProcessorCount ? 152 : 227 * 1024;
+    return cudaSuccess;
+}
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) {
+    *s = reinterpret_cast<cudaStream_t>(static_cast<uintptr_t>(100 + ++handles));
+    return cudaSuccess;
+}
+cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t s) { if (s != kMain) waited[s] = work[s]; return cudaSuccess; }
+cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned) {
+    if (s == kMain && events[e].s && waited[events[e].s] < events[e].at) waited[events[e].s] = events[e].at;
+    return cudaSuccess;
+}
+cudaError_t cudaEventCreate(cudaEvent_t *e) { *e = reinterpret_cast<cudaEvent_t>(static_cast<uintptr_t>(1000 + ++handles)); return cudaSuccess; }
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return cudaEventCreate(e); }
+cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) { events[e] = Event{s, work[s]}; return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t) { std::memcpy(d, s, n); return cudaSuccess; }
+cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) { std::memcpy(d, s, n); return cudaSuccess; }
+cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t) { std::memset(d, v, n); return cudaSuccess; }
+cudaError_t cudaMemset(void *d, int v, size_t n) { std::memset(d, v, n); return cudaSuccess; }
+cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) { *p = std::calloc(1, n); return cudaSuccess; }
+cudaError_t cudaFreeHost(void *p) { std::free(p); return cudaSuccess; }
+const char *cudaGetErrorName(cudaError_t) { return "fake"; }
+void **__cudaRegisterFatBinary(void *) { static void *h; return &h; }
+void __cudaRegisterFatBinaryEnd(void **) {}
+void __cudaUnregisterFatBinary(void **) {}
+void __cudaRegisterFunction(void **, const char *, char *, const char *, int, uint3 *, uint3 *, dim3 *, dim3 *, int *) {}
+}
+
+// --- the kernels -----------------------------------------------------------------
+namespace ops {
+int num_kernel_count() { return 3; }
+int sym_kernel_count() { return 3; }
+const KernelDesc &num_kernel(int id) { return kKernels[id]; }
+const KernelDesc &sym_kernel(int id) { return kKernels[id]; }
+cudaError_t num_prepare(int) { return cudaSuccess; }
+cudaError_t sym_prepare(int) { return cudaSuccess; }
+cudaError_t win_prepare(int) { return cudaSuccess; }
+cudaError_t rep_prepare() { return cudaSuccess; }
+int64_t bin_tile_rows() { return 4096; }
+size_t num_bitmap_head_bytes(bool) { return 1024; }
+int mlp_param_count() { return 4673; }
+int default_sym_bins(long long *range, int32_t *kernel) {
+    const long long r[] = {32, 128, -1};
+    for (int j = 0; j < 3; ++j) {
+        range[j] = r[j];
+        kernel[j] = j;
+    }
+    return 3;
+}
+cudaError_t launch_setup(const Operands &, int64_t, int64_t *, int64_t, int64_t, Counters *, int, cudaStream_t s, const RepWord *,
+                         const RepGate &, bool) { return launch(s); }
+cudaError_t launch_feature_scan(const Operands &, int64_t, int64_t *, unsigned *, unsigned *, int, cudaStream_t s, const RepGate &) { return launch(s); }
+// every bin has rows, most of the rows repeat
+cudaError_t launch_bin_pass1(const int64_t *, int64_t n, const Ranges &rg, const Operands &, Counters *cnt, long long *tiles, cudaStream_t s,
+                             const RepArgs &) {
+    for (int j = 0; j < rg.nb; ++j) {
+        cnt->bin_cnt[j] = j + 1 < rg.nb ? 8000 : static_cast<unsigned long long>(n - 8000 * (rg.nb - 1));
+        cnt->bin_own[j] = 100;
+    }
+    cnt->rep_cnt[0] = static_cast<unsigned long long>(n - 100 * rg.nb);
+    cnt->total = 100;
+    (void)tiles;
+    return launch(s);
+}
+cudaError_t launch_bin_pass2(const int64_t *, int64_t, const Ranges &, const long long *, Counters *, int32_t *, cudaStream_t s, const RepArgs &) { return launch(s); }
+cudaError_t launch_scan(int64_t *, int64_t, long long *, cudaStream_t s) { return launch(s); }
+cudaError_t launch_iota(int32_t *, int64_t, cudaStream_t s) { return launch(s); }
+cudaError_t launch_sym(int, const Operands &, const BinWork &, size_t, cudaStream_t s) { return launch(s); }
+cudaError_t launch_num(int, const Operands &, const BinWork &, size_t, cudaStream_t s) { return launch(s); }
+cudaError_t launch_num_onephase(int, const Operands &, const BinWork &w, cudaStream_t s) {
+    *w.xcount += 5;   // mispredicted rows
+    return launch(s);
+}
+cudaError_t launch_copy_rows(const BinWork &, bool, bool, cudaStream_t s) { return launch(s); }
+cudaError_t launch_predict(const Operands &, int64_t, const float *, const int64_t *, const unsigned *, const unsigned *, long long *, float, long long,
+                           cudaStream_t s) { return launch(s); }
+cudaError_t launch_predict_few(const Operands &, int64_t, const float *, const int64_t *, const unsigned *, const unsigned *, const RepWord *,
+                               const RepGate &, long long, long long, long long *, int64_t *, const SizeFactors &, uint8_t *, unsigned long long *,
+                               float, long long, cudaStream_t s) { return launch(s); }
+cudaError_t launch_learned_sizes(const int64_t *, const long long *, int64_t, long long, long long, int64_t *, const SizeFactors &, uint8_t *,
+                                 unsigned long long *, cudaStream_t s) { return launch(s); }
+cudaError_t launch_row_patterns(const void *, int, const int32_t *, int64_t, int64_t, int64_t, uint8_t *, unsigned long long *, const RepGate &,
+                                cudaStream_t s) { return launch(s); }
+cudaError_t launch_repeats(const Operands &, int64_t, const uint8_t *, const uint8_t *, RepWord *, const RepGate &, cudaStream_t s) { return launch(s); }
+cudaError_t launch_repeats_finish(int64_t, int64_t *, long long, const RepWord *, RepWord *, cudaStream_t s) { return launch(s); }
+cudaError_t launch_repeat_numeric(int, int, const Operands &, const RepWord *, const int64_t *, int32_t *, double *, int *, cudaStream_t s) { return launch(s); }
+cudaError_t launch_win_bindex(const Operands &, int64_t, const WinPlan &, long long, int32_t *, int32_t *, long long, unsigned long long *,
+                              cudaStream_t s) { return launch(s); }
+}  // namespace ops
+
+// One product, launch number `k` failing; false when the product has fewer.
+static bool product(int mode, long long k) {
+    work.clear();
+    waited.clear();
+    events.clear();
+    launches = 0;
+    fail_at = k;
+    where = mode == SPGEMM_MODE_LEARNED ? "learned" : "plain";
+    spgemm_handle *h = nullptr;
+    if (spgemm_create(&h, nullptr, take, give, nullptr, kMain) != SPGEMM_OK) std::abort();
+    if (mode == SPGEMM_MODE_LEARNED) {
+        static float theta[4673];
+        if (spgemm_set_predictor(h, theta, 0.f) != SPGEMM_OK || spgemm_set_mode(h, mode) != SPGEMM_OK) std::abort();
+    }
+    static int32_t rpt[kRows + 1], col[1];
+    static double val[1];
+    spgemm_csr_in A{};
+    A.rows = A.cols = kRows;
+    A.nnz = 16 * kRows;
+    A.rpt = rpt;
+    A.col = col;
+    A.val = val;
+    spgemm_csr_out C{};
+    int64_t nnz = 0;
+    int rc = spgemm_symbolic(h, &A, &A, 0, kRows, &nnz);
+    check("spgemm_symbolic returns");
+    if (rc == SPGEMM_OK) {
+        rc = spgemm_numeric(h, &A, &A, &C);
+        check("spgemm_numeric returns");
+    }
+    if (rc == SPGEMM_OK && mode == SPGEMM_MODE_PLAIN) {
+        rc = spgemm_numeric_values(h, &A, &A, &C);
+        check("spgemm_numeric_values returns");
+    }
+    const bool failed = launches >= k;
+    if ((rc != SPGEMM_OK) != failed) {
+        std::printf("%s, launch %lld failed: result %d\n", where, k, rc);
+        faults = true;
+    }
+    if (C.rpt) {
+        std::free(C.rpt);
+        std::free(C.col);
+        std::free(C.val);
+    }
+    spgemm_destroy(h);
+    return failed;
+}
+
+int main() {
+    for (int mode : {SPGEMM_MODE_PLAIN, SPGEMM_MODE_LEARNED}) {
+        long long k = 1;
+        while (product(mode, k)) ++k;
+        std::printf("%s: %lld launches\n", where, k - 1);
+    }
+    return faults ? 1 : 0;
+}
