@@ -45,6 +45,38 @@ __device__ __forceinline__ int64_t block_row_of(const void *rpt, int is64, int64
     return lo;
 }
 
+// What is left of a tile after kWalkSteps steps from row to row is not walked:
+// its entries search their rows. Runs of empty rows in one tile are one
+// block's: 8.4M of them in A 24.0 ms when walked and 2.1 ms this way (whole
+// product), in B 9.5 and 0.17, 16.8M rows with 2,000 entries 44.5 and 2.4.
+constexpr int kWalkSteps = 32;
+
+// The entries [p0, t1) of A's tile that begins at t0, in the rows [row, row + n)
+// of which the first begins at or before p0; s_len as in row_lengths. (One entry
+// at a time, added by atomics: merging neighbours would cost the walk registers.)
+template <bool FEAT>
+__device__ __forceinline__ void sparse_tile_lengths(const Operands &op, int64_t *nprod, unsigned *maxlen,
+                                                    unsigned *minlen, const RepWord *words, int64_t row, int n,
+                                                    int64_t p0, int64_t t0, int64_t t1, const int *s_len) {
+#pragma unroll 1
+    for (int e = static_cast<int>(p0 - t0) + static_cast<int>(threadIdx.x); t0 + e < t1; e += kTileBlock) {
+        const int64_t r = upper_bound_rpt(op.arpt, op.a64, row, row + n, t0 + e) - op.row0;
+        unsigned len;
+        if (words) {
+            if ((words[r >> 5].fol >> (r & 31)) & 1u) continue;
+            const int c = __ldg(op.acol + t0 + e);
+            len = static_cast<unsigned>(ld_rpt(op.brpt, op.b64, c + 1) - ld_rpt(op.brpt, op.b64, c));
+        } else {
+            len = static_cast<unsigned>(s_len[e]);
+        }
+        atomicAdd(reinterpret_cast<unsigned long long *>(nprod + r), static_cast<unsigned long long>(len));
+        if (FEAT) {
+            atomicMax(maxlen + r, len);
+            atomicMin(minlen + r, len);
+        }
+    }
+}
+
 // Threads that reduce one row's part of a tile: a quarter of the mean row
 // length, so that a mean row takes about four steps and a tile of short rows
 // about as many rounds as its rows over the block.
@@ -87,7 +119,7 @@ __device__ __forceinline__ void row_lengths(const Operands &op, int64_t *nprod, 
                 s_len[j * kTileBlock + threadIdx.x] =
                     static_cast<int>(ld_rpt(op.brpt, op.b64, k[j] + 1) - ld_rpt(op.brpt, op.b64, k[j]));
         __syncthreads();
-        for (;; row += rows_per) {
+        for (int step = 1;; ++step, row += rows_per) {
             const int64_t i = row + g;
             long long sum = 0;
             unsigned mx = 0, mn = UINT_MAX;
@@ -138,10 +170,17 @@ __device__ __forceinline__ void row_lengths(const Operands &op, int64_t *nprod, 
             }
             // stop at the batch that reaches the end of the tile; the next
             // tile starts in its last row that begins at or before the end
-            const bool stop = row + rows_per >= hi || ld_rpt(op.arpt, op.a64, row + rows_per) >= t1;   // uniform
+            const int64_t next = row + rows_per;
+            const bool stop = next >= hi || ld_rpt(op.arpt, op.a64, next) >= t1;   // uniform
             if (stop) {
                 const int begun = __syncthreads_count(l == 0 && i < hi && s <= t1);
                 row += begun - 1;
+                break;
+            }
+            if (step == kWalkSteps) {
+                row = block_row_of(op.arpt, op.a64, next, hi, t1);
+                sparse_tile_lengths<FEAT>(op, nprod, maxlen, minlen, words, next, static_cast<int>(row - next + 1),
+                                          ld_rpt(op.arpt, op.a64, next), t0, t1, s_len);
                 break;
             }
         }
@@ -174,16 +213,40 @@ __device__ __forceinline__ void order_check(const Operands &op, int64_t brows, i
             c1[j] = e + 1 < bnnz && e < t1 ? __ldg(op.bcol + e + 1) : INT_MAX;
         }
         __syncthreads();
-        for (;; row += kTileBlock) {   // row starts in (t0, t1]
+        bool sparse = true;
+        for (int step = 0; step < kWalkSteps; ++step, row += kTileBlock) {   // row starts in (t0, t1]
             const int64_t i = row + threadIdx.x;
             const int64_t s = i < brows ? ld_rpt(op.brpt, op.b64, i) : INT64_MAX;
             if (s > t0 && s <= t1) s_start[s - t0] = 1;
-            const bool stop = row + kTileBlock >= brows || ld_rpt(op.brpt, op.b64, row + kTileBlock) > t1;   // uniform
+            const int64_t next = row + kTileBlock;
+            const bool stop = next >= brows || ld_rpt(op.brpt, op.b64, next) > t1;   // uniform
             if (stop) {
                 const int begun = __syncthreads_count(s <= t1);
                 row += begun - 1;
+                sparse = false;
                 break;
             }
+        }
+        if (sparse) {
+            // the starts from row `row` on are searched for
+            const int64_t end = block_row_of(op.brpt, op.b64, row, brows, t1);
+#pragma unroll 1
+            for (int e = static_cast<int>(ld_rpt(op.brpt, op.b64, row) - t0) + static_cast<int>(threadIdx.x); t0 + e <= t1;
+                 e += kTileBlock) {
+                const int64_t r = upper_bound_rpt(op.brpt, op.b64, row, end + 1, t0 + e);
+                if (ld_rpt(op.brpt, op.b64, r) == t0 + e) s_start[e] = 1;
+            }
+            __syncthreads();
+            row = end;
+#pragma unroll 1
+            for (int e = threadIdx.x; t0 + e < t1 && t0 + e + 1 < bnnz; e += kTileBlock) {
+                const int a = __ldg(op.bcol + t0 + e), b = __ldg(op.bcol + t0 + e + 1);
+                if (b <= a && !s_start[e + 1]) {
+                    bad |= b < a;
+                    dup |= b == a;
+                }
+            }
+            continue;
         }
 #pragma unroll
         for (int j = 0; j < kTileItems; ++j)
@@ -197,9 +260,11 @@ __device__ __forceinline__ void order_check(const Operands &op, int64_t brows, i
         atomicOr(&cnt->flags, (any_bad ? 1ull : 0ull) | (any_dup ? 2ull : 0ull));
 }
 
+// (Five blocks on an SM, 48 registers: at six the searches of sparse tiles spill
+// into the walk, 27-point stencil 128^3 170 us for n_prod instead of 164.)
 // Both scans in one launch: the first `nprod_blocks` blocks count products,
 // the others check B's order (either part may have no blocks).
-__global__ void __launch_bounds__(kTileBlock)
+__global__ void __launch_bounds__(kTileBlock, 5)
 setup_kernel(Operands op, int64_t *nprod, const RepWord *words, RepGate gate, bool only_open, int nprod_blocks,
              int64_t brows, int64_t bnnz, Counters *cnt) {
     __shared__ int s_len[kTileEntries + 4];
@@ -212,7 +277,7 @@ setup_kernel(Operands op, int64_t *nprod, const RepWord *words, RepGate gate, bo
                     reinterpret_cast<unsigned char *>(s_len));
 }
 
-__global__ void __launch_bounds__(kTileBlock)
+__global__ void __launch_bounds__(kTileBlock, 5)
 feature_scan_kernel(Operands op, int64_t *nprod, unsigned *maxlen, unsigned *minlen, RepGate gate) {
     __shared__ int s_len[kTileEntries];
     if (gate.found && !gate.shut()) return;   // uniform over the grid

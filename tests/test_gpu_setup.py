@@ -88,3 +88,122 @@ def test_order_check_at_tile_edges(at, kind):
         h.status()
     for g, w in zip(got.numpy(), oracle.spgemm(A, B)[:3]):
         assert np.array_equal(g, w)
+
+
+# Entries in more rows than the scans walk (32 steps of at most 256 rows):
+# their tiles search the rows instead.
+SPARSE = {
+    **{f"{k} empty rows": [5, 3] + [0] * k + [4, 2] for k in (8189, 8190, 8191, 8192, 8193)},
+    "several gaps": [3] * 10 + [0] * 200000 + [2] * 3000 + [0] * 50000 + [1] + [0] * 30000,
+    "a row in 37": [1 + i % 3 if i % 37 == 5 else 0 for i in range(150000)],
+    "long rows apart": [1500] + [0] * 9000 + [1500] + [0] * 9000 + [2 * TILE + 700] + [0] * 9000 + [3],
+    "gap at a tile's edge": [TILE - 1] + [0] * 20000 + [1] + [0] * 20000 + [1, 2],
+}
+
+
+@pytest.mark.parametrize("i64", [False, True])
+@pytest.mark.parametrize("name", SPARSE)
+def test_entries_in_far_apart_rows_of_A(name, i64):
+    K = 7000
+    A = rows_of(SPARSE[name], K, 1)
+    B = rows_of(np.random.default_rng(2).integers(0, 4, K), 900, 3)
+    want = oracle.nprod(A, B)
+    t = np.int64 if i64 else np.int32
+    dA, dB = (ops.CSR.from_arrays(m.rows, m.cols, m.rpt.astype(t), m.col, m.val) for m in (A, B))
+    with ops.Handle() as h:
+        got = h.multiply(dA, dB)
+        st = h.stats()
+        h.status()
+        r0 = A.rows // 3
+        h.symbolic(dA, dB, r0, A.rows)
+        part = h.numeric(dA, dB)
+        h.status()
+    assert st["total_nprod"] == want.sum() and st["max_nprod"] == want.max(initial=0)
+    for r, C in ((0, got), (r0, part)):
+        for g, w in zip(C.numpy(), oracle.spgemm(A, B, r, A.rows)[:3]):
+            assert np.array_equal(g, w)
+    X = learned.features(dA, dB).cpu().numpy()
+    length = np.diff(B.rpt)
+    full = np.flatnonzero(np.diff(A.rpt))
+    for k, f in ((2, np.maximum), (4, np.minimum)):
+        w = f.reduceat(length[A.col], A.rpt[full])
+        np.testing.assert_allclose(X[full, k], np.log1p(w.astype(np.float64)), rtol=4e-7, atol=0)
+
+
+@pytest.mark.parametrize("fault", ["none", "repeat", "decrease"])
+@pytest.mark.parametrize("name", SPARSE)
+def test_order_check_with_far_apart_rows_of_B(name, fault):
+    # one entry in B's last long row breaks the order; entries that only
+    # follow the end of another row do not
+    B = rows_of(SPARSE[name], 9000, 5)
+    lens = np.diff(B.rpt)
+    q = B.rpt[np.flatnonzero(lens >= 2)[-1]]
+    if fault == "repeat":
+        B.col[q + 1] = B.col[q]
+    elif fault == "decrease":
+        B.col[[q, q + 1]] = B.col[[q + 1, q]]
+    full = np.flatnonzero(lens)[-40:]
+    A = W.Csr(3, B.rows, np.array([0, full.size, full.size, 2 * full.size], dtype=np.int32),
+              np.concatenate([full, full]).astype(np.int32), np.arange(2.0 * full.size) - 30)
+    with ops.Handle() as h:
+        got = h.multiply(ops.CSR.from_workload(A), ops.CSR.from_workload(B))
+        h.status()
+    for g, w in zip(got.numpy(), oracle.spgemm(A, B)[:3]):
+        assert np.array_equal(g, w)
+
+
+def test_repeating_rows_around_a_gap():
+    # a band of 33 columns with 40,000 empty rows inside: repeating rows are
+    # left out of the scan of a tile whose entries search their rows, too
+    n, offs = 45000, np.arange(-16, 17)
+    lists = [np.zeros(0, int) if 20000 <= i < 60000 else (j := i if i < 20000 else i - 40000) + offs[(j + offs >= 0) & (j + offs < n)]
+             for i in range(n + 40000)]
+    rpt = np.zeros(len(lists) + 1, dtype=np.int32)
+    np.cumsum([x.size for x in lists], out=rpt[1:])
+    col = np.concatenate(lists).astype(np.int32)
+    rng = np.random.default_rng(4)
+    A = W.Csr(len(lists), n, rpt, col, rng.integers(-3, 4, col.size).astype(np.float64))
+    B = rows_of([9] * n, 300, 3)
+    for k in range(n):   # rows that repeat the row before, moved by one
+        B.col[9 * k:9 * k + 9] = k + np.arange(9)
+    B.cols = n + 9
+    with ops.Handle() as h:
+        got = h.multiply(ops.CSR.from_workload(A), ops.CSR.from_workload(B))
+        st = h.stats()
+        h.status()
+    assert st["total_nprod"] == oracle.nprod(A, B).sum()
+    for g, w in zip(got.numpy(), oracle.spgemm(A, B)[:3]):
+        assert np.array_equal(g, w)
+
+
+@pytest.mark.parametrize("side", ["A", "B"])
+def test_empty_rows_are_not_walked_by_one_block(side):
+    # 8M empty rows between two ends of 20,000 rows: what a row costs with all
+    # blocks at work (rows of A: row pointers, counters, bins and offsets,
+    # about 100 bytes; rows of B: nothing) is below 3 ms at a fifth of the
+    # memory rate; one block alone waits about 1.2 us for every 256 rows
+    gap = 1 << 23
+    lens = np.concatenate([np.full(20000, 4), np.zeros(gap, int), np.full(20000, 4)])
+    rpt = np.zeros(lens.size + 1, dtype=np.int32)
+    np.cumsum(lens, out=rpt[1:])
+    other = rows_of([4] * 20000, 20000, 2)
+    rng = np.random.default_rng(6)
+    if side == "A":
+        A = W.Csr(lens.size, 20000, rpt, rng.integers(0, 20000, rpt[-1]).astype(np.int32), np.ones(rpt[-1]))
+        B = other
+    else:
+        A = W.Csr(20000, lens.size, other.rpt, (other.col % 20000 + (gap + 20000) * (other.col % 2)).astype(np.int32), other.val)
+        B = W.Csr(lens.size, 20000, rpt, np.tile(np.arange(0, 20000, 5000, dtype=np.int32), 40000), np.ones(rpt[-1]))
+    dA, dB = ops.CSR.from_workload(A), ops.CSR.from_workload(B)
+    with ops.Handle() as h:
+        best = np.inf
+        for _ in range(6):
+            e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            e0.record()
+            C = h.multiply(dA, dB)
+            e1.record()
+            h.status()
+            best = min(best, e0.elapsed_time(e1))
+        for g, w in zip(C.numpy(), oracle.spgemm(A, B)[:3]):
+            assert np.allclose(g, w, rtol=1e-12, atol=1e-12)
+    assert best < (6.0 if side == "A" else 3.0), best
