@@ -607,7 +607,7 @@ struct SideWork {
 // Launch the kernels of one phase, one per non-empty bin, largest rows first,
 // spread over the side streams. runs: plan of a windowed pass 2 for the
 // numeric bitmap kernel (nullptr or runs->lists == 0: whole-row pass 2).
-int run_bins(spgemm_handle *h, int phase, const Operands &op, const long long *size,
+int run_bins(spgemm_handle *h, int phase, const Operands &op, const spgemm_csr_in *B, const long long *size,
              const long long *offset, bool identity, int64_t *crpt, int32_t *ccol, double *cval,
              const RunPlan *runs = nullptr, const WinCall *win = nullptr) {
     const int nb = phase ? h->cfg.num_nbins : h->cfg.sym_nbins;
@@ -628,6 +628,7 @@ int run_bins(spgemm_handle *h, int phase, const Operands &op, const long long *s
         w.unroll = h->cfg.bitmap_unroll;
         w.multi = h->cfg.hash_access;
         w.distinct = h->b_distinct;
+        w.by_column = phase && h->b_distinct && span_rows(B->nnz, B->rows);
         w.clk = phase == 1 && h->phase_clk ? h->d_clk : nullptr;
         w.err = d_err(h);
         const KernelDesc &d = phase ? num_kernel(kid[j]) : sym_kernel(kid[j]);
@@ -927,6 +928,7 @@ int symbolic_learned(spgemm_handle *h, const Operands &op, const spgemm_csr_in *
         w.crpt = crpt;
         w.lanes = h->cfg.num_lanes_per_brow;
         w.distinct = h->b_distinct;
+        w.by_column = h->b_distinct && span_rows(B->nnz, B->rows);
         w.err = d_err(h);
         w.tcol = h->tcol; w.tval = h->tval;
         w.tbase = h->ltbase[j]; w.tcap = h->ltcap[j];
@@ -1378,7 +1380,7 @@ int spgemm_symbolic(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_i
         wc0.on = nbm > 0;
     }
     // step 3: symbolic kernels, largest rows first
-    if ((rc = run_bins(h, 0, op, ssize, soff, sid, crpt, nullptr, nullptr, nullptr, &wc0))) return fail(rc);
+    if ((rc = run_bins(h, 0, op, B, ssize, soff, sid, crpt, nullptr, nullptr, nullptr, &wc0))) return fail(rc);
     // windows of the rows of the last numeric bin (their count sizes the list)
     if (h->wp_on &&
         note(launch_win_count(h->wplan, crpt, mw, wc0.on ? h->wcells : nullptr, wc0.on ? h->wcslot : nullptr,
@@ -1569,7 +1571,7 @@ int spgemm_numeric(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_in
         }
         rp.bs = bs;
     }
-    rc = run_bins(h, 1, op, h->num_size, off, nid, crpt, ccol, cval, &rp, &wc);
+    rc = run_bins(h, 1, op, B, h->num_size, off, nid, crpt, ccol, cval, &rp, &wc);
     if (!rc && h->rep_num) rc = run_repeats(h, op, crpt, ccol, cval);
     dev_free(h, bs);
     if (rc) {
@@ -1645,7 +1647,7 @@ int spgemm_numeric_values(spgemm_handle *h, const spgemm_csr_in *A, const spgemm
         wc.bidx = h->wbidx;
     }
     int64_t *crpt = static_cast<int64_t *>(C->rpt);
-    rc = run_bins(h, 1, op, h->num_size, off, nonempty <= 1 && !h->rep_num, crpt, C->col, C->val, nullptr, &wc);
+    rc = run_bins(h, 1, op, B, h->num_size, off, nonempty <= 1 && !h->rep_num, crpt, C->col, C->val, nullptr, &wc);
     if (!rc && h->rep_num) rc = run_repeats(h, op, crpt, C->col, C->val);
     return rc;
 }

@@ -49,6 +49,8 @@ struct BinWork {
     int distinct;         // every row of B has strictly ascending columns (checked): warp-row
                           // kernels may bound a row's columns by the ends of its B rows, and
                           // update values without atomics
+    int by_column;        // numeric phase, with distinct: B's rows are long enough for a warp to
+                          // add rows by column (span_rows)
     int *err;             // device error word
     // numeric bitmap kernel, pass 2 by column windows (B rows sorted)
     const int32_t *bs;    // run boundaries of B rows at the sub-ranges (G + 1 per row), or nullptr
@@ -205,6 +207,17 @@ struct KernelDesc {
     int bitmap;       // 1: shared-memory column bitmap kernel
     size_t smem;      // dynamic shared memory per block
 };
+
+// Adding a row by column takes one B row per step, so short B rows leave most
+// of the warp idle: it is looked at when B's rows have more than 4 entries on
+// average (the numeric phase then reads the ends of a row's B rows first), and
+// used for rows whose own B rows fill 16 lanes, or 8 when A has at most
+// kSpanShort entries there. Numeric phase by the table and by column, 20,000
+// rows over 100 columns: B rows of 1 entry and 400 entries of A 151 and 520 us,
+// of 4 and 400 299 and 536, of 8 and 50 87 and 84, of 8 and 1,600 1,855 and
+// 2,049, of 16 and 50 133 and 84, of 16 and 400 841 and 559.
+constexpr int kSpanShort = 128;
+inline bool span_rows(int64_t bnnz, int64_t brows) { return bnnz > 4 * brows; }
 
 // --- setup.cu ----------------------------------------------------------------
 // n_prod of every row of the window, added into nprod (zeroed by the caller;

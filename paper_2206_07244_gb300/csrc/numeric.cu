@@ -322,17 +322,17 @@ num_hash_kernel(Operands op, BinWork w) {
         }
     }
     // A warp's row whose columns span at most kSpan columns is accumulated by
-    // column in the table's memory (B's rows strictly ascending): no probes, no
-    // condense and no sort.
+    // column in the table's memory (B's rows strictly ascending and not too short,
+    // kSpanShort): no probes, no condense and no sort.
     constexpr bool kMaySpan = TPR == 32 && !MULTI;
     constexpr int kSpan = (T * 12 / 8) / 32 * 32;
     int S = TPR, col0 = 0, span = 0, len0 = 0;
     long long q0 = 0;
-    if (kMaySpan && w.distinct && w.lanes == 0) {
+    if (kMaySpan && w.by_column && w.lanes == 0) {
         long long sum;
         row_span(op, p0, p1, sum, col0, span, q0, len0);
         S = pick_lanes_distinct(0, sum, p1 - p0, TPR);
-        if (span > kSpan) span = 0;
+        if (span > kSpan || S < 8 || (S == 8 && p1 - p0 > kSpanShort)) span = 0;
     } else {
         S = numeric_lanes<TPR>(op, w.lanes, p0, p1, lg, red64);
     }

@@ -87,3 +87,43 @@ def test_special_values():
     got = C.numpy()
     assert np.array_equal(got[0], rpt) and np.array_equal(got[1], col)
     assert np.array_equal(got[2], val, equal_nan=True)
+
+
+def even(rows, per_row, cols, seed, reverse=False):
+    """Every row `per_row` distinct columns, ascending (or descending)."""
+    rng = np.random.default_rng(seed)
+    col = np.sort(rng.random((rows, cols)).argpartition(per_row - 1, axis=1)[:, :per_row], axis=1)
+    if reverse:
+        col = col[:, ::-1]
+    return W.Csr(rows, cols, np.arange(0, rows * per_row + 1, per_row, dtype=np.int32), col.astype(np.int32).ravel(),
+                 rng.integers(-3, 4, rows * per_row).astype(np.float64))
+
+
+def numeric_ms(h, dA, dB):
+    C = h.multiply(dA, dB)
+    best = np.inf
+    for _ in range(9):
+        e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        e0.record()
+        h.numeric_values(dA, dB, C)
+        e1.record()
+        h.status()
+        best = min(best, e0.elapsed_time(e1))
+    return best, C
+
+
+@pytest.mark.parametrize("entries, length", [(200, 2), (400, 2), (400, 4), (1600, 4), (1600, 8)])
+def test_short_rows_of_B_are_not_added_one_at_a_time(entries, length):
+    # descending columns take the table whatever the rows of B are; ascending
+    # ones must not be slower by more than a tenth of it and the noise
+    times = []
+    A = even(4000, entries, 2000, 1)
+    for reverse in (False, True):
+        B = even(2000, length, 100, 2, reverse)
+        dA, dB = (ops.CSR.from_arrays(m.rows, m.cols, m.rpt, m.col, m.val) for m in (A, B))
+        with ops.Handle() as h:
+            ms, C = numeric_ms(h, dA, dB)
+        times.append(ms)
+        for g, w in zip(C.numpy(), oracle.spgemm(A, B)[:3]):
+            assert np.array_equal(g, w)
+    assert times[0] < 1.25 * times[1], times
