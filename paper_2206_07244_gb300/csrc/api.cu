@@ -122,6 +122,10 @@ struct spgemm_handle {
     size_t rcode_bytes = 0;
     RepWord *rwords = nullptr;    // the last symbolic call's words, one per 32 window rows, and as many unfinished ones
     size_t rwords_bytes = 0;
+    int32_t *rowq = nullptr;      // row queues of the numeric kernels
+    size_t rowq_bytes = 0;
+    double num_na[kMaxBins] = {};          // numeric bins: mean A entries of a row
+    long long max_nprod = 0;               // of a window row
     bool rep_num = false;         // the numeric phase leaves them out of its bins
     long long rep_cnt[kRepClasses] = {};   // rows per class
     // column-window numeric path for the last numeric bin (window.cu)
@@ -604,6 +608,24 @@ struct SideWork {
     }
 };
 
+// Warp- or block-per-row form of numeric bin j's rows (num_row_limits): na A
+// entries a row on average, at most `most` products. cnt holds the queue's
+// length, which a second numeric call over the same bins clears on the bin's
+// stream s. Without memory for the queue every row takes the block form.
+cudaError_t set_row_form(spgemm_handle *h, int j, const Operands &op, const spgemm_csr_in *B, double na,
+                         long long most, Counters *cnt, BinWork &w, cudaStream_t s) {
+    const double mean_b = static_cast<double>(B->nnz) / static_cast<double>(std::max<int64_t>(B->rows, 1));
+    if (!num_row_limits(h->cfg.num_kernel[j], op, na, mean_b, most, w)) return cudaSuccess;
+    if (ensure_buf(h, &h->rowq, &h->rowq_bytes, sizeof(int32_t) * (size_t)op.mw)) {
+        w.block_rows = 1;
+        return cudaSuccess;
+    }
+    w.queue = h->rowq + w.off;
+    w.queued = cnt->queued + j;
+    w.queue_grid = h->sm_count * 12;
+    return h->reuse ? cudaMemsetAsync(w.queued, 0, sizeof(unsigned), s) : cudaSuccess;
+}
+
 // Launch the kernels of one phase, one per non-empty bin, largest rows first,
 // spread over the side streams. runs: plan of a windowed pass 2 for the
 // numeric bitmap kernel (nullptr or runs->lists == 0: whole-row pass 2).
@@ -628,9 +650,10 @@ int run_bins(spgemm_handle *h, int phase, const Operands &op, const spgemm_csr_i
         w.unroll = h->cfg.bitmap_unroll;
         w.multi = h->cfg.hash_access;
         w.distinct = h->b_distinct;
-        w.by_column = phase && h->b_distinct && span_rows(B->nnz, B->rows);
+        w.by_column = phase && h->b_distinct && span_rows(h->num_na[j], B->nnz, B->rows);
         w.clk = phase == 1 && h->phase_clk ? h->d_clk : nullptr;
         w.err = d_err(h);
+        if (phase) CK(set_row_form(h, j, op, B, h->num_na[j], h->max_nprod, d_counters(h, 1), w, s));
         const KernelDesc &d = phase ? num_kernel(kid[j]) : sym_kernel(kid[j]);
         size_t smem = 0;
         const int slot = (phase ? kSlotNumBin : kSlotSymBin) + j;
@@ -928,7 +951,9 @@ int symbolic_learned(spgemm_handle *h, const Operands &op, const spgemm_csr_in *
         w.crpt = crpt;
         w.lanes = h->cfg.num_lanes_per_brow;
         w.distinct = h->b_distinct;
-        w.by_column = h->b_distinct && span_rows(B->nnz, B->rows);
+        const Counters &c = h->h_cnt[0];
+        const double na = c.bin_cnt[j] ? static_cast<double>(c.bin_nnza[j]) / static_cast<double>(c.bin_cnt[j]) : 0.0;
+        w.by_column = h->b_distinct && span_rows(na, B->nnz, B->rows);
         w.err = d_err(h);
         w.tcol = h->tcol; w.tval = h->tval;
         w.tbase = h->ltbase[j]; w.tcap = h->ltcap[j];
@@ -938,6 +963,7 @@ int symbolic_learned(spgemm_handle *h, const Operands &op, const spgemm_csr_in *
         w.lcls = L.cls;
         w.fb = L.fb;
         w.tprev = j > 0 ? num_kernel(h->cfg.num_kernel[j - 1]).table : 0;
+        CK(set_row_form(h, j, op, B, na, exact_above < 0 ? LLONG_MAX : exact_above, d_counters(h, 0), w, ss));
         const int slot = kSlotNumBin + j;
         time_begin(h, slot, ss);
         CK(launch_num_onephase(h->cfg.num_kernel[j], op, w, ss));
@@ -1359,6 +1385,7 @@ int spgemm_symbolic(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_i
     if (!repeats) rep = RepArgs{};
     h->stats[0] = static_cast<int64_t>(h->h_cnt[0].total);
     h->stats[1] = static_cast<int64_t>(h->h_cnt[0].max_size);
+    h->max_nprod = static_cast<long long>(h->h_cnt[0].max_size);
     for (int j = 0; j < SPGEMM_MAX_BINS; ++j) h->stats[4 + j] = j < rs.nb ? static_cast<int64_t>(h->h_cnt[0].bin_cnt[j]) : 0;
     if (!sid) {
         time_begin(h, kSlotSymPass2, h->stream);
@@ -1406,6 +1433,10 @@ int spgemm_symbolic(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_i
     h->stats[3] = static_cast<int64_t>(h->h_cnt[1].max_size);
     for (int j = 0; j < SPGEMM_MAX_BINS; ++j)
         h->stats[4 + SPGEMM_MAX_BINS + j] = j < rn.nb ? static_cast<int64_t>(h->h_cnt[1].bin_cnt[j]) : 0;
+    for (int j = 0; j < rn.nb; ++j) {
+        const Counters &c = h->h_cnt[1];
+        h->num_na[j] = c.bin_cnt[j] ? static_cast<double>(c.bin_nnza[j]) / static_cast<double>(c.bin_cnt[j]) : 0.0;
+    }
     // repeating rows are added without atomics: distinct columns in B's rows
     h->rep_num = false;
     for (int c = 0; c < kRepClasses; ++c) {
@@ -2052,6 +2083,7 @@ int spgemm_destroy(spgemm_handle *h) {
     win_release(h);
     dev_free(h, h->rcode);
     dev_free(h, h->rwords);
+    dev_free(h, h->rowq);
     dev_free(h, h->wcells);
     dev_free(h, h->wcslot);
     dev_free(h, h->wspill);

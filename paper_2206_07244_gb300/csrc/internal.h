@@ -51,6 +51,13 @@ struct BinWork {
                           // update values without atomics
     int by_column;        // numeric phase, with distinct: B's rows are long enough for a warp to
                           // add rows by column (span_rows)
+    // warp-per-row forms of block-per-row numeric kernels (num_row_limits): rows of
+    // more products than their limit go to the queue, for the block form
+    long long long_col, long_near, long_far;
+    int32_t *queue;       // places in the bin (room for cnt), nullptr: every row is taken
+    unsigned *queued;     // their number (0 before)
+    int queue_grid;       // blocks of the block form's launch over the queue, at most
+    int block_rows;       // every row by the block form
     int *err;             // device error word
     // numeric bitmap kernel, pass 2 by column windows (B rows sorted)
     const int32_t *bs;    // run boundaries of B rows at the sub-ranges (G + 1 per row), or nullptr
@@ -185,6 +192,7 @@ struct Counters {
     unsigned long long bin_own[kMaxBins];   // pass 1: the bin's rows that do not repeat a row before
     unsigned long long rep_cnt[kRepClasses];   // numeric pass 1: repeating rows per class
     unsigned long long rep_found;           // rows of A that look like the row before
+    unsigned queued[kMaxBins];              // rows in the numeric kernels' queues
     unsigned long long max_size;
     unsigned long long total;
     unsigned long long flags;         // bit 0: some row of B has decreasing columns; bit 1: repeated ones
@@ -209,15 +217,17 @@ struct KernelDesc {
 };
 
 // Adding a row by column takes one B row per step, so short B rows leave most
-// of the warp idle: it is looked at when B's rows have more than 4 entries on
-// average (the numeric phase then reads the ends of a row's B rows first), and
-// used for rows whose own B rows fill 16 lanes, or 8 when A has at most
-// kSpanShort entries there. Numeric phase by the table and by column, 20,000
+// of the warp idle: it is used for rows whose own B rows fill 16 lanes, or 8
+// when A has at most kSpanShort entries there, and looked at (the numeric phase
+// then reads the ends of a row's B rows first) in bins whose mean lengths say
+// so. Numeric phase by the table and by column, 20,000
 // rows over 100 columns: B rows of 1 entry and 400 entries of A 151 and 520 us,
 // of 4 and 400 299 and 536, of 8 and 50 87 and 84, of 8 and 1,600 1,855 and
 // 2,049, of 16 and 50 133 and 84, of 16 and 400 841 and 559.
 constexpr int kSpanShort = 128;
-inline bool span_rows(int64_t bnnz, int64_t brows) { return bnnz > 4 * brows; }
+inline bool span_rows(double na, int64_t bnnz, int64_t brows) {
+    return bnnz > 8 * brows || (bnnz > 4 * brows && na <= kSpanShort);
+}
 
 // --- setup.cu ----------------------------------------------------------------
 // n_prod of every row of the window, added into nprod (zeroed by the caller;
@@ -265,6 +275,12 @@ cudaError_t launch_sym(int id, const Operands &op, const BinWork &w, size_t smem
                        cudaStream_t s);
 cudaError_t launch_num(int id, const Operands &op, const BinWork &w, size_t smem_bitmap,
                        cudaStream_t s);
+// Which rows of the bin `w` kernel `id` multiplies by a warp each and which by a
+// block each: sets the limits and block_rows of w (cnt, lanes, multi and
+// by_column set before). na: A entries of the bin's rows, mean_b: entries of B's
+// rows, both on average; most: products of any row. True when rows may have to
+// change form, so that the launch needs a queue.
+bool num_row_limits(int id, const Operands &op, double na, double mean_b, long long most, BinWork &w);
 // one-phase numeric kernel `id` (a hash kernel of the numeric table)
 cudaError_t launch_num_onephase(int id, const Operands &op, const BinWork &w, cudaStream_t s);
 

@@ -20,6 +20,7 @@
 // float64 atomicAdd in global memory (L2). 227 KB cover 1.2M columns per
 // pass; wider matrices take several column windows. This replaces the
 // paper's global-memory hash kernel (its kernel 7) and its condense/sort.
+#include <algorithm>
 #include <climits>
 
 #include "common.cuh"
@@ -82,9 +83,9 @@ __device__ __forceinline__ bool num_insert_owned(int *tk, double *tv, int key, d
 // group recomputes it from B.rpt (those lines are needed right after).
 template <int TPR>
 __device__ __forceinline__ int numeric_lanes(const Operands &op, int fixed, int64_t p0,
-                                             int64_t p1, int lg, long long *red) {
+                                             int64_t p1, int lg, long long *red, long long &sum) {
+    sum = 0;   // products of the row, unless the lanes are fixed
     if (fixed > 0) return pick_lanes_distinct(fixed, 0, 1, TPR);
-    long long sum = 0;
     for (int64_t p = p0 + lg; p < p1; p += TPR) {
         const int k = __ldg(op.acol + p);
         sum += ld_rpt(op.brpt, op.b64, k + 1) - ld_rpt(op.brpt, op.b64, k);
@@ -272,11 +273,14 @@ __device__ __forceinline__ void warp_sort_store(const int *tk, const double *tv,
 // than the table can sort in place, marks the row as mispredicted: it is
 // queued for the exact path and nothing is written. Otherwise the row's
 // size goes to C.rpt and its sorted entries to its temporary slot.
-template <int TPR, int BLOCK, int T, bool ONE_PHASE = false, bool MULTI = false>
+// QUEUE: warp-per-row kernels leave rows past their limit in the queue, block-per-
+// row kernels take theirs from it, a block one row after the other.
+template <int TPR, int BLOCK, int T, bool ONE_PHASE = false, bool MULTI = false, bool QUEUE = false>
 __global__ void __launch_bounds__(BLOCK, (T * 12 * (BLOCK / TPR) > 110 * 1024) ? 1
                                          : (TPR == 32 ? (T <= 256 ? 1280 : T <= 512 ? 896 : 576) : (TPR > 32 ? 1536 : 2048)) / BLOCK)
 num_hash_kernel(Operands op, BinWork w) {
     constexpr int RPB = BLOCK / TPR;
+    constexpr bool kTake = QUEUE && TPR > 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ long long red64[32];
     __shared__ int red32[33];
@@ -284,9 +288,16 @@ num_hash_kernel(Operands op, BinWork w) {
     const int g = threadIdx.x / TPR, lg = threadIdx.x % TPR;
     double *tv = reinterpret_cast<double *>(smem_raw + static_cast<size_t>(g) * (T * 12));   // the row's table
     int *tk = reinterpret_cast<int *>(tv + T);
+    unsigned turn = blockIdx.x;
+[[maybe_unused]] next_row:
+    if constexpr (kTake) {
+        if (turn >= __ldcg(w.queued)) return;   // uniform over the block
+        __syncthreads();   // readers of the row before are done
+    }
     bool failed = false;
     if (lg == 0) full[g] = 0;
-    const int64_t r = static_cast<int64_t>(blockIdx.x) * RPB + g;
+    const int64_t r = kTake ? w.queue[turn] : static_cast<int64_t>(blockIdx.x) * RPB + g;   // the row's place in the bin
+    turn += gridDim.x;
     const bool valid = r < w.cnt;
     const int64_t row = valid ? (w.bins ? static_cast<int64_t>(w.bins[w.off + r]) : w.off + r) : 0;
     int64_t cbase = 0, n_expect = 0, p0 = 0, p1 = 0;
@@ -327,14 +338,21 @@ num_hash_kernel(Operands op, BinWork w) {
     constexpr bool kMaySpan = TPR == 32 && !MULTI;
     constexpr int kSpan = (T * 12 / 8) / 32 * 32;
     int S = TPR, col0 = 0, span = 0, len0 = 0;
-    long long q0 = 0;
+    long long q0 = 0, sum = 0;
+    bool far = false;   // QUEUE: a block would sort the row's entries, not place them by its span bitmap
     if (kMaySpan && w.by_column && w.lanes == 0) {
-        long long sum;
         row_span(op, p0, p1, sum, col0, span, q0, len0);
         S = pick_lanes_distinct(0, sum, p1 - p0, TPR);
+        far = QUEUE && (ONE_PHASE ? T / 2 : n_expect) + 2 * ((static_cast<int64_t>(span) + 31) >> 5) > T;
         if (span > kSpan || S < 8 || (S == 8 && p1 - p0 > kSpanShort)) span = 0;
     } else {
-        S = numeric_lanes<TPR>(op, w.lanes, p0, p1, lg, red64);
+        S = numeric_lanes<TPR>(op, w.lanes, p0, p1, lg, red64, sum);
+    }
+    if constexpr (QUEUE && TPR == 32) {
+        if (sum > (span > 0 && S >= 16 ? w.long_col : far ? w.long_far : w.long_near)) {
+            if (lg == 0) w.queue[atomicAdd(w.queued, 1u)] = static_cast<int32_t>(r);   // r < cnt: sum > 0
+            return;   // uniform over the warp; no block barrier follows
+        }
     }
     const bool dense = kMaySpan && span > 0;   // uniform over the warp, and over the row group
     if (dense) {
@@ -429,7 +447,8 @@ num_hash_kernel(Operands op, BinWork w) {
                 if (at < static_cast<unsigned long long>(w.xlimit)) w.xlist[at] = static_cast<int32_t>(row);
                 else set_error(w.err, DERR_BOUNDS);
             }
-            return;   // uniform over the row group
+            if constexpr (kTake) goto next_row;
+            else return;   // uniform over the row group
         }
         n_expect = n;
         if (valid && lg == 0) {
@@ -560,7 +579,8 @@ num_hash_kernel(Operands op, BinWork w) {
                         }
                     }
                 }
-                return;   // uniform over the block
+                if constexpr (kTake) goto next_row;
+                else return;   // uniform over the block
             }
         }
     }
@@ -602,6 +622,7 @@ num_hash_kernel(Operands op, BinWork w) {
             oval[t] = tv[t];
         }
     }
+    if constexpr (kTake) goto next_row;
 }
 
 // Rank of every bitmap word's first column: pre[i] = set bits in words
@@ -1023,15 +1044,20 @@ static NumFn g_num_multi[] = {NUM_TABLE(NUM_MULTI_ENTRY)};
 // which sort by a span bitmap or in shared memory, 64 and 128 threads wide;
 // so does the read-then-swap probe.
 constexpr int64_t kWarpRowCols = int64_t{1} << 23;
-#define NUM_WARP(BLOCK, T)                                                                          \
-    {BLOCK, (sizeof(int) + sizeof(double)) * (BLOCK / 32 * (size_t)T + kStage * (size_t)BLOCK),      \
-     &num_hash_kernel<32, BLOCK, T>, &num_hash_kernel<32, BLOCK, T, true>}
+// [0] every row, [1] with a queue; fn and one-phase.
+#define NUM_WARP(TPR, BLOCK, T)                                                                  \
+    {BLOCK, (sizeof(int) + sizeof(double)) * (BLOCK / 32 * (size_t)T + kStage * (size_t)BLOCK),  \
+     {{&num_hash_kernel<32, BLOCK, T>, &num_hash_kernel<32, BLOCK, T, true>},                    \
+      {&num_hash_kernel<32, BLOCK, T, false, false, true>, &num_hash_kernel<32, BLOCK, T, true, false, true>}}, \
+     {&num_hash_kernel<TPR, TPR, T, false, false, true>, &num_hash_kernel<TPR, TPR, T, true, false, true>}}
 static const struct {
     int block;
     size_t smem;
-    NumFn fn, onephase;
-} g_num_warp[] = {NUM_WARP(128, 512), NUM_WARP(64, 1024)};
+    NumFn fn[2][2];
+    NumFn queued[2];   // the block form over the queue
+} g_num_warp[] = {NUM_WARP(64, 128, 512), NUM_WARP(128, 64, 1024)};
 constexpr int kNumWarpFirst = 3;   // kernels 3 and 4 of the table
+constexpr int kNumWarp = sizeof(g_num_warp) / sizeof(g_num_warp[0]);
 
 static constexpr int kNumHash = sizeof(g_num) / sizeof(g_num[0]);
 static KernelDesc g_num_bitmap{1024, 1024, 0, LLONG_MAX, 1, 0};
@@ -1073,12 +1099,16 @@ cudaError_t num_prepare(int smem_optin) {
                                  static_cast<int>(g_num[i].d.smem));
         if (e != cudaSuccess) return e;
     }
-    for (const auto &v : g_num_warp)
-        for (const NumFn fn : {v.fn, v.onephase}) {
-            const cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(fn),
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       static_cast<int>(v.smem));
-            if (e != cudaSuccess) return e;
+    for (int k = 0; k < kNumWarp; ++k)
+        for (int phase = 0; phase < 2; ++phase) {
+            const auto &v = g_num_warp[k];
+            for (const NumFn fn : {v.fn[0][phase], v.fn[1][phase], v.queued[phase]}) {
+                const size_t smem = fn == v.queued[phase] ? g_num[kNumWarpFirst + k].d.smem : v.smem;
+                const cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void *>(fn),
+                                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                           static_cast<int>(smem));
+                if (e != cudaSuccess) return e;
+            }
         }
     g_num_bitmap.table = static_cast<long long>((smem_optin - sizeof(WalkScratch)) / 12) * 64;
     for (const auto &v : g_num_bm) {
@@ -1114,19 +1144,80 @@ static int pick_bitmap_variant(size_t smem_total, int iters) {
 // The warp-per-row form of kernel `id` for these operands, -1: none.
 static int warp_row_form(int id, const Operands &op, const BinWork &w) {
     const int k = id - kNumWarpFirst;
-    return k >= 0 && k < static_cast<int>(sizeof(g_num_warp) / sizeof(g_num_warp[0])) && op.ncols <= kWarpRowCols &&
-                   !w.multi ? k : -1;
+    return k >= 0 && k < kNumWarp && op.ncols <= kWarpRowCols &&
+                   !w.multi && !w.block_rows ? k : -1;
+}
+
+// A warp takes a row without block barriers, but a row of many products keeps
+// it long after the others, and the 1024-slot table leaves half as many warps
+// on an SM as the block form has. Numeric phase, block and warp form in us, n
+// entries a row (n = 200: 512 slots, 400: 1024 slots):
+//   unsorted, n = 200, 6,400 products: 300 rows 87 and 125, 3,000 rows 209 and
+//     149; n = 400, 1,200 products: 300 rows 31 and 43, 20,000 rows 311 and 325;
+//   a hub of 10^6 products among 30,000 short rows: 10,500 and 25,600;
+//   by column, n = 400, B rows of 48: 2,400 products, 300 rows 33 and 42, 20,000
+//     rows 368 and 297; B rows of 24, 2,400 products, 3,000 rows 83 and 63;
+//   columns too far apart for a block's span bitmap, so that it sorts: n = 400,
+//     2,400 products: 300 rows 58 and 71, 3,000 rows 155 and 135, 20,000 rows
+//     925 and 628; 12,800 products, 20,000 rows 1,857 and 1,856.
+// The limits lie where the two meet. What most rows are like is told from the
+// mean lengths and B's width, and whole bins past their limit take the block
+// form; a row is looked at, and sent to the block form's queue, only when some
+// row passes that limit: a queue that nothing needed cost 4 us to 8 us, one that
+// held most rows of a bin up to 60% of its time.
+bool num_row_limits(int id, const Operands &op, double na, double mean_b, long long most, BinWork &w) {
+    w.long_col = w.long_near = w.long_far = LLONG_MAX;
+    const int k = warp_row_form(id, op, w);
+    if (k < 0) return false;
+    const double mean = na * mean_b;
+    const auto or_mean = [&](long long limit) { return std::max(limit, static_cast<long long>(4.0 * mean)); };
+    const long long table = g_num[id].d.table;
+    const bool narrow = op.ncols <= 8 * table;                        // no row is too wide for the span bitmap
+    const bool fits = op.ncols <= table * 12 / 8 / 32 * 32;           // every row's span fits the accumulator
+    if (k == 0) {
+        const bool many = w.cnt >= 2048;
+        w.long_col = or_mean(16384);
+        w.long_near = many ? or_mean(1024) : 1024;
+        w.long_far = many ? or_mean(4096) : 2048;
+    } else {
+        const bool many = w.cnt >= 16384;
+        w.long_col = many ? or_mean(2048) : w.cnt >= 2048 ? 3072 : w.cnt >= 512 ? 2048 : 1024;
+        w.long_near = many || !narrow ? 1024 : 0;
+        w.long_far = many ? 8192 : w.cnt >= 2048 ? 3072 : 1536;
+    }
+    long long least, most_rows;   // limits of the rows that the bin may hold
+    if (w.by_column && fits) {
+        least = most_rows = w.long_col;
+    } else if (w.by_column && !narrow) {
+        least = std::min(w.long_col, w.long_far);
+        most_rows = std::max(w.long_col, w.long_far);
+    } else {
+        least = most_rows = w.long_near;
+    }
+    if (most <= least) return false;
+    if (w.lanes > 0 || mean > static_cast<double>(most_rows)) {   // fixed lanes: products are not counted
+        w.block_rows = 1;
+        return false;
+    }
+    return true;
+}
+
+// Kernel `id` in its warp-per-row form k, then the rows in the queue.
+static cudaError_t launch_warp_rows(int k, int phase, const Operands &op, const BinWork &w, cudaStream_t s) {
+    const auto &v = g_num_warp[k];
+    const int64_t rpb = v.block / 32;
+    v.fn[w.queue ? 1 : 0][phase]<<<static_cast<unsigned>((w.cnt + rpb - 1) / rpb), v.block, v.smem, s>>>(op, w);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess || !w.queue) return e;
+    const KernelDesc &d = g_num[kNumWarpFirst + k].d;
+    v.queued[phase]<<<static_cast<unsigned>(std::min<int64_t>(w.cnt, w.queue_grid)), d.block, d.smem, s>>>(op, w);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_num_onephase(int id, const Operands &op, const BinWork &w, cudaStream_t s) {
     if (w.cnt <= 0) return cudaSuccess;
     if (id < 0 || id >= kNumHash) return cudaErrorInvalidValue;
-    if (const int k = warp_row_form(id, op, w); k >= 0) {
-        const auto &v = g_num_warp[k];
-        const int64_t rpb = v.block / 32;
-        v.onephase<<<static_cast<unsigned>((w.cnt + rpb - 1) / rpb), v.block, v.smem, s>>>(op, w);
-        return cudaGetLastError();
-    }
+    if (const int k = warp_row_form(id, op, w); k >= 0) return launch_warp_rows(k, 1, op, w, s);
     const KernelDesc &d = g_num[id].d;
     const int rpb = d.block / d.tpr;
     const int64_t grid = (w.cnt + rpb - 1) / rpb;
@@ -1183,11 +1274,8 @@ cudaError_t launch_copy_rows(const BinWork &w, bool cols, bool vals, cudaStream_
 cudaError_t launch_num(int id, const Operands &op, const BinWork &w, size_t smem_bitmap,
                        cudaStream_t s) {
     if (w.cnt <= 0) return cudaSuccess;
-    if (const int k = warp_row_form(id, op, w); k >= 0) {
-        const auto &v = g_num_warp[k];
-        const int64_t rpb = v.block / 32;
-        v.fn<<<static_cast<unsigned>((w.cnt + rpb - 1) / rpb), v.block, v.smem, s>>>(op, w);
-    } else if (id < kNumHash) {
+    if (const int k = warp_row_form(id, op, w); k >= 0) return launch_warp_rows(k, 0, op, w, s);
+    if (id < kNumHash) {
         const KernelDesc &d = g_num[id].d;
         const int rpb = d.block / d.tpr;
         const int64_t grid = (w.cnt + rpb - 1) / rpb;

@@ -102,6 +102,7 @@ cudaError_t win_prepare(int) { return cudaSuccess; }
 cudaError_t rep_prepare() { return cudaSuccess; }
 int64_t bin_tile_rows() { return 4096; }
 size_t num_bitmap_head_bytes(bool) { return 1024; }
+bool num_row_limits(int, const Operands &, double, double, long long, BinWork &) { return true; }
 int mlp_param_count() { return 4673; }
 int default_sym_bins(long long *range, int32_t *kernel) {
     const long long r[] = {32, 128, -1};
