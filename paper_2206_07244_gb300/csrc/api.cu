@@ -754,6 +754,12 @@ bool plan_bins(const Counters &c, int nb, long long *size, long long *offset, bo
     return all && nonempty <= 1;
 }
 
+// Entries of a window of mw rows at A's mean row length.
+int64_t window_entries(const spgemm_csr_in *A, int64_t mw) {
+    return static_cast<int64_t>(static_cast<double>(A->nnz) * static_cast<double>(mw) /
+                                static_cast<double>(std::max<int64_t>(A->rows, 1)));
+}
+
 // Compares the rows of A and B with the row before them when the product is
 // large enough for repeating rows to pay (kRepMinRows and following; *on).
 // A goes first: without an eighth of its rows repeating (*gate) B is not
@@ -777,7 +783,8 @@ int scan_patterns(spgemm_handle *h, const Operands &op, const spgemm_csr_in *A, 
     gate->found = found;
     gate->least = static_cast<unsigned long long>(std::max<int64_t>(1, (same ? B->rows : mw) / 8));
     if (!same)
-        CK(launch_row_patterns(op.arpt, op.a64, op.acol, op.row0, mw, A->nnz, code, found, RepGate(), h->stream));
+        CK(launch_row_patterns(op.arpt, op.a64, op.acol, op.row0, mw, window_entries(A, mw), code, found, RepGate(),
+                               h->stream));
     CK(launch_row_patterns(op.brpt, op.b64, op.bcol, 0, B->rows, B->nnz, h->rcode, same ? found : nullptr,
                            same ? RepGate() : *gate, h->stream));
     *acode = code;
@@ -867,7 +874,7 @@ int symbolic_learned(spgemm_handle *h, const Operands &op, const spgemm_csr_in *
     if ((rc = scan_patterns(h, op, A, B, &acode, &gate, &repeats))) return rc;
     RepWord *found_words = repeats ? h->rwords + (mw + 31) / 32 : nullptr;
     if (repeats) {
-        CK(launch_repeats(op, annz, acode, h->rcode, found_words, gate, s));
+        CK(launch_repeats(op, window_entries(A, mw), acode, h->rcode, found_words, gate, s));
         time_end(h, kSlotPatterns, s);
     }
     for (bool again = false;; again = true) {
@@ -1348,7 +1355,7 @@ int spgemm_symbolic(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_i
     if ((rc = scan_patterns(h, op, A, B, &acode, &gate, &repeats))) return fail(rc);
     if (repeats) {
         found_words = h->rwords + (mw + 31) / 32;
-        if (note(launch_repeats(op, A->nnz, acode, h->rcode, found_words, gate, h->stream)) != cudaSuccess)
+        if (note(launch_repeats(op, window_entries(A, mw), acode, h->rcode, found_words, gate, h->stream)) != cudaSuccess)
             return fail(SPGEMM_ERR_CUDA);
         time_end(h, kSlotPatterns, h->stream);
     }

@@ -3,6 +3,7 @@
 // that its stream has work, and launch number `k` fails. Drives one product
 // per k and reports memory that is freed, or a call that returns, while a
 // side stream has work that the handle's stream does not wait for.
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -26,6 +27,7 @@ std::map<cudaEvent_t, Event> events;
 long long now_ = 0, handles = 0;
 long long launches = 0, fail_at = 0;
 bool faults = false;
+double mean_entries = 0;   // of a row, in the pattern scans' launches
 const cudaStream_t kMain = reinterpret_cast<cudaStream_t>(uintptr_t{1});
 const char *where = "";
 
@@ -144,9 +146,15 @@ cudaError_t launch_predict_few(const Operands &, int64_t, const float *, const i
                                float, long long, cudaStream_t s) { return launch(s); }
 cudaError_t launch_learned_sizes(const int64_t *, const long long *, int64_t, long long, long long, int64_t *, const SizeFactors &, uint8_t *,
                                  unsigned long long *, cudaStream_t s) { return launch(s); }
-cudaError_t launch_row_patterns(const void *, int, const int32_t *, int64_t, int64_t, int64_t, uint8_t *, unsigned long long *, const RepGate &,
-                                cudaStream_t s) { return launch(s); }
-cudaError_t launch_repeats(const Operands &, int64_t, const uint8_t *, const uint8_t *, RepWord *, const RepGate &, cudaStream_t s) { return launch(s); }
+cudaError_t launch_row_patterns(const void *, int, const int32_t *, int64_t, int64_t n, int64_t entries, uint8_t *, unsigned long long *, const RepGate &,
+                                cudaStream_t s) {
+    mean_entries = std::max(mean_entries, static_cast<double>(entries) / static_cast<double>(n));
+    return launch(s);
+}
+cudaError_t launch_repeats(const Operands &op, int64_t entries, const uint8_t *, const uint8_t *, RepWord *, const RepGate &, cudaStream_t s) {
+    mean_entries = std::max(mean_entries, static_cast<double>(entries) / static_cast<double>(op.mw));
+    return launch(s);
+}
 cudaError_t launch_repeats_finish(int64_t, int64_t *, long long, const RepWord *, RepWord *, cudaStream_t s) { return launch(s); }
 cudaError_t launch_repeat_numeric(int, int, const Operands &, const RepWord *, const int64_t *, int32_t *, double *, int *, cudaStream_t s) { return launch(s); }
 cudaError_t launch_win_bindex(const Operands &, int64_t, const WinPlan &, long long, int32_t *, int32_t *, long long, unsigned long long *,
@@ -154,7 +162,7 @@ cudaError_t launch_win_bindex(const Operands &, int64_t, const WinPlan &, long l
 }  // namespace ops
 
 // One product, launch number `k` failing; false when the product has fewer.
-static bool product(int mode, long long k) {
+static bool product(int mode, long long k, int64_t row_entries = 16, int64_t rows = kRows, bool same = true) {
     work.clear();
     waited.clear();
     events.clear();
@@ -171,23 +179,26 @@ static bool product(int mode, long long k) {
     static double val[1];
     spgemm_csr_in A{};
     A.rows = A.cols = kRows;
-    A.nnz = 16 * kRows;
+    A.nnz = row_entries * kRows;
     A.rpt = rpt;
     A.col = col;
     A.val = val;
+    static int32_t other[1];
+    spgemm_csr_in B = A;
+    if (!same) B.col = other;
     spgemm_csr_out C{};
     int64_t nnz = 0;
-    int rc = spgemm_symbolic(h, &A, &A, 0, kRows, &nnz);
+    int rc = spgemm_symbolic(h, &A, &B, 0, rows, &nnz);
     check("spgemm_symbolic returns");
     if (rc == SPGEMM_OK) {
-        rc = spgemm_numeric(h, &A, &A, &C);
+        rc = spgemm_numeric(h, &A, &B, &C);
         check("spgemm_numeric returns");
     }
     if (rc == SPGEMM_OK && mode == SPGEMM_MODE_PLAIN) {
-        rc = spgemm_numeric_values(h, &A, &A, &C);
+        rc = spgemm_numeric_values(h, &A, &B, &C);
         check("spgemm_numeric_values returns");
     }
-    const bool failed = launches >= k;
+    const bool failed = k > 0 && launches >= k;
     if ((rc != SPGEMM_OK) != failed) {
         std::printf("%s, launch %lld failed: result %d\n", where, k, rc);
         faults = true;
@@ -206,6 +217,15 @@ int main() {
         long long k = 1;
         while (product(mode, k)) ++k;
         std::printf("%s: %lld launches\n", where, k - 1);
+    }
+    // a row window: its rows' mean length, not the whole matrix's entries over them
+    for (bool same : {true, false}) {
+        mean_entries = 0;
+        product(SPGEMM_MODE_PLAIN, 0, 64, 5000, same);
+        if (mean_entries < 63 || mean_entries > 65) {
+            std::printf("pattern scans of a window launched for %.0f entries a row, not 64\n", mean_entries);
+            faults = true;
+        }
     }
     return faults ? 1 : 0;
 }
