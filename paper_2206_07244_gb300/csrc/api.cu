@@ -765,7 +765,8 @@ int64_t window_entries(const spgemm_csr_in *A, int64_t mw) {
 // A goes first: without an eighth of its rows repeating (*gate) B is not
 // looked at. The column-window form (bitmap_path 2) plans its windows from
 // the sizes of all rows before they are filled in, and the read-then-swap
-// probe is there to be measured: both multiply every row on its own.
+// probe is there to be measured: both multiply every row on its own, and so does
+// a call without memory for the codes and words.
 int scan_patterns(spgemm_handle *h, const Operands &op, const spgemm_csr_in *A, const spgemm_csr_in *B,
                   const uint8_t **acode, RepGate *gate, bool *on) {
     const int64_t mw = op.mw;
@@ -776,8 +777,9 @@ int scan_patterns(spgemm_handle *h, const Operands &op, const spgemm_csr_in *A, 
     if (per_row < kRepMinProducts || (mw < kRepManyRows && per_row * static_cast<double>(mw) < kRepManyProducts))
         return SPGEMM_OK;
     const bool same = A->rpt == B->rpt && A->rpt_is_i64 == B->rpt_is_i64 && A->col == B->col && A->rows == B->rows;
-    int rc = ensure_buf(h, &h->rcode, &h->rcode_bytes, (size_t)B->rows + (same ? 0 : (size_t)mw));
-    if (rc || (rc = ensure_buf(h, &h->rwords, &h->rwords_bytes, 2 * sizeof(RepWord) * (size_t)((mw + 31) / 32)))) return rc;
+    if (ensure_buf(h, &h->rcode, &h->rcode_bytes, (size_t)B->rows + (same ? 0 : (size_t)mw)) ||
+        ensure_buf(h, &h->rwords, &h->rwords_bytes, 2 * sizeof(RepWord) * (size_t)((mw + 31) / 32)))
+        return SPGEMM_OK;
     uint8_t *code = same ? h->rcode + op.row0 : h->rcode + B->rows;
     unsigned long long *found = &d_counters(h, 0)->rep_found;
     gate->found = found;

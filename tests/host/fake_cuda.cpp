@@ -46,7 +46,10 @@ cudaError_t launch(cudaStream_t s) {
     return cudaSuccess;
 }
 
-void *take(size_t bytes, void *, void *) { return std::calloc(1, bytes); }
+long long allocations = 0, fail_allocation = 0;
+void *take(size_t bytes, void *, void *) {
+    return ++allocations == fail_allocation ? nullptr : std::calloc(1, bytes);
+}
 void give(void *p, void *, void *) {
     check("memory is freed");
     std::free(p);
@@ -162,18 +165,31 @@ cudaError_t launch_win_bindex(const Operands &, int64_t, const WinPlan &, long l
 }  // namespace ops
 
 // One product, launch number `k` failing; false when the product has fewer.
-static bool product(int mode, long long k, int64_t row_entries = 16, int64_t rows = kRows, bool same = true) {
+static bool product(int mode, long long k, int64_t row_entries = 16, int64_t rows = kRows, bool same = true, int patterns = 1,
+                    int *result = nullptr) {
     work.clear();
     waited.clear();
     events.clear();
-    launches = 0;
+    launches = allocations = 0;
     fail_at = k;
     where = mode == SPGEMM_MODE_LEARNED ? "learned" : "plain";
     spgemm_handle *h = nullptr;
     if (spgemm_create(&h, nullptr, take, give, nullptr, kMain) != SPGEMM_OK) std::abort();
     if (mode == SPGEMM_MODE_LEARNED) {
         static float theta[4673];
-        if (spgemm_set_predictor(h, theta, 0.f) != SPGEMM_OK || spgemm_set_mode(h, mode) != SPGEMM_OK) std::abort();
+        const int rc = spgemm_set_predictor(h, theta, 0.f);
+        if (rc == SPGEMM_ERR_OOM && result) {
+            *result = rc;
+            spgemm_destroy(h);
+            return true;
+        }
+        if (rc != SPGEMM_OK || spgemm_set_mode(h, mode) != SPGEMM_OK) std::abort();
+    }
+    if (!patterns) {   // the read-then-swap probe: every row on its own
+        spgemm_config cfg;
+        spgemm_get_config(h, &cfg);
+        cfg.hash_access = 1;
+        if (spgemm_set_config(h, &cfg) != SPGEMM_OK) std::abort();
     }
     static int32_t rpt[kRows + 1], col[1];
     static double val[1];
@@ -198,7 +214,8 @@ static bool product(int mode, long long k, int64_t row_entries = 16, int64_t row
         rc = spgemm_numeric_values(h, &A, &B, &C);
         check("spgemm_numeric_values returns");
     }
-    const bool failed = k > 0 && launches >= k;
+    if (result) *result = rc;
+    const bool failed = (k > 0 && launches >= k) || (fail_allocation > 0 && allocations >= fail_allocation && rc == SPGEMM_ERR_OOM);
     if ((rc != SPGEMM_OK) != failed) {
         std::printf("%s, launch %lld failed: result %d\n", where, k, rc);
         faults = true;
@@ -224,6 +241,23 @@ int main() {
         product(SPGEMM_MODE_PLAIN, 0, 64, 5000, same);
         if (mean_entries < 63 || mean_entries > 65) {
             std::printf("pattern scans of a window launched for %.0f entries a row, not 64\n", mean_entries);
+            faults = true;
+        }
+    }
+    // an allocation that fails: looking for repeating rows takes memory of its
+    // own, without which every row is multiplied on its own
+    for (int mode : {SPGEMM_MODE_PLAIN, SPGEMM_MODE_LEARNED}) {
+        int refused[2] = {};
+        for (int patterns : {0, 1})
+            for (fail_allocation = 1;; ++fail_allocation) {
+                int rc = SPGEMM_OK;
+                product(mode, 0, 16, kRows, true, patterns, &rc);
+                if (allocations < fail_allocation) break;
+                refused[patterns] += rc != SPGEMM_OK;
+            }
+        fail_allocation = 0;
+        if (refused[0] != refused[1]) {
+            std::printf("%s: %d allocations that fail the product, %d without the pattern scans\n", where, refused[1], refused[0]);
             faults = true;
         }
     }

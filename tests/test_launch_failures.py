@@ -1,6 +1,7 @@
 """A launch that fails inside a call, with kernels of the same call on side
 streams: before the call frees memory or returns, the handle's stream waits
-for them. And what the pattern scans of a row window are launched for. CPU only: the object of api.cu is linked with a host stand-in for
+for them. What the pattern scans of a row window are launched for, and what
+happens without memory for them. CPU only: the object of api.cu is linked with a host stand-in for
 the CUDA runtime and the kernels (host/fake_cuda.cpp)."""
 
 import os
