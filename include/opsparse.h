@@ -348,7 +348,10 @@ int spgemm_mlp_param_count(void);
 int spgemm_set_predictor(spgemm_handle *h, const float *theta, float margin);
 
 /* SPGEMM_MODE_PLAIN or SPGEMM_MODE_LEARNED (needs a predictor; not between
- * spgemm_symbolic and spgemm_numeric: SPGEMM_ERR_STATE). */
+ * spgemm_symbolic and spgemm_numeric: SPGEMM_ERR_STATE). In learned mode the
+ * handle keeps the temporary memory of the one-phase rows, up to 400 MB of it,
+ * from call to call; it goes back when the mode is set to plain, when another
+ * allocation of the handle would fail, and in spgemm_destroy. */
 int spgemm_set_mode(spgemm_handle *h, int mode);
 
 /* After a learned-mode spgemm_symbolic (up to 6 + SPGEMM_MAX_BINS values):

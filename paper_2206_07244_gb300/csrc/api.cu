@@ -108,8 +108,9 @@ struct spgemm_handle {
     unsigned char *lscratch = nullptr;
     size_t lscratch_bytes = 0;
     int32_t *tcol = nullptr;      // temporary one-phase rows of the current call (kept for the next
-    double *tval = nullptr;       // one up to kTempKeep entries)
+    double *tval = nullptr;       // one up to kTempKeep entries, until other memory runs out)
     long long tcap_have = 0;
+    bool temp_used = false;       // between their allocation and the copy into C
     long long lsize[kMaxBins] = {}, loff[kMaxBins] = {}, ltbase[kMaxBins] = {}, ltcap[kMaxBins] = {};
     long long ltotal = 0;
     bool lid = false;
@@ -171,21 +172,33 @@ struct spgemm_handle {
 
 namespace {
 
-void *dev_alloc(spgemm_handle *h, size_t bytes) {
-    bytes = std::max<size_t>(bytes, 256);
-    if (h->alloc) return h->alloc(bytes, h->stream, h->ctx);
-    void *p = nullptr;
-    if (cudaMallocFromPoolAsync(&p, bytes, h->pool, h->stream) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    return p;
-}
-
 void dev_free(spgemm_handle *h, void *p) {
     if (!p) return;
     if (h->freefn) h->freefn(p, h->stream, h->ctx);
     else cudaFreeAsync(p, h->stream);
+}
+
+void release_temp(spgemm_handle *h) {
+    dev_free(h, h->tcol);
+    dev_free(h, h->tval);
+    h->tcol = nullptr;
+    h->tval = nullptr;
+    h->tcap_have = 0;
+    h->temp_used = false;
+}
+
+void *dev_alloc(spgemm_handle *h, size_t bytes) {
+    bytes = std::max<size_t>(bytes, 256);
+    for (;;) {
+        void *p = nullptr;
+        if (h->alloc) p = h->alloc(bytes, h->stream, h->ctx);
+        else if (cudaMallocFromPoolAsync(&p, bytes, h->pool, h->stream) != cudaSuccess) {
+            cudaGetLastError();
+            p = nullptr;
+        }
+        if (p || h->temp_used || h->tcap_have == 0) return p;
+        release_temp(h);   // kept for another learned call, not in use: once more without
+    }
 }
 
 void flush_slot(spgemm_handle *h, int k) {
@@ -294,14 +307,6 @@ int ensure_lscratch(spgemm_handle *h, int64_t mw) {
 // The one-phase rows' temporary memory is allocated while the GPU waits, so up
 // to 2^25 entries (400 MB) stay with the handle from call to call.
 constexpr long long kTempKeep = 1ll << 25;
-
-void release_temp(spgemm_handle *h) {
-    dev_free(h, h->tcol);
-    dev_free(h, h->tval);
-    h->tcol = nullptr;
-    h->tval = nullptr;
-    h->tcap_have = 0;
-}
 
 unsigned long long *d_xcount(spgemm_handle *h) {
     return reinterpret_cast<unsigned long long *>(h->arena + 2 * sizeof(Counters) + 8);
@@ -946,6 +951,7 @@ int symbolic_learned(spgemm_handle *h, const Operands &op, const spgemm_csr_in *
         if (!h->tcol || !h->tval) return SPGEMM_ERR_OOM;
         h->tcap_have = total_t;
     }
+    h->temp_used = true;
     // one-phase kernels, largest rows first on the side streams
     CK(cudaEventRecord(h->ev_fork, s));
     int used = 0;
@@ -1159,6 +1165,7 @@ int numeric_learned(spgemm_handle *h, const Operands &op, int64_t *crpt, int32_t
     if (h->rep_num)
         if (const int rc = run_repeats(h, op, crpt, *pcol, *pval)) return rc;
     CK(side.join());
+    h->temp_used = false;
     if (h->tcap_have > kTempKeep) release_temp(h);
     return SPGEMM_OK;
 }
@@ -2071,6 +2078,7 @@ int spgemm_set_mode(spgemm_handle *h, int mode) {
     if (mode == SPGEMM_MODE_LEARNED && !h->theta) return SPGEMM_ERR_STATE;
     if (h->state == 1) return SPGEMM_ERR_STATE;
     h->mode = mode;
+    if (mode == SPGEMM_MODE_PLAIN) release_temp(h);
     return SPGEMM_OK;
 }
 

@@ -47,11 +47,18 @@ cudaError_t launch(cudaStream_t s) {
 }
 
 long long allocations = 0, fail_allocation = 0;
+size_t live = 0, most = SIZE_MAX;   // bytes handed out, and at most
+std::map<void *, size_t> held;
 void *take(size_t bytes, void *, void *) {
-    return ++allocations == fail_allocation ? nullptr : std::calloc(1, bytes);
+    if (++allocations == fail_allocation || live + bytes > most) return nullptr;
+    void *p = std::calloc(1, bytes);
+    live += held[p] = bytes;
+    return p;
 }
 void give(void *p, void *, void *) {
     check("memory is freed");
+    live -= held[p];
+    held.erase(p);
     std::free(p);
 }
 
@@ -125,9 +132,9 @@ cudaError_t launch_bin_pass1(const int64_t *, int64_t n, const Ranges &rg, const
                              const RepArgs &) {
     for (int j = 0; j < rg.nb; ++j) {
         cnt->bin_cnt[j] = j + 1 < rg.nb ? 8000 : static_cast<unsigned long long>(n - 8000 * (rg.nb - 1));
-        cnt->bin_own[j] = 100;
+        cnt->bin_own[j] = static_cast<unsigned long long>(n / 10);
     }
-    cnt->rep_cnt[0] = static_cast<unsigned long long>(n - 100 * rg.nb);
+    cnt->rep_cnt[0] = static_cast<unsigned long long>(n - n / 10 * rg.nb);
     cnt->total = 100;
     (void)tiles;
     return launch(s);
@@ -220,13 +227,59 @@ static bool product(int mode, long long k, int64_t row_entries = 16, int64_t row
         std::printf("%s, launch %lld failed: result %d\n", where, k, rc);
         faults = true;
     }
-    if (C.rpt) {
-        std::free(C.rpt);
-        std::free(C.col);
-        std::free(C.val);
-    }
+    for (void *p : {static_cast<void *>(C.rpt), static_cast<void *>(C.col), static_cast<void *>(C.val)})
+        if (p) spgemm_free(h, p);
     spgemm_destroy(h);
     return failed;
+}
+
+// A plain product, or a learned one of half the rows, after a learned one, with
+// no more memory than that one left: it gets what is kept for the next one.
+static void kept_memory(bool back_to_plain) {
+    work.clear();
+    waited.clear();
+    events.clear();
+    fail_at = 0;
+    where = back_to_plain ? "plain after learned" : "learned after learned";
+    static float theta[4673];
+    static int32_t rpt[kRows + 1], col[1];
+    static double val[1];
+    spgemm_handle *h = nullptr;
+    spgemm_csr_in A{};
+    A.rows = A.cols = kRows;
+    A.nnz = 64 * kRows;
+    A.rpt = rpt;
+    A.col = col;
+    A.val = val;
+    spgemm_csr_out C{};
+    int64_t nnz = 0;
+    if (spgemm_create(&h, nullptr, take, give, nullptr, kMain) || spgemm_set_predictor(h, theta, 0.f) ||
+        spgemm_set_mode(h, SPGEMM_MODE_LEARNED) || spgemm_multiply(h, &A, &A, &C))
+        std::abort();
+    for (void *p : {static_cast<void *>(C.rpt), static_cast<void *>(C.col), static_cast<void *>(C.val)}) spgemm_free(h, p);
+    const size_t before = live;
+    if (back_to_plain) {
+        spgemm_set_mode(h, SPGEMM_MODE_PLAIN);
+        if (live + 4000 * (32 + 128) * 12 > before) {
+            std::printf("%s: temporary rows kept in plain mode\n", where);
+            faults = true;
+        }
+    }
+    most = before;
+    C = spgemm_csr_out{};
+    const int rc = back_to_plain ? spgemm_multiply(h, &A, &A, &C) : spgemm_symbolic(h, &A, &A, 0, kRows / 2, &nnz);
+    most = SIZE_MAX;
+    if (rc != SPGEMM_OK) {
+        std::printf("%s: result %d\n", where, rc);
+        faults = true;
+    }
+    for (void *p : {static_cast<void *>(C.rpt), static_cast<void *>(C.col), static_cast<void *>(C.val)})
+        if (p) spgemm_free(h, p);
+    spgemm_destroy(h);
+    if (live != 0) {
+        std::printf("%s: %zu bytes not given back\n", where, live);
+        faults = true;
+    }
 }
 
 int main() {
@@ -261,5 +314,6 @@ int main() {
             faults = true;
         }
     }
+    for (bool back_to_plain : {true, false}) kept_memory(back_to_plain);
     return faults ? 1 : 0;
 }
