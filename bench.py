@@ -62,7 +62,7 @@ WORKLOADS = {
 
 SLOT_NAMES = ([f"sym_bin{j}" for j in range(16)] + [f"num_bin{j}" for j in range(16)]
               + ["nprod", "sym_pass1", "sym_pass2", "num_pass1", "num_pass2", "scan",
-                 "features", "mlp_sizes", "copy_rows"])
+                 "features", "mlp_sizes", "copy_rows", "patterns", "repeat_rows"])
 NSLOTS = len(SLOT_NAMES)
 
 
@@ -450,14 +450,45 @@ def hash_ablation_eval(reps=3):
             "num_speedup_single_over_multi": round(res[1]["num_hash_ms"] / max(res[0]["num_hash_ms"], 1e-9), 3)}
 
 
+REPEAT_SLOT = SLOT_NAMES.index("repeat_rows")
+KERNEL_SLOTS = list(range(32)) + [REPEAT_SLOT]   # kernels that go over the products
+
+
 def _kernel_bytes(bins_sym, bins_num, k, b_bytes):
-    """Algorithmic bytes of bin kernel k (slot index) in one multiply: its
-    A rows, the referenced B rows (b_bytes, the whole product's) and its
-    output (C rows for a numeric bin, 16 bytes per row for a symbolic one)."""
+    """Algorithmic bytes of kernel slot k in one multiply, from the bin
+    statistics: its A rows, the referenced B rows (b_bytes, the whole
+    product's) and its output (C rows for a numeric kernel, 16 bytes per row
+    for a symbolic one); with their description. The repeating rows' kernels
+    are charged for all rows when most repeat. (None, why) where the bin's
+    kernel takes only some of its rows: which B rows those reference is not
+    counted."""
+    if k == REPEAT_SLOT:
+        rows, size, nnza, own = (sum(bins_num[16 * q:16 * q + 16]) for q in range(4))
+        if 2 * own > rows:
+            return None, "fewer than half of the rows repeat the row before"
+        return (24 * rows + 12 * (nnza + size) + b_bytes,
+                f"repeating rows: all but {own} of {rows} rows, {nnza} A entries, n_nz {size}; bytes = the whole "
+                "product's A rows (12/entry + 8/row) + B rows + C rows (12/entry + 16/row)")
     phase, j = divmod(k, 16)
-    bs = list(bins_num if phase else bins_sym)
-    rows_j, size_j, nnza_j = bs[j], bs[16 + j], bs[32 + j]
-    return 8 * rows_j + 12 * nnza_j + b_bytes + ((16 * rows_j + 12 * size_j) if phase else 16 * rows_j)
+    bins = bins_num if phase else bins_sym
+    rows, size, nnza, own = bins[j], bins[16 + j], bins[32 + j], bins[48 + j]
+    if own != rows:
+        return None, f"{own} of the bin's {rows} rows: the others repeat the row before"
+    return (8 * rows + 12 * nnza + b_bytes + ((16 * rows + 12 * size) if phase else 16 * rows),
+            f"{'numeric' if phase else 'symbolic'} bin {j}: {rows} rows, {nnza} A entries, "
+            f"{'n_nz' if phase else 'n_prod'} {size}; bytes = A rows (12/entry + 8/row) + referenced B rows + "
+            f"{'C rows (12/entry + 16/row)' if phase else 'n_nz out (16/row)'}")
+
+
+def _bin_stats(lib, h):
+    """Bin statistics of the last call, (symbolic, numeric)."""
+    import ctypes
+    out = []
+    for phase in (0, 1):
+        a = (ctypes.c_int64 * 64)()
+        lib.spgemm_bin_stats(h._h, phase, a, 64)
+        out.append(list(a))
+    return out
 
 
 def nprod_rows(A):
@@ -531,28 +562,28 @@ def config_line(name, A, slabs, cfg=None, learned_theta=None, margin=0.0, warm=1
         st = h.stats()
         nprod += st["total_nprod"]
         nnz += st["total_nnz"]
-        bins_sym = (ctypes.c_int64 * 48)()
-        bins_num = (ctypes.c_int64 * 48)()
-        lib.spgemm_bin_stats(h._h, 0, bins_sym, 48)
-        lib.spgemm_bin_stats(h._h, 1, bins_num, 48)
+        bins_sym, bins_num = _bin_stats(lib, h)
         tb, b_bytes = compulsory_bytes(A, r0, r1, st["total_nnz"])
         total_bytes += tb
-        for k in range(32):
-            kbytes[k] = kbytes.get(k, 0) + _kernel_bytes(bins_sym, bins_num, k, b_bytes)
+        for k in KERNEL_SLOTS:
+            kb = _kernel_bytes(bins_sym, bins_num, k, b_bytes)[0]
+            kbytes[k] = None if kb is None or kbytes.get(k, 0) is None else kbytes.get(k, 0) + kb
     lib.spgemm_set_timing(h._h, 0)
     lstats = h.learned_stats() if learned_theta is not None else None
     h.close()
     del dA
     torch.cuda.empty_cache()
-    k = int(np.argmax(slot_ms[:32]))
-    kb = kbytes[k]
-    kgbs = kb / (slot_ms[k] / 1e3) / 1e9
+    k = max(KERNEL_SLOTS, key=lambda i: slot_ms[i])
+    # (learned sizing bins its rows by prediction: no bytes per bin)
+    kb = kbytes[k] if learned_theta is None else None
+    kgbs = kb / (slot_ms[k] / 1e3) / 1e9 if kb else None
     wgbs = total_bytes / (ms / 1e3) / 1e9
     out = {"config": name, "slabs": len(slabs), "ms": round(ms, 3), "nprod": int(nprod), "nnzC": int(nnz),
            "gflops": round(2.0 * nprod / (ms / 1e3) / 1e9, 3),
            "dominant_kernel": SLOT_NAMES[k], "dominant_kernel_ms_serial": round(float(slot_ms[k]), 3),
-           "dominant_kernel_share_serial": round(float(slot_ms[k] / max(slot_ms[:38].sum(), 1e-9)), 4),
-           "dominant_kernel_gbs": round(kgbs, 2), "dominant_kernel_frac": round(kgbs / peak, 4),
+           "dominant_kernel_share_serial": round(float(slot_ms[k] / max(slot_ms.sum(), 1e-9)), 4),
+           "dominant_kernel_gbs": round(kgbs, 2) if kb else None,
+           "dominant_kernel_frac": round(kgbs / peak, 4) if kb else None,
            "whole_step_gbs": round(wgbs, 2), "whole_step_frac": round(wgbs / peak, 4),
            "peak_gbs": peak, "peak_kind": f"{peak_kind} copy bandwidth",
            "kernel_ms_serial": {SLOT_NAMES[i]: round(float(slot_ms[i]), 3)
@@ -796,26 +827,15 @@ def main():
     # dominant kernel (longest in the serialised pass) and its roofline,
     # from its live launches in the timed region
     k = int(np.argmax(sms_))
-    bins_sym = (ctypes.c_int64 * 48)()
-    bins_num = (ctypes.c_int64 * 48)()
-    lib.spgemm_bin_stats(h._h, 0, bins_sym, 48)
-    lib.spgemm_bin_stats(h._h, 1, bins_num, 48)
+    bins_sym, bins_num = _bin_stats(lib, h)
     rpt64 = A.rpt.astype(np.int64)
     total_bytes, b_bytes = compulsory_bytes(A, r0, r1, nnzC_slab)
-    if k < 32:
-        phase, j = divmod(k, 16)
-        bs = list(bins_num if phase else bins_sym)
-        rows_j, size_j, nnza_j = bs[j], bs[16 + j], bs[32 + j]
-        a_b = 8 * rows_j + 12 * nnza_j
-        out_b = (16 * rows_j + 12 * size_j) if phase else 16 * rows_j
-        algo = a_b + b_bytes + out_b
-        algo_desc = (f"{'numeric' if phase else 'symbolic'} bin {j}: {rows_j} rows, "
-                     f"{nnza_j} A entries, {'n_nz' if phase else 'n_prod'} {size_j}; bytes = A rows "
-                     f"(12/entry + 8/row) + referenced B rows + "
-                     f"{'C rows (12/entry + 16/row)' if phase else 'n_nz out (16/row)'}")
-    else:
+    algo = None
+    if k in KERNEL_SLOTS:
+        algo, algo_desc = _kernel_bytes(bins_sym, bins_num, k, b_bytes)
+    if algo is None:
         algo = total_bytes
-        algo_desc = "whole product (A + referenced B + C)"
+        algo_desc = "whole product (A + referenced B + C)" + (f"; {algo_desc}" if k in KERNEL_SLOTS else "")
     launches = max(kln[k], 1)
     avg_ms = kms[k] / launches
     peak, peak_kind = peaks()
@@ -882,10 +902,11 @@ def main():
              "achieved_gbs": round(total_bytes / (ms / args.steps / 1e3) / 1e9, 2),
              "frac": round(total_bytes / (ms / args.steps / 1e3) / 1e9 / peak, 4)}
     breakdown = {SLOT_NAMES[i]: round(kms[i] / args.steps, 3) for i in range(len(kms)) if kms[i] > 0}
-    gpu_launches = int(sum(kln) + kln[37])   # the scan slot covers two kernels
+    # the scan slot covers two kernels; the patterns slot two, and a third in the n_prod slot
+    gpu_launches = int(sum(kln) + kln[37] + 2 * kln[SLOT_NAMES.index("patterns")])
 
-    bins = {"sym_rows": list(bins_sym)[:16], "sym_nprod": list(bins_sym)[16:32],
-            "num_rows": list(bins_num)[:16], "num_nnz": list(bins_num)[16:32]}
+    bins = {"sym_rows": bins_sym[:16], "sym_nprod": bins_sym[16:32], "sym_rows_taken": bins_sym[48:],
+            "num_rows": bins_num[:16], "num_nnz": bins_num[16:32], "num_rows_taken": bins_num[48:]}
     cfg_used = h.get_config()
 
     tuned = None

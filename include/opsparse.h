@@ -256,8 +256,10 @@ int spgemm_multiply_host(spgemm_handle *h, const spgemm_csr_in *A,
                          spgemm_host_sink_fn sink, void *ctx, int64_t *nnzC);
 
 /* Per-bin statistics of the last symbolic call for phase 0 (symbolic bins)
- * or 1 (numeric bins): 3 * SPGEMM_MAX_BINS int64: rows per bin, sum of the
- * row sizes per bin (n_prod or n_nz), A entries of the bin's rows. */
+ * or 1 (numeric bins): 4 * SPGEMM_MAX_BINS int64: rows per bin, sum of the
+ * row sizes per bin (n_prod or n_nz), A entries of the bin's rows, and rows
+ * that the bin's own kernel takes (the others repeat the pattern of the row
+ * before: they need no symbolic work and have numeric kernels of their own). */
 int spgemm_bin_stats(const spgemm_handle *h, int phase, int64_t *out, int n);
 
 /* Column windows of the last symbolic/numeric pair (see bitmap_path), up to

@@ -98,7 +98,7 @@ struct spgemm_handle {
     bool reuse = false;
     int64_t reuse_arows = 0, reuse_annz = 0, reuse_brows = 0, reuse_bnnz = 0;
     int64_t stats[4 + 2 * SPGEMM_MAX_BINS] = {};
-    int64_t bin_stats[2][3 * SPGEMM_MAX_BINS] = {};
+    int64_t bin_stats[2][4 * SPGEMM_MAX_BINS] = {};
     // learned sizing
     int mode = 0;                 // SPGEMM_MODE_PLAIN / SPGEMM_MODE_LEARNED
     float *theta = nullptr;       // predictor parameters (device)
@@ -829,6 +829,7 @@ int read_counters(spgemm_handle *h) {
             h->bin_stats[phase][j] = static_cast<int64_t>(h->h_cnt[phase].bin_cnt[j]);
             h->bin_stats[phase][SPGEMM_MAX_BINS + j] = static_cast<int64_t>(h->h_cnt[phase].bin_sum[j]);
             h->bin_stats[phase][2 * SPGEMM_MAX_BINS + j] = static_cast<int64_t>(h->h_cnt[phase].bin_nnza[j]);
+            h->bin_stats[phase][3 * SPGEMM_MAX_BINS + j] = static_cast<int64_t>(h->h_cnt[phase].bin_own[j]);
         }
     return err ? SPGEMM_ERR_INTERNAL : SPGEMM_OK;
 }
@@ -1461,6 +1462,7 @@ int spgemm_symbolic(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_i
     }
     for (int j = 0; j < kMaxBins; ++j)
         h->num_size[j] = j < rn.nb ? (h->rep_num ? h->h_cnt[1].bin_own[j] : h->h_cnt[1].bin_cnt[j]) : 0;
+    for (int j = 0; j < SPGEMM_MAX_BINS; ++j) h->bin_stats[1][3 * SPGEMM_MAX_BINS + j] = h->num_size[j];
     h->crpt = crpt;
     h->row0 = row_begin;
     h->ncols = B->cols;
@@ -1987,7 +1989,7 @@ int spgemm_multiply_host(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_
 
 int spgemm_bin_stats(const spgemm_handle *h, int phase, int64_t *out, int n) {
     if (!h || !out || phase < 0 || phase > 1 || n < 0) return SPGEMM_ERR_INVALID;
-    const int m = std::min<int>(n, 3 * SPGEMM_MAX_BINS);
+    const int m = std::min<int>(n, 4 * SPGEMM_MAX_BINS);
     std::memcpy(out, h->bin_stats[phase], sizeof(int64_t) * (size_t)m);
     return SPGEMM_OK;
 }

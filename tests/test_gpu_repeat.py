@@ -235,3 +235,34 @@ def test_learned_sizing_with_some_rows_mispredicted(name, every):
             same(C, want)
             if weights is theta:
                 assert 0 < st["mispredicted_rows"] < A.rows // 2
+
+
+@pytest.mark.parametrize("kind", ["band", "unsorted rows of B", "window below the rule"])
+def test_bin_statistics_tell_the_rows_that_the_kernels_take(kind):
+    import ctypes
+    from paper_2206_07244_gb300 import _abi
+    A = offsets(N, range(-8, 9), 1)
+    B = A
+    rows = N
+    if kind == "unsorted rows of B":
+        B = W.Csr(A.rows, A.cols, A.rpt, A.col.copy(), A.val)
+        B.col[5:7] = B.col[5:7][::-1].copy()
+    elif kind == "window below the rule":
+        rows = 4000
+    with ops.Handle() as h:
+        nnz = h.symbolic(dev(A), dev(B), 0, rows)
+        st = []
+        for phase in (0, 1):
+            a = (ctypes.c_int64 * 64)()
+            _abi.check(_abi.lib().spgemm_bin_stats(h._h, phase, a, 64), "spgemm_bin_stats")
+            st.append(np.array(a).reshape(4, 16))
+    for phase in (0, 1):
+        assert st[phase][0].sum() == rows and st[phase][2].sum() == A.rpt[rows]
+        taken = st[phase][3]
+        if kind == "band":
+            assert 0 < taken.sum() < rows // 8
+        elif kind == "window below the rule" or phase == 1:   # numeric kernels need ascending rows of B
+            assert np.array_equal(taken, st[phase][0])
+        else:
+            assert taken.sum() < rows // 8
+    assert st[1][1].sum() == nnz
