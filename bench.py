@@ -399,19 +399,40 @@ def batched_eval(count=512, seed=0, reps=3, tune=True):
     return out
 
 
+def relabelled(A, seed):
+    """A's rows and columns in one random order and the entries of every row
+    shuffled, on the GPU: no row repeats the row before it, and no row's
+    columns ascend, so every product goes through a hash probe."""
+    import torch
+
+    import paper_2206_07244_gb300 as ops
+    dA = ops.CSR.from_workload(A)
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    p = torch.randperm(dA.rows, generator=g, device="cuda")
+    lens = (dA.rpt[1:] - dA.rpt[:-1]).long()
+    row = p[torch.repeat_interleave(torch.arange(dA.rows, device="cuda"), lens)]
+    key = torch.argsort(row * (1 << 31) + torch.randint(0, 1 << 31, row.shape, generator=g, device="cuda"))
+    rpt = torch.zeros(dA.rows + 1, dtype=torch.int64, device="cuda")
+    rpt[1:] = torch.cumsum(torch.bincount(row, minlength=dA.rows), 0)
+    return ops.CSR(dA.rows, dA.cols, rpt.to(torch.int32), p[dA.col.long()[key]].to(torch.int32), dA.val[key])
+
+
 def hash_ablation_eval(reps=3):
     """The paper's hashing comparison (Sec. 6): one atomicCAS per probe
     (Algorithms 4-5, hash_access = 0) against a read of the slot before the
-    compare-and-swap (hash_access = 1), everything else the same, on the
-    27-point stencil 128^3, whose rows all take hash kernels. Kernel times of
-    the symbolic and numeric hash bins, serialised on one stream."""
+    compare-and-swap (hash_access = 1), on the 27-point stencil 128^3 with its
+    points relabelled at random and every row shuffled: repeating rows, sums by
+    column, column bitmaps and value updates without atomics, which only one
+    side has, take no row of it. Kernel times of the symbolic and numeric hash
+    bins, serialised on one stream. (The symbolic warp-row kernel of the
+    single-access side keeps 1,536 threads on an SM, the other's 2,048.)"""
     import ctypes
     import torch
     import paper_2206_07244_gb300 as ops
     from paper_2206_07244_gb300 import _abi
     lib = _abi.lib()
     S = W.stencil27(128, seed=3)
-    dS = ops.CSR.from_workload(S)
+    dS = relabelled(S, 5)
     del S
     res = {}
     for mode in (0, 1):
@@ -441,10 +462,18 @@ def hash_ablation_eval(reps=3):
         nbs, nbn = len(ops.kernel_table(0)) - 1, len(ops.kernel_table(1)) - 1
         sym = sum(ms[j] for j, k in enumerate(cfg["sym_kernel"]) if k != nbs) / reps
         num = sum(ms[16 + j] for j, k in enumerate(cfg["num_kernel"]) if k != nbn) / reps
+        for phase, st in enumerate(_bin_stats(lib, h)):
+            # every row in a bin of its own kernel, none in a form that only
+            # single access has (rows of at most 8 products; the 512- and
+            # 1024-slot kernels)
+            bins = cfg["num_kernel" if phase else "sym_kernel"]
+            assert st[48:] == st[:16] and ln[REPEAT_SLOT] == 0, "repeating rows in the hashing comparison"
+            assert sum(n for n, k in zip(st[:16], bins) if ops.kernel_table(phase)[k][2] > 256) == 0 or phase == 0
         res[mode] = {"sym_hash_ms": round(sym, 3), "num_hash_ms": round(num, 3),
                      "multiply_ms_serial": round(e0.elapsed_time(e1) / reps, 3)}
         h.close()
-    return {"workload": "C = A*A, A = 27-point stencil 128^3 (every row in a hash bin)",
+    return {"workload": "C = A*A, A = 27-point stencil 128^3, points relabelled at random, rows shuffled "
+                        "(every row in a hash bin, every product a probe)",
             "single_access": res[0], "multi_access": res[1],
             "sym_speedup_single_over_multi": round(res[1]["sym_hash_ms"] / max(res[0]["sym_hash_ms"], 1e-9), 3),
             "num_speedup_single_over_multi": round(res[1]["num_hash_ms"] / max(res[0]["num_hash_ms"], 1e-9), 3)}
