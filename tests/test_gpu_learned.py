@@ -336,3 +336,42 @@ def test_load_feedback_settles_on_stencil():
     assert last["factor_log2"] == stats[-2]["factor_log2"]
     assert last["rows_over_3_4_full"] + last["mispredicted_rows"] <= 0.25 * (
         last["one_phase_rows"] + last["mispredicted_rows"])
+
+
+@pytest.mark.parametrize("rows", [32768, 38912, 38913, 65536, 622593])   # 64, 64, 96, 128 and 1,024 rows a block
+def test_prediction_of_rows_of_which_none_repeat(rows):
+    # the prediction kernel for products that look for repeating rows: every
+    # row is sized (C is right), and a small product is spread over the GPU
+    # (32 rows take a block about 3 us: 65,536 rows on 64 blocks took 148 us,
+    # a thread each 82 us)
+    import ctypes
+    from paper_2206_07244_gb300 import _abi
+    rng = np.random.default_rng(rows)
+    K = 5000
+
+    def even(n, k, cols):
+        col = (rng.integers(0, cols, (n, 1)) + np.cumsum(rng.integers(1, cols // k, (n, k)), axis=1)) % cols
+        return W.Csr(n, cols, np.arange(0, n * k + 1, k, dtype=np.int32), np.sort(col, axis=1).astype(np.int32).ravel(),
+                     rng.integers(-3, 4, n * k).astype(np.float64))
+
+    A, B = even(rows, 3, K), even(K, 4, 3000)
+    want = oracle.spgemm(A, B)[:3]
+    dA, dB = dev(A), dev(B)
+    with ops.Handle() as h:
+        h.set_predictor(np.load(learned.WEIGHTS), 0.25)
+        h.set_mode("learned")
+        ms, ln = (ctypes.c_double * 43)(), (ctypes.c_int64 * 43)()
+        best = np.inf
+        lib = _abi.lib()
+        _abi.check(lib.spgemm_set_timing(h._h, 1), "spgemm_set_timing")
+        for _ in range(6):
+            C = h.multiply(dA, dB)
+            h.status()
+            _abi.check(lib.spgemm_kernel_times(h._h, ms, ln, 43, 1), "spgemm_kernel_times")
+            best = min(best, 1e3 * ms[39])
+        for g, w in zip(C.numpy(), want):
+            assert np.array_equal(g, w)
+        st = h.learned_stats()
+        assert st["one_phase_rows"] + st["mispredicted_rows"] + st["exact_rows"] == rows
+    if rows <= 65536:
+        assert best < 110.0, best
