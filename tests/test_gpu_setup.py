@@ -207,3 +207,75 @@ def test_empty_rows_are_not_walked_by_one_block(side):
         for g, w in zip(C.numpy(), oracle.spgemm(A, B)[:3]):
             assert np.allclose(g, w, rtol=1e-12, atol=1e-12)
     assert best < (6.0 if side == "A" else 3.0), best
+
+
+# Rows whose part of a tile is more than 32 steps of their threads (one thread
+# a row up to 4 entries on average, then as many as a quarter of the average):
+# at that limit, over tiles, in one warp and in rows next to each other.
+HUBS = {
+    "one thread a row": [1, 2, 32, 33, 34, 0, 31, 65] + [1] * 3000 + [900, 33, 1],
+    "hub over tiles": [2] * 700 + [5 * TILE + 77] + [2] * 3000,
+    "hubs side by side": [1] * 4000 + [TILE, TILE + 1, 40, 2 * TILE, 3] + [1] * 4000,
+    "two threads a row": [7] * 400 + [64, 65, 66, 400] + [5] * 300 + [130, 63],
+    "eight threads a row": [25] * 200 + [256, 257, 300, 1] + [30] * 100 + [2000],
+    "sixteen threads a row": [60] * 100 + [512, 513, 1800] + [62] * 50,
+    "a warp a row": [130] * 60 + [1024, 1025, 1500] + [140] * 30,
+}
+
+
+@pytest.mark.parametrize("i64", [False, True])
+@pytest.mark.parametrize("name", HUBS)
+def test_long_rows_among_short_ones(name, i64):
+    K = 15000
+    A = rows_of(HUBS[name], K, 1)
+    B = rows_of(np.random.default_rng(2).integers(0, 4, K), 900, 3)
+    want = oracle.nprod(A, B)
+    t = np.int64 if i64 else np.int32
+    dA, dB = (ops.CSR.from_arrays(m.rows, m.cols, m.rpt.astype(t), m.col, m.val) for m in (A, B))
+    with ops.Handle() as h:
+        got = h.multiply(dA, dB)
+        st = h.stats()
+        h.status()
+    assert st["total_nprod"] == want.sum() and st["max_nprod"] == want.max()
+    for g, w in zip(got.numpy(), oracle.spgemm(A, B)[:3]):
+        assert np.array_equal(g, w)
+    X = learned.features(dA, dB).cpu().numpy()
+    length = np.diff(B.rpt)
+    full = np.flatnonzero(np.diff(A.rpt))
+    np.testing.assert_allclose(X[:, 1], np.log1p(want.astype(np.float64)), rtol=4e-7, atol=0)
+    for k, f in ((2, np.maximum), (4, np.minimum)):
+        w = f.reduceat(length[A.col], A.rpt[full])
+        np.testing.assert_allclose(X[full, k], np.log1p(w.astype(np.float64)), rtol=4e-7, atol=0)
+
+
+def test_full_last_row_of_a_tridiagonal_matrix():
+    # the row repeats no other and is counted where most rows are left out;
+    # 64 tiles are in flight at once, and the 64 loads that a lane takes there
+    # wait for memory about 1 us each at most
+    import ctypes
+    from paper_2206_07244_gb300 import _abi
+    n = 1 << 17
+    lists = [np.arange(max(i - 1, 0), min(i + 2, n)) for i in range(n - 1)] + [np.arange(n)]
+    rpt = np.zeros(n + 1, dtype=np.int32)
+    np.cumsum([x.size for x in lists], out=rpt[1:])
+    rng = np.random.default_rng(4)
+    A = W.Csr(n, n, rpt, np.concatenate(lists).astype(np.int32), rng.integers(-3, 4, rpt[-1]).astype(np.float64))
+    B = W.Csr(n, n, A.rpt.copy(), A.col, A.val)
+    B.rpt[-1] = B.rpt[-2] + 2   # tridiagonal
+    last = B.rpt[-2]
+    B.col, B.val = np.concatenate([A.col[:last], [n - 2, n - 1]]).astype(np.int32), A.val[:last + 2].copy()
+    dA, dB = ops.CSR.from_workload(A), ops.CSR.from_workload(B)
+    ms, ln = (ctypes.c_double * 43)(), (ctypes.c_int64 * 43)()
+    best = np.inf
+    with ops.Handle() as h:
+        _abi.check(_abi.lib().spgemm_set_timing(h._h, 1), "spgemm_set_timing")
+        for _ in range(6):
+            C = h.multiply(dA, dB)
+            h.status()
+            st = h.stats()
+            _abi.check(_abi.lib().spgemm_kernel_times(h._h, ms, ln, 43, 1), "spgemm_kernel_times")
+            best = min(best, 1e3 * ms[32])
+        for g, w in zip(C.numpy(), oracle.spgemm(A, B)[:3]):
+            assert np.array_equal(g, w)
+    assert st["total_nprod"] == oracle.nprod(A, B).sum()
+    assert best < 100.0, best
