@@ -310,7 +310,9 @@ int spgemm_last_stats(const spgemm_handle *h, int64_t *out, int n);
 /* Describe kernel `id` of a phase (0 symbolic, 1 numeric): its threads per
  * row, threads per block, table capacity (entries; for the bitmap kernel
  * the number of columns one pass covers) and the largest row size it
- * accepts. Returns SPGEMM_ERR_INVALID past the last kernel. */
+ * accepts. The numeric kernels of 64 and 128 threads per row also have a form
+ * of one warp per row, chosen per row by its products. Returns
+ * SPGEMM_ERR_INVALID past the last kernel. */
 int spgemm_kernel_info(int phase, int id, int32_t *threads_per_row,
                        int32_t *block, int64_t *table, int64_t *max_size);
 

@@ -4,21 +4,29 @@
 //
 // Bins 0..8: a row group of TPR threads owns a shared-memory table of T
 // (int32 key, float64 value) slots, 12 bytes each, keys -1 = empty. Each
-// product probes with one atomicCAS; on an empty slot or the same key the
-// value is added with a shared-memory float64 atomicAdd (Algorithm 5). Then
-// the three phases of Sec. 5.6.2 follow: condense the occupied slots to the
-// front of the table (ballot/popc prefix per chunk of TPR slots, in place),
-// sort them by column (bitonic network in shared memory over the next power
-// of two), and store them with coalesced writes. The row size is known from
-// the symbolic phase and checked.
+// product probes with one atomicCAS; on an empty slot or the same key its
+// fused multiply-add is a 64-bit compare-and-swap loop (Algorithm 5), or a
+// plain update where a warp or less takes one B row per step and B's rows are
+// strictly ascending. Then the three phases of Sec. 5.6.2 follow: condense the
+// occupied slots to the front of the table (ballot/popc prefix per chunk of TPR
+// slots, in place), sort them by column (in a warp's registers, by a span bitmap,
+// or a bitonic network in shared memory) and store them coalesced. The row size
+// is known from the symbolic phase and checked. Three kinds of rows go another
+// way:
+//  - rows of at most 8 products stay in the registers of 8 lanes (tiny_load);
+//  - a warp adds a row that spans few columns by column in the table's memory,
+//    without probes and sort (span_walk; kSpanShort says when);
+//  - the 512- and 1024-slot tables have a warp-per-row form, and num_row_limits
+//    decides which rows take it and which the block-per-row form.
+// Rows that repeat the pattern of the row before are not in the bins (repeat.cu).
 //
 // Rows past the largest table go to num_bitmap_kernel (one 1024-thread block
 // per row). Pass 1 marks the row's columns in a shared-memory bitmap (set
-// with 32-bit atomicOr, read as 64-bit words) and forms per-word prefix counts, which give every column its rank
-// in the sorted row: C.col is written straight from the bitmap in column
-// order, no sort needed. Pass 2 adds each product into C.val[rank] with a
-// float64 atomicAdd in global memory (L2). 227 KB cover 1.2M columns per
-// pass; wider matrices take several column windows. This replaces the
+// with 32-bit atomicOr, read as 64-bit words) and forms per-word prefix counts,
+// which give every column its rank in the sorted row: C.col is written straight
+// from the bitmap in column order, no sort needed. Pass 2 adds each product into
+// C.val[rank] with a float64 atomicAdd in global memory (L2). 227 KB cover 1.2M
+// columns per pass; wider matrices take several column windows. This replaces the
 // paper's global-memory hash kernel (its kernel 7) and its condense/sort.
 #include <algorithm>
 #include <climits>
@@ -1042,7 +1050,7 @@ static NumFn g_num_multi[] = {NUM_TABLE(NUM_MULTI_ENTRY)};
 // 132 us; about 290 entries, 7,482 rows: 239 -> 94 us; block-diagonal n = 2^20
 // with 437 entries a row: 11.9 -> 9.5 ms.) Wider B takes the block kernels,
 // which sort by a span bitmap or in shared memory, 64 and 128 threads wide;
-// so does the read-then-swap probe.
+// so do the read-then-swap probe and rows of many products (num_row_limits).
 constexpr int64_t kWarpRowCols = int64_t{1} << 23;
 // [0] every row, [1] with a queue; fn and one-phase.
 #define NUM_WARP(TPR, BLOCK, T)                                                                  \
