@@ -89,10 +89,10 @@ __device__ __forceinline__ int lanes_per_row(int64_t entries, int64_t rows) {
 // Block `blk` of `nblk`: lengths of the B rows that A's entries in the
 // window reference, reduced per row: the sum into nprod and, with FEAT, the
 // largest and smallest into maxlen / minlen (all set to their neutral value
-// before). With `words` the repeating rows are left out, and the entries of
-// the others are not staged (most of the tile is not read). A row inside one tile is stored by one thread, a row cut by a
-// tile's edge is combined with atomics.
-template <bool FEAT>
+// before). WORDS: the repeating rows are left out, and the entries of the others
+// are not staged (most of the tile is not read). A row inside one tile is stored
+// by one thread, a row cut by a tile's edge is combined with atomics.
+template <bool FEAT, bool WORDS>
 __device__ __forceinline__ void row_lengths(const Operands &op, int64_t *nprod, unsigned *maxlen, unsigned *minlen,
                                             const RepWord *words, int blk, int nblk, int *s_len) {
     const int64_t lo = op.row0, hi = op.row0 + op.mw;
@@ -111,7 +111,7 @@ __device__ __forceinline__ void row_lengths(const Operands &op, int64_t *nprod, 
 #pragma unroll
         for (int j = 0; j < kTileItems; ++j) {
             const int64_t p = t0 + j * kTileBlock + threadIdx.x;
-            k[j] = !words && p < t1 ? __ldg(op.acol + p) : -1;
+            k[j] = !WORDS && p < t1 ? __ldg(op.acol + p) : -1;
         }
 #pragma unroll
         for (int j = 0; j < kTileItems; ++j)
@@ -129,7 +129,7 @@ __device__ __forceinline__ void row_lengths(const Operands &op, int64_t *nprod, 
                 e = ld_rpt(op.arpt, op.a64, i + 1);
             }
             const int a = static_cast<int>((s > t0 ? s : t0) - t0), b = static_cast<int>((e < t1 ? e : t1) - t0);
-            bool own = s < t1 && !(words && ((words[(i - lo) >> 5].fol >> ((i - lo) & 31)) & 1u));
+            bool own = s < t1 && !(WORDS && ((words[(i - lo) >> 5].fol >> ((i - lo) & 31)) & 1u));
             // A piece of more than 32 steps of its row's threads (hub rows among
             // short ones) is the whole warp's: tridiagonal matrix of 2^17 rows with
             // a full last row 236 us for n_prod, now 33; n = 2^20 522 and 117. (The
@@ -143,7 +143,7 @@ __device__ __forceinline__ void row_lengths(const Operands &op, int64_t *nprod, 
                 unsigned most = 0, least = UINT_MAX;
                 for (int q = a1 + lane; q < b1; q += 32) {
                     int len;
-                    if (words) {
+                    if (WORDS) {
                         const int c = __ldg(op.acol + t0 + q);
                         len = static_cast<int>(ld_rpt(op.brpt, op.b64, c + 1) - ld_rpt(op.brpt, op.b64, c));
                     } else {
@@ -173,7 +173,7 @@ __device__ __forceinline__ void row_lengths(const Operands &op, int64_t *nprod, 
             if (own)
                 for (int q = a + l; q < b; q += L) {
                     int len;
-                    if (words) {
+                    if (WORDS) {
                         const int c = __ldg(op.acol + t0 + q);
                         len = static_cast<int>(ld_rpt(op.brpt, op.b64, c + 1) - ld_rpt(op.brpt, op.b64, c));
                     } else {
@@ -219,7 +219,7 @@ __device__ __forceinline__ void row_lengths(const Operands &op, int64_t *nprod, 
             }
             if (step == kWalkSteps) {
                 row = block_row_of(op.arpt, op.a64, next, hi, t1);
-                sparse_tile_lengths<FEAT>(op, nprod, maxlen, minlen, words, next, static_cast<int>(row - next + 1),
+                sparse_tile_lengths<FEAT>(op, nprod, maxlen, minlen, WORDS ? words : nullptr, next, static_cast<int>(row - next + 1),
                                           ld_rpt(op.arpt, op.a64, next), t0, t1, s_len);
                 break;
             }
@@ -300,10 +300,13 @@ __device__ __forceinline__ void order_check(const Operands &op, int64_t brows, i
         atomicOr(&cnt->flags, (any_bad ? 1ull : 0ull) | (any_dup ? 2ull : 0ull));
 }
 
-// (Five blocks on an SM, 48 registers: at six the searches of sparse tiles spill
-// into the walk, 27-point stencil 128^3 170 us for n_prod instead of 164.)
 // Both scans in one launch: the first `nprod_blocks` blocks count products,
-// the others check B's order (either part may have no blocks).
+// the others check B's order (either part may have no blocks). WORDS: with
+// repeating rows; the two walks are apart because one that decides at run time
+// keeps the registers of both (27-point stencil 128^3 174 us, now 155). Five
+// blocks on an SM, 48 registers: at six the searches of sparse tiles spill into
+// the walk (160 us).
+template <bool WORDS>
 __global__ void __launch_bounds__(kTileBlock, 5)
 setup_kernel(Operands op, int64_t *nprod, const RepWord *words, RepGate gate, bool only_open, int nprod_blocks,
              int64_t brows, int64_t bnnz, Counters *cnt) {
@@ -311,7 +314,8 @@ setup_kernel(Operands op, int64_t *nprod, const RepWord *words, RepGate gate, bo
     if (static_cast<int>(blockIdx.x) < nprod_blocks) {
         const bool shut = gate.shut();
         if (shut && only_open) return;   // uniform over the block
-        row_lengths<false>(op, nprod, nullptr, nullptr, shut ? nullptr : words, blockIdx.x, nprod_blocks, s_len);
+        if (WORDS && !shut) row_lengths<false, WORDS>(op, nprod, nullptr, nullptr, words, blockIdx.x, nprod_blocks, s_len);
+        else row_lengths<false, false>(op, nprod, nullptr, nullptr, nullptr, blockIdx.x, nprod_blocks, s_len);
     } else
         order_check(op, brows, bnnz, cnt, blockIdx.x - nprod_blocks, gridDim.x - nprod_blocks,
                     reinterpret_cast<unsigned char *>(s_len));
@@ -321,7 +325,7 @@ __global__ void __launch_bounds__(kTileBlock, 5)
 feature_scan_kernel(Operands op, int64_t *nprod, unsigned *maxlen, unsigned *minlen, RepGate gate) {
     __shared__ int s_len[kTileEntries];
     if (gate.found && !gate.shut()) return;   // uniform over the grid
-    row_lengths<true>(op, nprod, maxlen, minlen, nullptr, blockIdx.x, gridDim.x, s_len);
+    row_lengths<true, false>(op, nprod, maxlen, minlen, nullptr, blockIdx.x, gridDim.x, s_len);
 }
 
 // Blocks for `entries` entries: at most `grid`, no more than there are tiles.
@@ -336,7 +340,8 @@ cudaError_t launch_setup(const Operands &op, int64_t annz, int64_t *nprod, int64
     const int na = nprod && op.mw > 0 ? tile_grid(annz, grid) : 0;
     const int nb = cnt && bnnz > 1 && brows > 0 ? tile_grid(bnnz, grid) : 0;
     if (na + nb == 0) return cudaSuccess;
-    setup_kernel<<<na + nb, kTileBlock, 0, s>>>(op, nprod, words, gate, only_open, na, brows, bnnz, cnt);
+    const auto kernel = words ? &setup_kernel<true> : &setup_kernel<false>;
+    kernel<<<na + nb, kTileBlock, 0, s>>>(op, nprod, words, gate, only_open, na, brows, bnnz, cnt);
     return cudaGetLastError();
 }
 
@@ -380,6 +385,8 @@ __device__ __forceinline__ unsigned long long group_total(unsigned same, unsigne
 // by the loads of the sizes and row pointers. (Before: two 64-bit shared
 // atomics per row, compare-and-swap loops that all rows of a bin contend
 // for: 57 us for 4,096 rows, 0.265 ms for 2.1M rows in one bin.)
+// REP: with repeating rows (rep.words).
+template <bool REP>
 __global__ void __launch_bounds__(kBinBlock)
 bin_pass1_kernel(const int64_t *sizes, int64_t n, Ranges rg, Operands op, Counters *cnt,
                  long long *tile_sums, RepArgs rep) {
@@ -397,7 +404,7 @@ bin_pass1_kernel(const int64_t *sizes, int64_t n, Ranges rg, Operands op, Counte
         s_bsum[w][lane] = 0;
         s_bnza[w][lane] = 0;
     }
-    if (rep.words) {   // uniform
+    if (REP) {
         if (threadIdx.x < kRepClasses) s_rep[threadIdx.x] = 0;
         __syncthreads();
     }
@@ -415,7 +422,7 @@ bin_pass1_kernel(const int64_t *sizes, int64_t n, Ranges rg, Operands op, Counte
         }
     }
     unsigned out = 0;   // bit it: the row is left out of the bins
-    if (rep.words) {
+    if (REP) {
 #pragma unroll
         for (int it = 0; it < kBinItems; ++it) {
             const int64_t i = tile0 + it * kBinBlock + threadIdx.x;
@@ -438,7 +445,7 @@ bin_pass1_kernel(const int64_t *sizes, int64_t n, Ranges rg, Operands op, Counte
 #pragma unroll
     for (int it = 0; it < kBinItems; ++it) {
         const bool valid = tile0 + it * kBinBlock + threadIdx.x < n;
-        const unsigned left = __ballot_sync(0xffffffffu, (out >> it) & 1u);
+        const unsigned left = REP ? __ballot_sync(0xffffffffu, (out >> it) & 1u) : 0u;
         my_max = my_max > v[it] ? my_max : v[it];
         const int j = valid ? bin_of(static_cast<long long>(v[it]), rg) : -1;
         const unsigned same = __match_any_sync(0xffffffffu, j);
@@ -478,7 +485,7 @@ bin_pass1_kernel(const int64_t *sizes, int64_t n, Ranges rg, Operands op, Counte
             atomicAdd(&cnt->bin_nnza[lane], bn);
             if (own) atomicAdd(&cnt->bin_own[lane], static_cast<unsigned long long>(own));
         }
-        if (rep.words && lane < kRepClasses && s_rep[lane])
+        if (REP && lane < kRepClasses && s_rep[lane])
             atomicAdd(&cnt->rep_cnt[lane], static_cast<unsigned long long>(s_rep[lane]));
         if (lane == 0) {
             atomicMax(&cnt->max_size, mx);
@@ -536,8 +543,8 @@ cudaError_t launch_bin_pass1(const int64_t *sizes, int64_t n, const Ranges &rg,
                              cudaStream_t s, const RepArgs &rep) {
     if (n <= 0) return cudaSuccess;
     const int64_t grid = (n + kBinTile - 1) / kBinTile;
-    bin_pass1_kernel<<<static_cast<unsigned>(grid), kBinBlock, 0, s>>>(sizes, n, rg, op, cnt,
-                                                                       tile_sums, rep);
+    const auto kernel = rep.words ? &bin_pass1_kernel<true> : &bin_pass1_kernel<false>;
+    kernel<<<static_cast<unsigned>(grid), kBinBlock, 0, s>>>(sizes, n, rg, op, cnt, tile_sums, rep);
     return cudaGetLastError();
 }
 
