@@ -126,7 +126,7 @@ struct spgemm_handle {
     int32_t *rowq = nullptr;      // row queues of the numeric kernels
     size_t rowq_bytes = 0;
     double num_na[kMaxBins] = {};          // numeric bins: mean A entries of a row
-    long long max_nprod = 0;               // of a window row
+    long long longest = 0;                 // products of any row of at most kLongMaxNnz entries, at most
     bool rep_num = false;         // the numeric phase leaves them out of its bins
     long long rep_cnt[kRepClasses] = {};   // rows per class
     // column-window numeric path for the last numeric bin (window.cu)
@@ -655,10 +655,13 @@ int run_bins(spgemm_handle *h, int phase, const Operands &op, const spgemm_csr_i
         w.unroll = h->cfg.bitmap_unroll;
         w.multi = h->cfg.hash_access;
         w.distinct = h->b_distinct;
+        w.longest = phase ? nullptr : &d_counters(h, 1)->longest;
         w.by_column = phase && h->b_distinct && span_rows(h->num_na[j], B->nnz, B->rows);
         w.clk = phase == 1 && h->phase_clk ? h->d_clk : nullptr;
         w.err = d_err(h);
-        if (phase) CK(set_row_form(h, j, op, B, h->num_na[j], h->max_nprod, d_counters(h, 1), w, s));
+        if (phase)   // (an explicit configuration may give these kernels longer rows)
+            CK(set_row_form(h, j, op, B, h->num_na[j], h->cfg.num_range[j] > kLongMaxNnz ? LLONG_MAX : h->longest,
+                            d_counters(h, 1), w, s));
         const KernelDesc &d = phase ? num_kernel(kid[j]) : sym_kernel(kid[j]);
         size_t smem = 0;
         const int slot = (phase ? kSlotNumBin : kSlotSymBin) + j;
@@ -1402,7 +1405,6 @@ int spgemm_symbolic(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_i
     if (!repeats) rep = RepArgs{};
     h->stats[0] = static_cast<int64_t>(h->h_cnt[0].total);
     h->stats[1] = static_cast<int64_t>(h->h_cnt[0].max_size);
-    h->max_nprod = static_cast<long long>(h->h_cnt[0].max_size);
     for (int j = 0; j < SPGEMM_MAX_BINS; ++j) h->stats[4 + j] = j < rs.nb ? static_cast<int64_t>(h->h_cnt[0].bin_cnt[j]) : 0;
     if (!sid) {
         time_begin(h, kSlotSymPass2, h->stream);
@@ -1450,6 +1452,7 @@ int spgemm_symbolic(spgemm_handle *h, const spgemm_csr_in *A, const spgemm_csr_i
     h->stats[3] = static_cast<int64_t>(h->h_cnt[1].max_size);
     for (int j = 0; j < SPGEMM_MAX_BINS; ++j)
         h->stats[4 + SPGEMM_MAX_BINS + j] = j < rn.nb ? static_cast<int64_t>(h->h_cnt[1].bin_cnt[j]) : 0;
+    h->longest = std::max<long long>(kLongLeast, static_cast<long long>(h->h_cnt[1].longest));
     for (int j = 0; j < rn.nb; ++j) {
         const Counters &c = h->h_cnt[1];
         h->num_na[j] = c.bin_cnt[j] ? static_cast<double>(c.bin_nnza[j]) / static_cast<double>(c.bin_cnt[j]) : 0.0;

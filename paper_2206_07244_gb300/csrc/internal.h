@@ -58,6 +58,7 @@ struct BinWork {
     unsigned *queued;     // their number (0 before)
     int queue_grid;       // blocks of the block form's launch over the queue, at most
     int block_rows;       // every row by the block form
+    unsigned long long *longest;   // symbolic kernels: Counters::longest (nullptr: not wanted)
     int *err;             // device error word
     // numeric bitmap kernel, pass 2 by column windows (B rows sorted)
     const int32_t *bs;    // run boundaries of B rows at the sub-ranges (G + 1 per row), or nullptr
@@ -193,6 +194,8 @@ struct Counters {
     unsigned long long rep_cnt[kRepClasses];   // numeric pass 1: repeating rows per class
     unsigned long long rep_found;           // rows of A that look like the row before
     unsigned queued[kMaxBins];              // rows in the numeric kernels' queues
+    unsigned long long longest;             // most products of a row of at most kLongMaxNnz entries (0: at
+                                            // most kLongLeast)
     unsigned long long max_size;
     unsigned long long total;
     unsigned long long flags;         // bit 0: some row of B has decreasing columns; bit 1: repeated ones
@@ -228,6 +231,11 @@ constexpr int kSpanShort = 128;
 inline bool span_rows(double na, int64_t bnnz, int64_t brows) {
     return bnnz > 8 * brows || (bnnz > 4 * brows && na <= kSpanShort);
 }
+
+// Rows that a warp-per-row numeric kernel may leave to a block (num_row_limits):
+// of at most kLongMaxNnz entries, and of more than kLongLeast products.
+constexpr int kLongMaxNnz = 512;
+constexpr int kLongLeast = 1024;
 
 // --- setup.cu ----------------------------------------------------------------
 // n_prod of every row of the window, added into nprod (zeroed by the caller;

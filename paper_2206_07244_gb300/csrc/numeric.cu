@@ -1171,8 +1171,9 @@ static int warp_row_form(int id, const Operands &op, const BinWork &w) {
 // The limits lie where the two meet. What most rows are like is told from the
 // mean lengths and B's width, and whole bins past their limit take the block
 // form; a row is looked at, and sent to the block form's queue, only when some
-// row passes that limit: a queue that nothing needed cost 4 us to 8 us, one that
-// held most rows of a bin up to 60% of its time.
+// row passes that limit (Counters::longest, from the symbolic kernels): a queue
+// that nothing needed cost 4 us to 8 us, one that held most rows of a bin up to
+// 60% of its time.
 bool num_row_limits(int id, const Operands &op, double na, double mean_b, long long most, BinWork &w) {
     w.long_col = w.long_near = w.long_far = LLONG_MAX;
     const int k = warp_row_form(id, op, w);

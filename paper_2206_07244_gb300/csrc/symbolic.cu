@@ -55,6 +55,12 @@ __device__ __forceinline__ int sym_insert(int *tab, int key, int *err) {
     return 0;
 }
 
+// A row of np products and n entries for Counters::longest.
+__device__ __forceinline__ void note_longest(const BinWork &w, long long np, long long n) {
+    if (w.longest && np > kLongLeast && n <= kLongMaxNnz)
+        atomicMax(w.longest, static_cast<unsigned long long>(np));
+}
+
 // Minimum resident blocks: enough for 2048 threads per SM (<= 32 registers
 // per thread, Sec. 5.6) unless the table is so large that one block fills
 // the SM's shared memory anyway; warp-per-row kernels 1536 (40 registers: the
@@ -149,7 +155,10 @@ sym_hash_kernel(Operands op, BinWork w) {
         });
     }
     cnt = group_sum<TPR>(cnt, red);
-    if (valid && lg == 0) w.crpt[row] = cnt;
+    if (valid && lg == 0) {
+        if (TPR > 32) note_longest(w, w.crpt[row], cnt);   // a warp's rows have at most kLongLeast products
+        w.crpt[row] = cnt;
+    }
 }
 
 // RUNS: several column passes over sorted B; each pass walks only the runs
@@ -217,7 +226,10 @@ sym_bitmap_kernel(Operands op, BinWork w, int words) {
         __syncthreads();
     }
     total = group_sum<kBmBlock>(total, red);
-    if (threadIdx.x == 0) w.crpt[row] = total;
+    if (threadIdx.x == 0) {
+        note_longest(w, w.crpt[row], total);
+        w.crpt[row] = total;
+    }
 }
 
 // --- kernel table ---------------------------------------------------------------
