@@ -613,6 +613,23 @@ struct SideWork {
     }
 };
 
+// Products of the longest row that numeric bin j may hold (plain calls; an
+// explicit configuration may give a kernel rows that the symbolic phase did
+// not look at).
+long long longest_row(const spgemm_handle *h, int j) {
+    return h->cfg.num_range[j] > kLongMaxNnz ? LLONG_MAX : h->longest;
+}
+
+// Memory for the row queues, before the side streams start: when a bin with
+// rows has a kernel with two forms and a row may be too long for a warp.
+void reserve_queue(spgemm_handle *h, const long long *size, int nb, int64_t mw, bool learned) {
+    for (int j = 0; j < nb; ++j)
+        if (size[j] > 0 && num_has_warp_form(h->cfg.num_kernel[j]) && (learned || longest_row(h, j) > kLongLeast)) {
+            ensure_buf(h, &h->rowq, &h->rowq_bytes, sizeof(int32_t) * (size_t)mw);
+            return;
+        }
+}
+
 // Warp- or block-per-row form of numeric bin j's rows (num_row_limits): na A
 // entries a row on average, at most `most` products. cnt holds the queue's
 // length, which a second numeric call over the same bins clears on the bin's
@@ -621,7 +638,7 @@ cudaError_t set_row_form(spgemm_handle *h, int j, const Operands &op, const spge
                          long long most, Counters *cnt, BinWork &w, cudaStream_t s) {
     const double mean_b = static_cast<double>(B->nnz) / static_cast<double>(std::max<int64_t>(B->rows, 1));
     if (!num_row_limits(h->cfg.num_kernel[j], op, na, mean_b, most, w)) return cudaSuccess;
-    if (ensure_buf(h, &h->rowq, &h->rowq_bytes, sizeof(int32_t) * (size_t)op.mw)) {
+    if (!h->rowq || h->rowq_bytes < sizeof(int32_t) * (size_t)op.mw) {
         w.block_rows = 1;
         return cudaSuccess;
     }
@@ -639,6 +656,7 @@ int run_bins(spgemm_handle *h, int phase, const Operands &op, const spgemm_csr_i
              const RunPlan *runs = nullptr, const WinCall *win = nullptr) {
     const int nb = phase ? h->cfg.num_nbins : h->cfg.sym_nbins;
     const int32_t *kid = phase ? h->cfg.num_kernel : h->cfg.sym_kernel;
+    if (phase) reserve_queue(h, size, nb, op.mw, false);
     CK(cudaEventRecord(h->ev_fork, h->stream));
     SideWork side(h);
     int used = 0;
@@ -659,9 +677,7 @@ int run_bins(spgemm_handle *h, int phase, const Operands &op, const spgemm_csr_i
         w.by_column = phase && h->b_distinct && span_rows(h->num_na[j], B->nnz, B->rows);
         w.clk = phase == 1 && h->phase_clk ? h->d_clk : nullptr;
         w.err = d_err(h);
-        if (phase)   // (an explicit configuration may give these kernels longer rows)
-            CK(set_row_form(h, j, op, B, h->num_na[j], h->cfg.num_range[j] > kLongMaxNnz ? LLONG_MAX : h->longest,
-                            d_counters(h, 1), w, s));
+        if (phase) CK(set_row_form(h, j, op, B, h->num_na[j], longest_row(h, j), d_counters(h, 1), w, s));
         const KernelDesc &d = phase ? num_kernel(kid[j]) : sym_kernel(kid[j]);
         size_t smem = 0;
         const int slot = (phase ? kSlotNumBin : kSlotSymBin) + j;
@@ -956,6 +972,7 @@ int symbolic_learned(spgemm_handle *h, const Operands &op, const spgemm_csr_in *
         h->tcap_have = total_t;
     }
     h->temp_used = true;
+    reserve_queue(h, h->lsize, last, mw, true);
     // one-phase kernels, largest rows first on the side streams
     CK(cudaEventRecord(h->ev_fork, s));
     int used = 0;

@@ -288,6 +288,7 @@ cudaError_t launch_num(int id, const Operands &op, const BinWork &w, size_t smem
 // by_column set before). na: A entries of the bin's rows, mean_b: entries of B's
 // rows, both on average; most: products of any row. True when rows may have to
 // change form, so that the launch needs a queue.
+bool num_has_warp_form(int id);
 bool num_row_limits(int id, const Operands &op, double na, double mean_b, long long most, BinWork &w);
 // one-phase numeric kernel `id` (a hash kernel of the numeric table)
 cudaError_t launch_num_onephase(int id, const Operands &op, const BinWork &w, cudaStream_t s);

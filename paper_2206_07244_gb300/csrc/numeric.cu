@@ -1156,6 +1156,8 @@ static int warp_row_form(int id, const Operands &op, const BinWork &w) {
                    !w.multi && !w.block_rows ? k : -1;
 }
 
+bool num_has_warp_form(int id) { return id >= kNumWarpFirst && id < kNumWarpFirst + kNumWarp; }
+
 // A warp takes a row without block barriers, but a row of many products keeps
 // it long after the others, and the 1024-slot table leaves half as many warps
 // on an SM as the block form has. Numeric phase, block and warp form in us, n

@@ -20,7 +20,8 @@ constexpr int64_t kRows = 40000;
 
 struct Event {
     cudaStream_t s = nullptr;
-    long long at = 0;
+    long long at = 0;     // last work of the stream
+    long long when = 0;   // when it was recorded
 };
 std::map<cudaStream_t, long long> work, waited;   // last work of a stream; of it, what the main stream waits for
 std::map<cudaEvent_t, Event> events;
@@ -49,16 +50,31 @@ cudaError_t launch(cudaStream_t s) {
 long long allocations = 0, fail_allocation = 0;
 size_t live = 0, most = SIZE_MAX;   // bytes handed out, and at most
 std::map<void *, size_t> held;
+std::map<void *, long long> born;                 // when memory was allocated
+std::map<cudaStream_t, long long> started;        // what a side stream waited for, last
+long long queued = 0;                             // launches with a row queue
+// Memory that a side stream's kernel uses is allocated before that stream starts.
+void check_order(const void *p, cudaStream_t s) {
+    queued += p != nullptr;
+    if (!p || s == kMain) return;
+    auto it = born.upper_bound(const_cast<void *>(p));
+    if (it != born.begin() && (--it)->second > started[s]) {
+        std::printf("%s: a side stream's kernel uses memory that was allocated after the stream started\n", where);
+        faults = true;
+    }
+}
 void *take(size_t bytes, void *, void *) {
     if (++allocations == fail_allocation || live + bytes > most) return nullptr;
     void *p = std::calloc(1, bytes);
     live += held[p] = bytes;
+    born[p] = ++now_;
     return p;
 }
 void give(void *p, void *, void *) {
     check("memory is freed");
     live -= held[p];
     held.erase(p);
+    born.erase(p);
     std::free(p);
 }
 
@@ -80,13 +96,14 @@ cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) {
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t s) { if (s != kMain) waited[s] = work[s]; return cudaSuccess; }
 cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned) {
+    if (s != kMain) started[s] = events[e].when;
     if (s == kMain && events[e].s && waited[events[e].s] < events[e].at) waited[events[e].s] = events[e].at;
     return cudaSuccess;
 }
 cudaError_t cudaEventCreate(cudaEvent_t *e) { *e = reinterpret_cast<cudaEvent_t>(static_cast<uintptr_t>(1000 + ++handles)); return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return cudaEventCreate(e); }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) { events[e] = Event{s, work[s]}; return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) { events[e] = Event{s, work[s], ++now_}; return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t) { std::memcpy(d, s, n); return cudaSuccess; }
@@ -114,7 +131,8 @@ cudaError_t win_prepare(int) { return cudaSuccess; }
 cudaError_t rep_prepare() { return cudaSuccess; }
 int64_t bin_tile_rows() { return 4096; }
 size_t num_bitmap_head_bytes(bool) { return 1024; }
-bool num_row_limits(int, const Operands &, double, double, long long, BinWork &) { return true; }
+bool num_has_warp_form(int id) { return id == 1; }
+bool num_row_limits(int id, const Operands &, double, double, long long, BinWork &) { return id == 1; }
 int mlp_param_count() { return 4673; }
 int default_sym_bins(long long *range, int32_t *kernel) {
     const long long r[] = {32, 128, -1};
@@ -136,6 +154,7 @@ cudaError_t launch_bin_pass1(const int64_t *, int64_t n, const Ranges &rg, const
     }
     cnt->rep_cnt[0] = static_cast<unsigned long long>(n - n / 10 * rg.nb);
     cnt->total = 100;
+    cnt->longest = 5000;   // some rows may go to a queue
     (void)tiles;
     return launch(s);
 }
@@ -143,8 +162,12 @@ cudaError_t launch_bin_pass2(const int64_t *, int64_t, const Ranges &, const lon
 cudaError_t launch_scan(int64_t *, int64_t, long long *, cudaStream_t s) { return launch(s); }
 cudaError_t launch_iota(int32_t *, int64_t, cudaStream_t s) { return launch(s); }
 cudaError_t launch_sym(int, const Operands &, const BinWork &, size_t, cudaStream_t s) { return launch(s); }
-cudaError_t launch_num(int, const Operands &, const BinWork &, size_t, cudaStream_t s) { return launch(s); }
+cudaError_t launch_num(int, const Operands &, const BinWork &w, size_t, cudaStream_t s) {
+    check_order(w.queue, s);
+    return launch(s);
+}
 cudaError_t launch_num_onephase(int, const Operands &, const BinWork &w, cudaStream_t s) {
+    check_order(w.queue, s);
     *w.xcount += 5;   // mispredicted rows
     return launch(s);
 }
@@ -285,8 +308,13 @@ static void kept_memory(bool back_to_plain) {
 int main() {
     for (int mode : {SPGEMM_MODE_PLAIN, SPGEMM_MODE_LEARNED}) {
         long long k = 1;
+        queued = 0;
         while (product(mode, k)) ++k;
         std::printf("%s: %lld launches\n", where, k - 1);
+        if (queued == 0) {
+            std::printf("%s: no row queue\n", where);
+            faults = true;
+        }
     }
     // a row window: its rows' mean length, not the whole matrix's entries over them
     for (bool same : {true, false}) {

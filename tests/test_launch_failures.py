@@ -1,7 +1,8 @@
 """A launch that fails inside a call, with kernels of the same call on side
 streams: before the call frees memory or returns, the handle's stream waits
 for them. What the pattern scans of a row window are launched for, and what
-happens without memory for them; and the memory that learned sizing keeps.
+happens without memory for them; the memory that learned sizing keeps; and that
+side streams start after their memory is allocated.
 CPU only: the object of api.cu is linked with a host stand-in for
 the CUDA runtime and the kernels (host/fake_cuda.cpp)."""
 
