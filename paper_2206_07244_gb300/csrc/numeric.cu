@@ -1164,13 +1164,16 @@ bool num_has_warp_form(int id) { return id >= kNumWarpFirst && id < kNumWarpFirs
 // entries a row (n = 200: 512 slots, 400: 1024 slots):
 //   unsorted, n = 200, 6,400 products: 300 rows 87 and 125, 3,000 rows 209 and
 //     149; n = 400, 1,200 products: 300 rows 31 and 43, 20,000 rows 311 and 325;
+//     400 products: 300 rows 26 and 31, 3,000 rows 51 and 52, 9,000 rows 112 and 94;
 //   a hub of 10^6 products among 30,000 short rows: 10,500 and 25,600;
 //   by column, n = 400, B rows of 48: 2,400 products, 300 rows 33 and 42, 20,000
 //     rows 368 and 297; B rows of 24, 2,400 products, 3,000 rows 83 and 63;
 //   columns too far apart for a block's span bitmap, so that it sorts: n = 400,
 //     2,400 products: 300 rows 58 and 71, 3,000 rows 155 and 135, 20,000 rows
 //     925 and 628; 12,800 products, 20,000 rows 1,857 and 1,856.
-// The limits lie where the two meet. What most rows are like is told from the
+// The limits lie where the two meet. Where B is not ascending the span is not
+// known: in large bins of wide B 2,048 products (1,600 products, 20,000 rows: 389
+// and 405 if a row's columns are close, 721 and 321 if far apart). What most rows are like is told from the
 // mean lengths and B's width, and whole bins past their limit take the block
 // form; a row is looked at, and sent to the block form's queue, only when some
 // row passes that limit (Counters::longest, from the symbolic kernels): a queue
@@ -1193,7 +1196,7 @@ bool num_row_limits(int id, const Operands &op, double na, double mean_b, long l
     } else {
         const bool many = w.cnt >= 16384;
         w.long_col = many ? or_mean(2048) : w.cnt >= 2048 ? 3072 : w.cnt >= 512 ? 2048 : 1024;
-        w.long_near = many || !narrow ? 1024 : 0;
+        w.long_near = many && !narrow && !w.by_column ? 2048 : !narrow || w.cnt >= 1024 ? 1024 : 0;
         w.long_far = many ? 8192 : w.cnt >= 2048 ? 3072 : 1536;
     }
     long long least, most_rows;   // limits of the rows that the bin may hold
